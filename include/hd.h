@@ -266,8 +266,8 @@ hd_status hd_timing(hd_ctx *ctx, int enable, double out[16]);
  * program that has already reserved all of the GPU's memory: make the first
  * call at start-up, before reserving memory, or run with
  * CUDA_MODULE_LOADING=EAGER.  Every call synchronises cuda_stream (it reads
- * back an error word and, with an open axis, the positions' extent), so it
- * cannot be called while that stream is being captured.  Every call shares
+ * back an error word), so it cannot be called while that stream is being
+ * captured.  Every call shares
  * the array and leaves its contents behind; counts, extent and the error
  * word are cleared at the start of each call, and calls that overlap on the
  * GPU race.  Returns HD_ERR_OVERFLOW if a row or a cell exceeded its
