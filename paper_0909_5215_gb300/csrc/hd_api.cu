@@ -24,6 +24,7 @@ constexpr size_t ALIGN = 256;
 
 struct Plan {
     int nrep = 0, natom = 0, ntile = 0, maxnb = 0, cell_cap = 0, ncell = 0, block = 128, prec = 0;
+    int nwg = 0, split = 1;
     std::vector<RepDev> rep;
     std::vector<int> tile_rep, tile_start, tile_n;
     // storage order: atoms of a replica are held cell-major (cells of the
@@ -37,7 +38,7 @@ struct Plan {
     size_t o_rep, o_st, o_sc, o_trep, o_tstart, o_tn, o_part, o_qpart, o_kpart;
     size_t o_x, o_xo, o_xq, o_v, o_vq, o_f, o_fq, o_h, o_dr;
     size_t o_pfix, o_pfixb, o_qpfix, o_qpfixb, o_cellid, o_nnb, o_nbr, o_ccnt, o_catoms;
-    size_t o_rebuild, o_qrebuild, o_err, o_bar, o_qdisp, o_qgate, o_drawvel, o_adopt, o_orig, o_rboff, o_rbaoff, o_rblist, o_rbmeta;
+    size_t o_rebuild, o_qrebuild, o_err, o_bar, o_qdisp, o_qgate, o_drawvel, o_adopt, o_orig, o_rboff, o_rbaoff, o_rblist, o_rbmeta, o_hlist, o_hlate, o_hmeta;
     size_t o_ctarep, o_pgfirst, o_pgcount, o_boff, o_bj;
     size_t o_eq, o_ev, o_ew, o_eg, o_ealpha, o_ebeta, o_ey, o_ecoef, o_epart, o_po;
     long long eig_q = 0, eig_t = 0;     // dbl4 entries of all Krylov bases, doubles of all tridiagonals
@@ -207,6 +208,8 @@ bool make_plan(const hd_replica_desc *reps, int n_rep, const hd_params *p, Plan 
         }
         R.ncell = R.nc[0] * R.nc[1] * R.nc[2];
         R.cell0 = (int)ncell;
+        R.wg0 = P.nwg;
+        P.nwg += (d.n_atoms + 31) / 32;
         // occupancy estimate of the initial configuration and the storage order
         {
             std::vector<int> occ(R.ncell, 0), key(d.n_atoms);
@@ -244,6 +247,16 @@ bool make_plan(const hd_replica_desc *reps, int n_rep, const hd_params *p, Plan 
         R.dvmax = d.dvmax;
         R.sig_lo = d.sig_lo;
         R.sig_hi = d.sig_hi;
+        // pair sweep: lengths in the common unit u (px = 1, times 2^zshift on the
+        // open axis; 1/u^2 = pu2) or, without one, in real lengths (px = lsb)
+        const double unit = R.exact_r2 ? 1.0 / R.fx_scale[0] : 1.0, pu2 = 1.0 / (unit * unit);
+        double near2 = 0.0;
+        for (int a = 0; a < 3; ++a) {
+            const double out = R.exact_r2 ? 1.0 / unit : 1.0 + (double)R.lsb_rel[a];
+            R.px_scale[a] = R.exact_r2 ? (float)(1 << (a == 1 ? R.shift_y : a == 2 ? R.shift_z : 0)) : R.fx_lsb[a];
+            R.out_hi[a] = (float)out;
+            R.out_lo[a] = (float)(out - (double)R.out_hi[a]);
+        }
         for (int a = 0; a < 2; ++a)
             for (int b = 0; b < 2; ++b) {
                 const double eps = d.eps[a][b], sig = d.sig[a][b];
@@ -255,18 +268,24 @@ bool make_plan(const hd_replica_desc *reps, int n_rep, const hd_params *p, Plan 
                 R.sig2f[a][b] = (float)(sig * sig);
                 R.shiftf[a][b] = (float)R.shift[a][b];
                 const double r0sq = std::cbrt(2.0) * sig * sig;   // LJ minimum 2^(1/6) sigma, squared
-                R.r0sq_hi[a][b] = (float)r0sq;
-                R.r0sq_lo[a][b] = (float)(r0sq - (double)R.r0sq_hi[a][b]);
-                R.eps24f[a][b] = (float)(24.0 * eps);
-                R.eps96f[a][b] = (float)(96.0 * eps);
-                R.eps24l[a][b] = (float)(24.0 * eps - (double)R.eps24f[a][b]);
-                R.eps96l[a][b] = (float)(96.0 * eps - (double)R.eps96f[a][b]);
-                // the pair sweep takes the exact r^2 where |r_0^2 - r^2| < r^2 / 4,
-                // i.e. r^2 < (4/3) r_0^2; class A of the list holds the pairs within
-                // that radius plus 0.1 sigma at build time
+                R.r0u_hi[a][b] = (float)(r0sq * pu2);
+                R.r0u_lo[a][b] = (float)(r0sq * pu2 - (double)R.r0u_hi[a][b]);
+                R.eps12f[a][b] = (float)(12.0 * eps);
+                R.eps12l[a][b] = (float)(12.0 * eps - (double)R.eps12f[a][b]);
+                near2 = std::max(near2, r0sq * 4.0 / 3.0);
+                // the pair sweep takes the exact r^2 where r^2 < (4/3) r_0^2; class A
+                // of the list holds the pairs within that radius plus 0.1 sigma at
+                // build time
                 const double rA = std::sqrt(r0sq * 4.0 / 3.0) + 0.1 * sig;
                 R.rA2f = std::max(R.rA2f, (float)(rA * rA));
             }
+        // FP32 r^2 of the split sweep is within ~3e-7 (relative) of the oracle's
+        // FP64 r^2 (fixed-point rounding of positions plus FP32 rounding); the
+        // band decided in FP64 is 2^-20 ~ 9.5e-7 wide on each side
+        const double rc2u = p->rc * p->rc * pu2;
+        R.rc2u_lo = (float)(rc2u * (1.0 - 1.0 / 1048576.0));
+        R.rc2u_hi = (float)(rc2u * (1.0 + 1.0 / 1048576.0));
+        R.near2u = R.exact_r2 ? std::min((float)(near2 * pu2), R.rc2u_lo) : 0.f;
         R.kr_n = nrig > 0 ? d.k_spring / nrig : 0.0;
         R.kr_nf = (float)R.kr_n;
         // eigenvalue bias: Lanczos steps at most, capped at the dimension of the
@@ -309,10 +328,8 @@ bool make_plan(const hd_replica_desc *reps, int n_rep, const hd_params *p, Plan 
             R.shift[1][1] = 0.0;
             R.epsf[1][1] = 0.f;
             R.shiftf[1][1] = 0.f;
-            R.eps24f[1][1] = 0.f;
-            R.eps96f[1][1] = 0.f;
-            R.eps24l[1][1] = 0.f;
-            R.eps96l[1][1] = 0.f;
+            R.eps12f[1][1] = 0.f;
+            R.eps12l[1][1] = 0.f;
         }
         P.rep[r] = R;
         for (int k = 0; k < R.ntile; ++k) {
@@ -350,6 +367,12 @@ bool make_plan(const hd_replica_desc *reps, int n_rep, const hd_params *p, Plan 
         for (int i = 0; i < P.natom; ++i) P.bond_j.insert(P.bond_j.end(), part[i].begin(), part[i].end());
     }
     P.cell_cap = p->cell_cap > 0 ? p->cell_cap : ((2 * max_occ + 8 + 7) / 8) * 8;
+    // Lanes that share a row of the pair sweep: with a thread a row, batches of
+    // fewer than ~8 warps an SM leave it waiting for its gathers (8 x 1,983
+    // atoms: 34.5 us a sweep with 1, 20.9 with 4; 8 x 113 atoms, FP64, one
+    // launch: 66.6 and 47.7 us a step); beyond that the split only adds work
+    // (57,088 atoms FP64: 513 us with 1, 570 with 4).
+    P.split = P.natom / 32 < 152 * 8 ? 4 : 1;
     // layout
     const size_t N = P.natom, T = P.ntile, R = P.nrep;
     const size_t v4 = P.prec == HD_FP64 ? sizeof(dbl4) : sizeof(float4);
@@ -360,8 +383,8 @@ bool make_plan(const hd_replica_desc *reps, int n_rep, const hd_params *p, Plan 
     P.o_trep = take(cur, T * 4);
     P.o_tstart = take(cur, T * 4);
     P.o_tn = take(cur, T * 4);
-    P.o_part = take(cur, T * NPART * 8);
-    P.o_qpart = take(cur, T * NPART * 8);
+    P.o_part = take(cur, T * P.split * NPART * 8);
+    P.o_qpart = take(cur, T * P.split * NPART * 8);
     P.o_kpart = take(cur, T * 8);
     P.o_x = take(cur, N * sizeof(dbl4));
     P.o_xo = take(cur, N * sizeof(dbl4));
@@ -372,13 +395,13 @@ bool make_plan(const hd_replica_desc *reps, int n_rep, const hd_params *p, Plan 
     P.o_fq = take(cur, N * v4);
     P.o_h = take(cur, N * v4);
     P.o_dr = take(cur, N * v4);
-    P.o_pfix = take(cur, N * sizeof(AtomRec));
+    P.o_pfix = take(cur, N * sizeof(int4));
     P.o_pfixb = take(cur, N * 16);
-    P.o_qpfix = take(cur, N * sizeof(AtomRec));
+    P.o_qpfix = take(cur, N * sizeof(int4));
     P.o_qpfixb = take(cur, N * 16);
     P.o_cellid = take(cur, N * 4);
     P.o_nnb = take(cur, N * 4);
-    P.o_nbr = take(cur, N * (size_t)P.maxnb * 4);
+    P.o_nbr = take(cur, (size_t)P.nwg * ((P.maxnb + 3) / 4) * 32 * sizeof(int4));
     P.o_ccnt = take(cur, (size_t)P.ncell * 4);
     P.o_catoms = take(cur, (size_t)P.ncell * P.cell_cap * 4);
     P.o_rebuild = take(cur, R * 4);
@@ -394,7 +417,10 @@ bool make_plan(const hd_replica_desc *reps, int n_rep, const hd_params *p, Plan 
     P.o_rbaoff = take(cur, (R + 1) * 4);
     P.o_rblist = take(cur, R * 4);
     P.o_rbmeta = take(cur, 4 * 4);
-    P.o_ctarep = take(cur, T * 4);       // at most one CTA per tile
+    P.o_hlist = take(cur, R * 4);
+    P.o_hlate = take(cur, R * 4);
+    P.o_hmeta = take(cur, 4 * 4);
+    P.o_ctarep = take(cur, T * P.split * 4);       // at most one CTA per part of a tile
     P.o_pgfirst = take(cur, R * 4);
     P.o_pgcount = take(cur, R * 4);
     P.o_po = take(cur, (P.prec == HD_FP64 ? 1 : N) * 16);   // split form: fixed-point image of r_O
@@ -552,6 +578,8 @@ void fill_dev(hd_ctx *c) {
     for (const RepDev &R : P.rep) D.max_cells = std::max(D.max_cells, R.ncell);
     D.prec = P.prec;
     D.block = P.block;
+    D.ngrp = (P.maxnb + 3) / 4;
+    D.split = P.split;
     D.rep = at<RepDev>(b, P.o_rep);
     D.st = at<RepState>(b, P.o_st);
     D.sc = at<Scal>(b, P.o_sc);
@@ -572,7 +600,7 @@ void fill_dev(hd_ctx *c) {
         D.f32 = at<float4>(b, P.o_f);
         D.h32 = at<float4>(b, P.o_h);
     }
-    D.rec = at<AtomRec>(b, P.o_pfix);
+    D.p = at<int4>(b, P.o_pfix);
     D.pfixb = at<int4>(b, P.o_pfixb);
     D.cellid = at<int>(b, P.o_cellid);
     D.nnb = at<int>(b, P.o_nnb);
@@ -589,6 +617,9 @@ void fill_dev(hd_ctx *c) {
     D.rb_aoff = at<int>(b, P.o_rbaoff);
     D.rb_list = at<int>(b, P.o_rblist);
     D.rb_meta = at<int>(b, P.o_rbmeta);
+    D.h_list = at<int>(b, P.o_hlist);
+    D.h_late = at<int>(b, P.o_hlate);
+    D.h_meta = at<int>(b, P.o_hmeta);
     D.cta_rep = at<int>(b, P.o_ctarep);
     // test hook for the barrier time-out path: HD_TEST_SKIP_ARRIVE=<replica>
     D.fault_rep = -1;
@@ -614,6 +645,7 @@ void fill_dev(hd_ctx *c) {
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
         D.nl_grid = nsm * 4;
+        D.hot_grid = std::min(P.ntile * P.split, nsm * std::max(1, 768 / P.block));   // what is resident at once
     }
     // quench view: the copy of the positions and its own velocity, force,
     // fixed-point image, rebuild flags and tile sums
@@ -627,7 +659,7 @@ void fill_dev(hd_ctx *c) {
         Q.v32 = at<float4>(b, P.o_vq);
         Q.f32 = at<float4>(b, P.o_fq);
     }
-    Q.rec = at<AtomRec>(b, P.o_qpfix);
+    Q.p = at<int4>(b, P.o_qpfix);
     Q.pfixb = at<int4>(b, P.o_qpfixb);
     Q.rebuild = at<int>(b, P.o_qrebuild);
     Q.part = at<double>(b, P.o_qpart);
@@ -640,18 +672,12 @@ void set_scalars(Dev &D, const hd_params *p) {
     const double rl = p->rc + p->skin;
     D.rl2 = rl * rl;
     D.half_skin2 = 0.25 * p->skin * p->skin;
-    D.rc2f = (float)D.rc2;
     D.rl2_lo_f = (float)(D.rl2 * (1.0 - 1.0 / 4096.0));
     D.rl2_hi_f = (float)(D.rl2 * (1.0 + 1.0 / 4096.0));
-    // FP32 r^2 of the split sweep is within ~3e-7 (relative) of the oracle's
-    // FP64 r^2 (fixed-point rounding of positions plus FP32 rounding); the
-    // band decided in FP64 is 2^-20 ~ 9.5e-7 wide on each side
     D.rc2_lo_f = (float)(D.rc2 * (1.0 - 1.0 / 1048576.0));
-    D.rc2_hi_f = (float)(D.rc2 * (1.0 + 1.0 / 1048576.0));
     D.half_skin2_f = (float)(D.half_skin2 * (1.0 - 1e-4));
     D.seed_lo = (uint32_t)p->seed;
     D.seed_hi = (uint32_t)(p->seed >> 32);
-    D.pair_x2 = p->pair_kernel == 1 ? 1 : 0;
 }
 
 hd_status check_device(hd_ctx *c) {
@@ -677,15 +703,16 @@ hd_status upload_reps(hd_ctx *c) {
 }
 
 // Kernels of one BAOAB step after the opening half (list, pair, scalars, update).
-void queue_step(hd_ctx *c, int mode, std::vector<hd_ctx::Span> *sink) {
+// next_last: the step after this one is the last of its call.
+void queue_step(hd_ctx *c, int mode, bool next_last, std::vector<hd_ctx::Span> *sink) {
     // per-atom energies are observables only: computed on the last step of a call
-    const bool last = !(mode & MODE_OPEN);
+    const bool last = !(mode & MODE_OPEN), lazy = c->D.lazy_h && !last;
     { Timed t(c, sink, T_REBUILD); launch_rebuild_prep(c->D, c->s); }
     { Timed t(c, sink, T_NLIST); launch_nlist(c->D, c->s); }
-    { Timed t(c, sink, T_PAIR); launch_pair(c->D, false, last, c->s); }
+    { Timed t(c, sink, T_PAIR); launch_pair(c->D, last ? PAIR_ENERGY : lazy ? PAIR_LAZY : PAIR_FULL, c->s); }
     if (c->D.any_eig) { Timed t(c, sink, T_EIG); launch_eig(c->D, c->s); }
-    { Timed t(c, sink, T_SCALAR); launch_scalar(c->D, mode, c->s); }
-    c->launches += c->D.any_eig ? 2 : 0;
+    { Timed t(c, sink, T_SCALAR); launch_scalar(c->D, mode, lazy, !last && !next_last, c->s); }
+    c->launches += (c->D.any_eig ? 2 : 0) + (lazy && c->D.bias_on ? 2 : 0);
     if (!c->D.any_nhc) {
         { Timed t(c, sink, T_UPDATE); launch_update(c->D, mode, c->s); }
         c->launches += 8;
@@ -700,14 +727,14 @@ void queue_step(hd_ctx *c, int mode, std::vector<hd_ctx::Span> *sink) {
 }
 
 void queue_steps(hd_ctx *c, int n, std::vector<hd_ctx::Span> *sink) {
-    { Timed t(c, sink, T_SCALAR); launch_scalar(c->D, MODE_OPEN, c->s); }
+    { Timed t(c, sink, T_SCALAR); launch_scalar(c->D, MODE_OPEN, false, n > 1, c->s); }
     if (c->D.any_nhc) {
         launch_nhc(c->D, MODE_OPEN, c->s);
         c->launches += 1;
     }
     { Timed t(c, sink, T_UPDATE); launch_update(c->D, c->D.any_nhc ? (MODE_OPEN | MODE_NHC) : MODE_OPEN, c->s); }
     c->launches += 2;
-    for (int k = 1; k <= n; ++k) queue_step(c, k < n ? (MODE_CLOSE | MODE_OPEN) : MODE_CLOSE, sink);
+    for (int k = 1; k <= n; ++k) queue_step(c, k < n ? (MODE_CLOSE | MODE_OPEN) : MODE_CLOSE, k + 1 == n, sink);
 }
 
 hd_status refresh_md(hd_ctx *c, bool relist) {
@@ -720,9 +747,9 @@ hd_status refresh_md(hd_ctx *c, bool relist) {
         c->launches += 5;
         CK(cudaStreamSynchronize(c->s));
     }
-    launch_pair(c->D, false, true, c->s);
+    launch_pair(c->D, PAIR_ENERGY, c->s);
     launch_eig(c->D, c->s);
-    launch_scalar(c->D, 0, c->s);
+    launch_scalar(c->D, 0, false, false, c->s);
     c->launches += 2 + (c->D.any_eig ? 2 : 0);
     CK(cudaGetLastError());
     return HD_OK;
@@ -815,7 +842,7 @@ bool setup_persistent(hd_ctx *c) {
     long long tot = 0;
     for (int r = 0; r < P.nrep; ++r) {
         int k = (int)std::floor(w[r] / wsum * (double)maxg);
-        k = std::max(1, std::min(k, P.rep[r].ntile));
+        k = std::max(1, std::min(k, P.rep[r].ntile * P.split));
         cnt[r] = k;
         tot += k;
     }
@@ -882,12 +909,20 @@ hd_status hd_create(const hd_replica_desc *reps, int n_rep, const hd_params *p, 
     c->D.any_nhc = 0;
     for (int r = 0; r < n_rep; ++r) c->D.any_nhc |= reps[r].nhc_len > 0;
     c->Q.any_nhc = c->D.any_nhc;
+    // Leave the Hessian term out of the sweeps where it is not used: always
+    // without a bias; with one, where the sweep is long enough to pay for the
+    // two launches more (~5 us) that a step then takes.  Measured per sweep with
+    // and without it: 259 and ~150 us at 913,408 atoms (split form), 54 and 49
+    // at 121,000, where the launches cost what it saves; 514 and 327 us at
+    // 57,088 in the FP64 form, whose pipe the term fills.  The eigenvalue bias
+    // keeps the plain order.
+    c->D.lazy_h = !c->P.any_eig && (!c->D.bias_on || c->P.natom >= (c->P.prec == HD_FP64 ? 8192 : 200000));
     Plan &P = c->P;
     const size_t N = P.natom;
     CK(cudaMemsetAsync(c->ws, 0, P.bytes, c->s));
     // host staging
     std::vector<dbl4> hx(N), hxo(N);
-    std::vector<AtomRec> hp(N);
+    std::vector<int4> hp(N);
     std::vector<char> hv(N * sizeof(dbl4));
     std::vector<RepState> hst(P.nrep);
     std::vector<int> draw(P.nrep), two(P.nrep, 2);
@@ -911,8 +946,7 @@ hd_status hd_create(const hd_replica_desc *reps, int n_rep, const hd_params *p, 
             const double *xo = d.pos_ref ? d.pos_ref + 3 * i : x;
             hx[a0 + sl] = make_dbl4(x[0], x[1], x[2], (double)d.type[i]);
             hxo[a0 + sl] = make_dbl4(xo[0], xo[1], xo[2], 0.0);
-            hp[a0 + sl].p = make_int4(0, 0, 0, (int)d.type[i] | ((int)d.role[i] << 8));
-            hp[a0 + sl].d = make_int4(0, 0, 0, 0);
+            hp[a0 + sl] = make_int4(0, 0, 0, (int)d.type[i] | ((int)d.role[i] << 8));
             double v[3] = {0, 0, 0};
             if (d.vel && d.role[i] != 0)
                 for (int a = 0; a < 3; ++a) v[a] = d.vel[3 * i + a];
@@ -927,7 +961,7 @@ hd_status hd_create(const hd_replica_desc *reps, int n_rep, const hd_params *p, 
     CK(cudaMemcpyAsync((void *)c->D.tile_n, P.tile_n.data(), P.ntile * 4, cudaMemcpyHostToDevice, c->s));
     CK(cudaMemcpyAsync(c->D.x, hx.data(), N * sizeof(dbl4), cudaMemcpyHostToDevice, c->s));
     CK(cudaMemcpyAsync(c->D.xo, hxo.data(), N * sizeof(dbl4), cudaMemcpyHostToDevice, c->s));
-    CK(cudaMemcpyAsync(c->D.rec, hp.data(), N * sizeof(AtomRec), cudaMemcpyHostToDevice, c->s));
+    CK(cudaMemcpyAsync(c->D.p, hp.data(), N * sizeof(int4), cudaMemcpyHostToDevice, c->s));
     CK(cudaMemcpyAsync((void *)c->D.orig, P.slot_orig.data(), N * 4, cudaMemcpyHostToDevice, c->s));
     CK(cudaMemcpyAsync((void *)c->D.bond_off, P.bond_off.data(), (N + 1) * 4, cudaMemcpyHostToDevice, c->s));
     if (!P.bond_j.empty())
@@ -938,9 +972,9 @@ hd_status hd_create(const hd_replica_desc *reps, int n_rep, const hd_params *p, 
     CK(cudaMemcpyAsync(c->D.rebuild, two.data(), P.nrep * 4, cudaMemcpyHostToDevice, c->s));
     launch_init(c->D, d_draw, c->s);
     launch_rebuild(c->D, c->s);
-    launch_pair(c->D, false, true, c->s);
+    launch_pair(c->D, PAIR_ENERGY, c->s);
     launch_eig(c->D, c->s);
-    launch_scalar(c->D, 0, c->s);
+    launch_scalar(c->D, 0, false, false, c->s);
     launch_update(c->D, MODE_KIN, c->s);  // kinetic energy of the initial velocities
     launch_nhc(c->D, MODE_KIN, c->s);     // the chains start from it
     launch_obs(c->D, c->s);
@@ -967,7 +1001,7 @@ hd_status hd_set_slider(hd_ctx *c, const double *slider, int requench_ref) {
         c->P.rep[r].slide_step0 = c->step0[r] + c->steps_done;   // a moving slider restarts from here
     }
     if (upload_reps(c) != HD_OK) return c->status;
-    launch_scalar(c->D, 0, c->s);
+    launch_scalar(c->D, 0, false, false, c->s);
     c->launches += 1;
     CK(cudaGetLastError());
     // FIRE from dt0 = 0.005 (fastest on thermal LJ states); the rigid body's
@@ -989,7 +1023,7 @@ hd_status hd_set_bias(hd_ctx *c, const double *bias) {
         c->P.rep[r].m_exp = (int)bias[4 * r + 3];
     }
     if (upload_reps(c) != HD_OK) return c->status;
-    launch_scalar(c->D, 0, c->s);
+    launch_scalar(c->D, 0, false, false, c->s);
     c->launches += 1;
     CK(cudaGetLastError());
     return HD_OK;
@@ -1074,7 +1108,8 @@ hd_status hd_step(hd_ctx *c, int n_steps) {
     }
     CK(cudaGraphLaunch(it->second, c->s));
     if (c->timing) c->graph_pending.push_back(key);
-    c->launches += (c->D.any_nhc ? 3 + 10LL * n_steps : 2 + 8LL * n_steps) + (c->D.any_eig ? 2LL * n_steps : 0);
+    c->launches += (c->D.any_nhc ? 3 + 10LL * n_steps : 2 + 8LL * n_steps) + (c->D.any_eig ? 2LL * n_steps : 0) +
+                   (c->D.lazy_h && c->D.bias_on ? 2LL * (n_steps - 1) : 0);
     return HD_OK;
 }
 
@@ -1241,22 +1276,23 @@ hd_status hd_read(hd_ctx *c, int field, int replica, void *h_dst, size_t bytes) 
                       cudaMemcpyDeviceToHost));
         c->d2h += 4LL * n;
         int *o = (int *)h_dst;
-        for (size_t sl = 0; sl < n; ++sl) o[P.slot_orig[a0 + sl]] = tmp[sl];
+        for (size_t sl = 0; sl < n; ++sl) o[P.slot_orig[a0 + sl]] = field == HD_FIELD_CELL ? tmp[sl] : NB_LEN(tmp[sl]);
         return HD_OK;
     }
     case HD_FIELD_NBR: {
         // rows in input numbering, ascending in j
         if (!need(n * P.maxnb * 4)) break;
-        std::vector<int> cnt(n), slab(n * P.maxnb);
+        const size_t blk = (size_t)c->D.ngrp * 128, nblk = (n + 31) / 32;    // entries of 32 rows
+        std::vector<int> cnt(n), slab(nblk * blk);
         CK(cudaMemcpy(cnt.data(), c->D.nnb + a0, n * 4, cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy2D(slab.data(), n * 4, c->D.nbr + a0, (size_t)P.natom * 4, n * 4, P.maxnb, cudaMemcpyDeviceToHost));
-        c->d2h += 4LL * n * (1 + P.maxnb);
+        CK(cudaMemcpy(slab.data(), c->D.nbr + R.wg0 * blk, slab.size() * 4, cudaMemcpyDeviceToHost));
+        c->d2h += 4LL * (n + slab.size());
         int *o = (int *)h_dst;
         std::vector<int> row;
         for (size_t sl = 0; sl < n; ++sl) {
             const int i = P.slot_orig[a0 + sl];
             row.clear();
-            for (int k = 0; k < cnt[sl] && k < P.maxnb; ++k) row.push_back(P.slot_orig[slab[(size_t)k * n + sl]]);
+            for (int k = 0; k < NB_LEN(cnt[sl]); ++k) row.push_back(P.slot_orig[slab[(sl >> 5) * blk + (size_t)(k >> 2) * 128 + (sl & 31) * 4 + (k & 3)]]);
             std::sort(row.begin(), row.end());
             for (int k = 0; k < P.maxnb; ++k) o[(size_t)i * P.maxnb + k] = k < (int)row.size() ? row[k] : -1;
         }

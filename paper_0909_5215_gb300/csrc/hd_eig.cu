@@ -34,7 +34,7 @@ namespace {
 
 constexpr int EIG_THREADS = 512;
 
-__device__ __forceinline__ int role_of(const Dev &D, int i) { return (D.rec[i].p.w >> 8) & 0xff; }
+__device__ __forceinline__ int role_of(const Dev &D, int i) { return (D.p[i].w >> 8) & 0xff; }
 
 // Sum of NV values over the CTA; every thread receives the sums.
 template <int NV>
@@ -85,9 +85,10 @@ __device__ __forceinline__ dbl4 hessvec_atom(const Dev &D, const RepDev &R, int 
     const int ti = (int)xi.w;
     const dbl4 ui = u[i - a0];
     double hx = 0, hy = 0, hz = 0;
-    const int nn = D.nnb[i];
+    const int nn = NB_LEN(D.nnb[i]);
+    const size_t row4 = nbr_row4(D, R, i);
     for (int k = 0; k < nn; ++k) {
-        const int j = D.nbr[(size_t)k * D.natom + i];
+        const int j = D.nbr[nbr_at(row4, k)];
         const dbl4 xj = D.x[j];
         const double dx = mi64(R, 0, xi.x - xj.x), dy = mi64(R, 1, xi.y - xj.y), dz = mi64(R, 2, xi.z - xj.z);
         const double r2 = dx * dx + dy * dy + dz * dz;
@@ -376,9 +377,10 @@ __global__ void __launch_bounds__(128) k_eig_grad(Dev D) {
             gy += cr * dy + 2.0 * B * rw * wy;
             gz += cr * dz + 2.0 * B * rw * wz;
         };
-        const int nn = D.nnb[i];
+        const int nn = NB_LEN(D.nnb[i]);
+        const size_t row4 = nbr_row4(D, R, i);
         for (int k = 0; k < nn; ++k) {
-            const int j = D.nbr[(size_t)k * D.natom + i];
+            const int j = D.nbr[nbr_at(row4, k)];
             const dbl4 xj = D.x[j];
             const double dx = mi64(R, 0, xi.x - xj.x), dy = mi64(R, 1, xi.y - xj.y), dz = mi64(R, 2, xi.z - xj.z);
             const double r2 = dx * dx + dy * dy + dz * dz;

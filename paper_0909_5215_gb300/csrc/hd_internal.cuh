@@ -7,17 +7,23 @@
 //     x      dbl4  FP64 position, w = LJ type           (never wrapped)
 //     xo     dbl4  basin minimum r_O
 //     v      dbl4     velocity (FP64 in both forms)
-//     po     int4 (split form)  fixed-point image of r_O
+//     p      int4    32-bit fixed-point position (w = type | role << 8), the
+//                     record that the pair sweep gathers per neighbour
+//     po     int4 (split form)  fixed-point image of r_O; r - r_O is the
+//                     difference of the two images
 //     f      dbl4 | float4   LJ force, w = per-atom energy (half of each pair)
 //     h      dbl4 | float4   H.(r - r_O), spring term included
 //     dr     dbl4 | float4   r - r_O
-//     rec    AtomRec  32-bit fixed-point position (w = type | role << 8) and,
-//                     in the split form, r - r_O as the difference of the
-//                     images of r and r_O, 32 bytes
-//     pfixb  int4     pfix at the last list build (displacement check)
-//     nbr    int32 [maxnb][natom] column-major Verlet list (global j), nnb int32
+//     pfixb  int4     p at the last list build (displacement check)
+//     nbr    int32    Verlet list (global j), nnb int32 row lengths.  32 atoms of
+//                     a replica share a block [ceil(maxnb / 4)][32][4]: four
+//                     entries of a row are one 16-byte load, a warp's loads are
+//                     contiguous and the position in the row is an immediate
+//                     offset.  A row's last group of four is filled up with the
+//                     row's own atom, so that every entry loaded is an index
 //   per cell: count int32, atoms int32 [cell_cap]
-//   per tile (block atoms of one replica): NPART FP64 partial sums, FP64 K part
+//   per tile (block atoms of one replica): split x NPART FP64 partial sums
+//     (split: lanes that share a row of the pair sweep), FP64 K part
 //   per replica: RepDev (settings), RepState (clocks, body), Scal (scalars)
 //
 // Fixed point: on a periodic axis x_fix = rint(x * 2^(32+k) / L) taken modulo
@@ -59,18 +65,9 @@ enum { QP_FMAX2 = 0, QP_P = 1, QP_VV = 2, QP_FF = 3, QP_FRIG = 4, QP_XRIG = 7, Q
 enum { MODE_CLOSE = 1, MODE_OPEN = 2, MODE_KIN = 4, MODE_NHC = 8, MODE_SCALE = 16 };
 enum { ROLE_FIXED = 0, ROLE_MOBILE = 1, ROLE_RIGID = 2 };
 
-// Per-atom record read by the pair sweep: fixed-point position (w = type |
-// role << 8) and, in the split form, r - r_O on the same fixed-point grid (w
-// unused); one 32-byte sector.  Differences of two atoms' r - r_O, which the
-// Hessian-vector term takes, are then exact integers.
-struct __align__(32) AtomRec {
-    int4 p;
-    int4 d;
-};
-
 struct RepDev {
     int dim, n, atom0, tile0, ntile, nrig, m_exp, rep_id;
-    int cell0, ncell, vert, pad0;
+    int cell0, ncell, vert, wg0;          // wg0: first 32-atom block of the list
     int nc[3], periodic[3];
     double L[3], invL[3];
     double kT, beta, c_ou, s_ou, kspring, fnormal, slider[2];
@@ -96,10 +93,14 @@ struct RepDev {
     int exact_r2, zshift, shift_y, shift_z;
     float u2_42, u2_21, u2_0, u2lo_42;     // u^2 2^42, u^2 2^21, u^2 (FP32) and the low part of u^2 2^42
     float lsb_rel[3];            // (unit - fl32(unit)) / fl32(unit) per axis
-    float pad2;
-    float r0sq_hi[2][2], r0sq_lo[2][2];  // 2^(1/3) sigma_ab^2 (LJ minimum, squared) as hi + lo
-    float eps24f[2][2], eps96f[2][2];    // 24 eps_ab, 96 eps_ab (FP32 rounding) ...
-    float eps24l[2][2], eps96l[2][2];    // ... and the remainders (hi + lo = the FP64 value)
+    // pair sweep: lengths in the common unit u where the axes share one
+    // (exact_r2), else in the axes' own units; separations are integer x
+    // px_scale, the finished sums are multiplied by out = hi + lo (1/u, or the
+    // rounding of lsb undone)
+    float px_scale[3], out_hi[3], out_lo[3];
+    float rc2u_lo, rc2u_hi, near2u;      // rc^2 (1 -+ 2^-20); the exact r^2 is taken below near2u = (4/3) r_0^2
+    float r0u_hi[2][2], r0u_lo[2][2];    // r_0^2 = 2^(1/3) sigma_ab^2 (LJ minimum, squared) as hi + lo
+    float eps12f[2][2], eps12l[2][2];    // 12 eps_ab as hi + lo
     float rA2f;                  // list class A (first shell): FP32 r^2 below this at build time
     float kbondf;                // Eq. 12 bonds: stiffness (FP32)
     double kbond, rbond;         // Eq. 12 bonds: stiffness, rest length
@@ -126,6 +127,7 @@ struct RepState {
     double q_dt, q_alpha, q_vb[3], q_fmax, q_disp;
     int q_npos, q_iter, q_done, q_flag;
     int q_stay, pad_q;           // the quench stopped inside its basin (at ftol_stay, not ftol)
+    double h_sig, h_step;        // the last slope and the largest recent change of it (decaying)
 };
 
 struct Scal {
@@ -139,15 +141,17 @@ struct Scal {
     double nhc_scale;            // chain: scale of the mobile velocities before the next kick
     double ce;                   // eigenvalue bias: F_tot += ce grad(epsilon), ce = -dDeltaV/depsilon
     double dV1, dV2;             // the two terms of Eq. 13
+    int need_h, pad_h;           // the next sweep takes H.(r - r_O) for this replica
 };
 
 struct Dev {
     int nrep, ntile, natom, maxnb, cell_cap, ncell, prec, bias_on, block;
+    int ngrp, split;             // groups of four per list row; lanes that share a row of the pair sweep (1 or 4)
     int q_method, max_cells;        // max_cells: largest cell count of one replica
     double dt, rc2, rl2, half_skin2, q_ftol, q_step, q_theta;
     double q_ftol_stay, q_keep2;    // quench: early stop inside the basin (0: off), (theta/2)^2
-    float rc2f, rl2_lo_f, rl2_hi_f, half_skin2_f;
-    float rc2_lo_f, rc2_hi_f;    // rc^2 (1 -+ 2^-20): band decided in FP64
+    float rl2_lo_f, rl2_hi_f, half_skin2_f;
+    float rc2_lo_f;              // rc^2 (1 - 2^-20): list class B ends here
     uint32_t seed_lo, seed_hi;
     const RepDev *rep;
     RepState *st;
@@ -158,7 +162,7 @@ struct Dev {
     dbl4 *v64, *f64, *h64, *dr64;
     float4 *v32, *f32, *h32;     // v32: the quench's FIRE velocities (split form)
     int4 *po;                    // split form: fixed-point image of r_O (r - r_O = image difference)
-    AtomRec *rec;                // fixed-point position + FP32 r - r_O
+    int4 *p;                     // fixed-point position, w = type | role << 8
     int4 *pfixb;
     int *cellid, *nnb, *nbr, *cell_cnt, *cell_atoms;
     int *rebuild;                // per replica: list rebuild requested
@@ -170,6 +174,9 @@ struct Dev {
     int *rb_list;                // replicas whose list is rebuilt, ascending (count rb_meta[0])
     int *rb_off, *rb_aoff;       // [count + 1] first compacted cell / atom of each of them
     int *rb_meta;                // {count, compacted cells, compacted atoms}
+    int *h_list, *h_late;        // replicas to sweep with H.(r - r_O): expected in their band; found there
+    int *h_meta;                 // {count of h_list, of h_late, CTAs done with each}
+    int lazy_h, hot_grid;        // the per-phase driver's MD sweeps are PAIR_LAZY; CTAs of the listed sweeps
     const int *cta_rep;          // persistent launch: replica of each CTA (-1: spare)
     const int *pg_first, *pg_count;  // persistent launch: first CTA and CTA count of each replica
     const int *bond_off, *bond_j;    // per slot: bond partners (slots) in bond_j[bond_off[i] .. bond_off[i+1])
@@ -177,7 +184,6 @@ struct Dev {
     int nl_pow2, nl_grid;        // neighbour-row buffer (power of two >= maxnb), k_nlist CTAs
     int any_nhc;                 // some replica runs a Nose-Hoover chain: the update splits around it
     int any_eig;                 // some replica has the eigenvalue bias
-    int pair_x2;                 // split form: the packed FP32x2 pair sweep (tiles <= 128 atoms)
     dbl4 *eq, *ev, *ew, *eg;     // eigenvalue bias: Krylov bases, eigenvector, work vector, grad epsilon
     double *ealpha, *ebeta, *ey, *ecoef;  // tridiagonal (alpha, beta), its eigenvector, coefficients
     double *epart;               // per tile: sum of grad epsilon over rigid atoms (4 doubles)
@@ -329,6 +335,31 @@ __device__ __forceinline__ void r2_split(const RepDev &R, int ix, int iy, int iz
     const float eb = (a - hi) + b;
     lo = (ea + eb) + fmaf(f0, R.u2_0, f2 * R.u2lo_42);
 }
+
+// The same in units of u^2 (the pieces' weights are powers of two, so only
+// the two sums round).
+__device__ __forceinline__ void r2_units(int ix, int iy, int iz, float &hi, float &lo) {
+    unsigned long long q = (unsigned long long)((long long)ix * (long long)ix);
+    q += (unsigned long long)((long long)iy * (long long)iy);
+    q += (unsigned long long)((long long)iz * (long long)iz);
+    const float f0 = exact_f23((unsigned int)q & 0x1FFFFFu);
+    const float b = exact_f23((unsigned int)(q >> 21) & 0x1FFFFFu) * 2097152.f;
+    const float a = exact_f23((unsigned int)(q >> 42)) * 4398046511104.f;
+    hi = a + b;
+    lo = ((a - hi) + b) + f0;
+}
+
+// Row lengths: the flag says that the row or its atom holds a tip atom.
+constexpr int NB_MIXED = 1 << 30;
+__host__ __device__ __forceinline__ int NB_LEN(int v) { return v & (NB_MIXED - 1); }
+
+// Verlet list: first group of four of atom i's row, in int4 (the next group
+// is 32 further), and the place of its entry k.
+__device__ __forceinline__ size_t nbr_row4(const Dev &D, const RepDev &R, int i) {
+    const int li = i - R.atom0;
+    return ((size_t)(R.wg0 + (li >> 5)) * D.ngrp << 5) + (li & 31);
+}
+__device__ __forceinline__ size_t nbr_at(size_t row4, int k) { return ((row4 + ((size_t)(k >> 2) << 5)) << 2) + (k & 3); }
 
 template <typename T>
 __device__ __forceinline__ T warp_sum(T v) {

@@ -40,74 +40,65 @@ __device__ __forceinline__ void cta_reduce(double (&v)[NV], double *out, int max
     __syncthreads();
 }
 
-// Tile sums of the split form: slots PART_D2, PART_G, PART_V are per-atom
-// FP64 values (products of FP32 factors, exact in FP64) summed in FP64, since
-// sigma = G / d (Eq. 5) feeds the bias; slots [3, nf) are FP32 per-atom values
-// summed in FP32 within each warp; xr (rigid positions, FP64) go to slots
-// PART_XRIG..+2 when some lane holds a rigid atom.  Warp results are added in
-// FP64 in warp order.  Slots never written by a warp count as zero.
-__device__ __forceinline__ void tile_reduce_mixed(double (&d3)[3], float (&v)[12], int nf, double (&xr)[3],
-                                                  bool anyrig, double *out) {
-    __shared__ double sm[32][NPART];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    double wsum[NPART];
-#pragma unroll
-    for (int q = 0; q < NPART; ++q) wsum[q] = 0.0;
-#pragma unroll
-    for (int q = 0; q < 3; ++q) wsum[q] = warp_sum(d3[q]);
-#pragma unroll
-    for (int q = 3; q < 12; ++q)
-        if (q < nf) wsum[q] = (double)warp_sum(v[q]);
-    if (anyrig)
-#pragma unroll
-        for (int a = 0; a < 3; ++a) wsum[PART_XRIG + a] = warp_sum(xr[a]);
-    if (lane == 0)
-#pragma unroll
-        for (int q = 0; q < NPART; ++q) sm[w][q] = wsum[q];
-    __syncthreads();
-    if (threadIdx.x < NPART) {
-        const int q = threadIdx.x;
-        double a = sm[0][q];
-        for (int k = 1; k < nw; ++k) a += sm[k][q];
-        out[q] = a;
-    }
-    __syncthreads();
+// Warp sums of up to four doubles in 6 additions (one each: 20): the lanes
+// split between the values as they halve, so after two exchanges each holds
+// a partial sum of one value.  The sum of v[q] ends in lane 8 q.  The FP64
+// pipe takes a warp instruction every 16 cycles an SM, so these sums, not
+// their latency, were a quarter of the pair sweep's time.
+__device__ __forceinline__ double warp_sum4(double v0, double v1, double v2, double v3) {
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const bool up = lane & 16, up2 = lane & 8;
+    // lanes 0-15 keep (v0, v1), lanes 16-31 keep (v2, v3)
+    const double s0 = up ? v0 : v2, s1 = up ? v1 : v3;
+    const double k0 = (up ? v2 : v0) + __shfl_xor_sync(full, s0, 16), k1 = (up ? v3 : v1) + __shfl_xor_sync(full, s1, 16);
+    double k = (up2 ? k1 : k0) + __shfl_xor_sync(full, up2 ? k0 : k1, 8);
+    k += __shfl_xor_sync(full, k, 4);
+    k += __shfl_xor_sync(full, k, 2);
+    k += __shfl_xor_sync(full, k, 1);
+    return k;
 }
 
-// Quench tile sums: slot QP_FMAX2 is a max; FIRE's power F.v, v.v and F.F
-// (pvf, FP64 per-atom products of FP32 factors) are summed in FP64, since the
-// sign of the power near convergence is a small difference of large sums; the
-// rigid forces are FP32 sums within warps.
-__device__ __forceinline__ void tile_reduce_quench(float (&v)[12], double (&pvf)[3], double (&xr)[3], bool anyrig,
-                                                   double *out) {
-    __shared__ double sm[32][NPART];
+// Tile sums of the split form.  Per-atom values are FP64 (products of FP32
+// factors, exact in FP64) where sigma = G / d (Eq. 5) or the sign of FIRE's
+// power depends on them: sum[0..3], summed in FP64.  sf[0..nf) are FP32
+// per-atom values (rigid atoms) summed in FP32 within a warp, xr the rigid
+// positions, both only where some lane holds a rigid atom (few warps do).
+// fm: largest of an FP32 value, or negative for none.  Warp results are
+// combined in FP64 in warp order.  out: slots in the order of `slot`.
+struct TileSlots {
+    int sum[4], f0, x0, max;      // out index of the sums (-1: unused), first FP32 sum, first position, the maximum
+};
+template <int NF>
+__device__ __forceinline__ void tile_reduce(double v0, double v1, double v2, double v3, const float (&sf)[NF],
+                                            const double (&xr)[3], bool anyrig, float fm, TileSlots L, double *out) {
+    __shared__ double sm[8][NPART];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    double wsum[NPART];
+    if (lane < NPART) sm[w][lane] = 0.0;
+    __syncwarp();
+    const double s = warp_sum4(v0, v1, v2, v3);
+    const int q = L.sum[lane >> 3];
+    if ((lane & 7) == 0 && q >= 0) sm[w][q] = s;
+    if (L.max >= 0) {
 #pragma unroll
-    for (int q = 0; q < NPART; ++q) wsum[q] = 0.0;
-    float m = v[QP_FMAX2];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_down_sync(0xffffffffu, m, o));
-    wsum[QP_FMAX2] = (double)m;
-    wsum[QP_P] = warp_sum(pvf[0]);
-    wsum[QP_VV] = warp_sum(pvf[1]);
-    wsum[QP_FF] = warp_sum(pvf[2]);
+        for (int o = 16; o > 0; o >>= 1) fm = fmaxf(fm, __shfl_xor_sync(0xffffffffu, fm, o));
+        if (lane == 0) sm[w][L.max] = (double)fm;
+    }
     if (anyrig) {
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            wsum[QP_FRIG + a] = (double)warp_sum(v[QP_FRIG + a]);
-            wsum[QP_XRIG + a] = warp_sum(xr[a]);
+        for (int k = 0; k < NF; ++k) {
+            const float a = warp_sum(sf[k]);
+            if (lane == 0) sm[w][L.f0 + k] = (double)a;
         }
+        const double x = warp_sum4(xr[0], xr[1], xr[2], 0.0);
+        if ((lane & 7) == 0 && lane < 24) sm[w][L.x0 + (lane >> 3)] = x;
     }
-    if (lane == 0)
-#pragma unroll
-        for (int q = 0; q < NPART; ++q) sm[w][q] = wsum[q];
     __syncthreads();
     if (threadIdx.x < NPART) {
-        const int q = threadIdx.x;
-        double a = sm[0][q];
-        for (int k = 1; k < nw; ++k) a = (q == QP_FMAX2) ? fmax(a, sm[k][q]) : a + sm[k][q];
-        out[q] = a;
+        const int k = threadIdx.x;
+        double a = sm[0][k];
+        for (int m = 1; m < nw; ++m) a = k == L.max ? fmax(a, sm[m][k]) : a + sm[m][k];
+        out[k] = a;
     }
     __syncthreads();
 }
@@ -121,17 +112,15 @@ __global__ void k_init(Dev D, const int *draw_vel) {
     const int i = D.tile_start[t] + threadIdx.x;
     const RepDev &R = D.rep[r];
     dbl4 x = D.x[i], xo = D.xo[i];
-    int4 p = D.rec[i].p;  // w (type | role << 8) preset by the host
+    int4 p = D.p[i];  // w (type | role << 8) preset by the host
     p = fix_pos(R, x, p.w);
-    D.rec[i].p = p;
+    D.p[i] = p;
     D.pfixb[i] = p;
     const int role = (p.w >> 8) & 0xff;
     if (D.prec == HD_FP64) {
         D.dr64[i] = make_dbl4(x.x - xo.x, x.y - xo.y, x.z - xo.z, 0.0);
     } else {
-        const int4 po = fix_pos(R, xo, 0);
-        D.po[i] = po;
-        D.rec[i].d = img_diff(p, po);
+        D.po[i] = fix_pos(R, xo, 0);
     }
     if (draw_vel[r]) {
         double v0 = 0, v1 = 0, v2 = 0;
@@ -215,7 +204,7 @@ __global__ void k_cell_clear(Dev D) {
 
 __device__ __forceinline__ void dev_bin_atom(const Dev &D, int r, int i) {
     const RepDev &R = D.rep[r];
-    const int4 p = D.rec[i].p;
+    const int4 p = D.p[i];
     const dbl4 x = D.x[i];
     const int cx = cell_of(R, 0, x.x), cy = cell_of(R, 1, x.y), cz = cell_of(R, 2, x.z);
     D.cellid[i] = cx | (cy << 10) | (cz << 20);
@@ -380,11 +369,12 @@ __device__ __forceinline__ void dev_nlist_cell(const Dev &D, int r, int c, NlSme
             }
             int4 pp[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) pp[u] = jj[u] >= 0 ? D.rec[jj[u]].p : make_int4(0, 0, 0, 0);
+            for (int u = 0; u < 4; ++u) pp[u] = jj[u] >= 0 ? D.p[jj[u]] : make_int4(0, 0, 0, 0);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int idx = base + u * blockDim.x;
-                if (idx < tot) sp[idx] = make_int4(pp[u].x, pp[u].y, pp[u].z, jj[u]);   // w: the candidate's slot
+                // w: the candidate's slot, top bit its type
+                if (idx < tot) sp[idx] = make_int4(pp[u].x, pp[u].y, pp[u].z, jj[u] | (pp[u].w << 31));
             }
         }
     }
@@ -392,13 +382,14 @@ __device__ __forceinline__ void dev_nlist_cell(const Dev &D, int r, int c, NlSme
     const int tot = M.tot, cap = D.maxnb;
     const unsigned full = 0xffffffffu;
     const float lx = R.fx_lsb[0], ly = R.fx_lsb[1], lz = R.fx_lsb[2];
-    const size_t stride = (size_t)D.natom;
     // per warp: three ballot masks (classes A, B, C) per 32 candidates
     unsigned *msk = smask + (size_t)w * nl_mask_words(D);
     for (int a = w; a < m; a += nw) {
         const int slot = M.off[M.kc] + a;
         const int4 pi = sp[slot];
-        const int i = pi.w;
+        const int i = pi.w & 0x7fffffff;
+        const size_t row4 = nbr_row4(D, R, i);
+        unsigned mixed = (unsigned)pi.w >> 31;
         int nA = 0, nB = 0, nC = 0;
         // pass 1: classify every candidate, count the classes
         for (int base = 0; base < tot; base += 32) {
@@ -406,7 +397,7 @@ __device__ __forceinline__ void dev_nlist_cell(const Dev &D, int r, int c, NlSme
             int cl = 0;
             if (q < tot) {
                 const int4 pj = sp[q];
-                const int j = pj.w;
+                const int j = pj.w & 0x7fffffff;
                 if (j != i) {
                     const float dx = (float)(int)((unsigned)pi.x - (unsigned)pj.x) * lx;
                     const float dy = (float)(int)((unsigned)pi.y - (unsigned)pj.y) * ly;
@@ -416,7 +407,10 @@ __device__ __forceinline__ void dev_nlist_cell(const Dev &D, int r, int c, NlSme
                     if (r2 < D.rl2_lo_f) in = true;
                     else if (r2 >= D.rl2_hi_f) in = false;
                     else in = exact_r2(R, D.x[i], D.x[j]) < D.rl2;
-                    if (in) cl = r2 < R.rA2f ? 1 : (r2 < D.rc2_lo_f ? 2 : 3);
+                    if (in) {
+                        cl = r2 < R.rA2f ? 1 : (r2 < D.rc2_lo_f ? 2 : 3);
+                        mixed |= (unsigned)pj.w >> 31;
+                    }
                 }
             }
             const unsigned mA = __ballot_sync(full, cl == 1), mB = __ballot_sync(full, cl == 2),
@@ -440,17 +434,21 @@ __device__ __forceinline__ void dev_nlist_cell(const Dev &D, int r, int c, NlSme
             if (cl) {
                 const int pos = cl == 1 ? bA + __popc(mA & below) : (cl == 2 ? bB + __popc(mB & below)
                                                                              : bC + __popc(mC & below));
-                if (pos < cap) D.nbr[(size_t)pos * stride + i] = sp[base + lane].w;
+                if (pos < cap) D.nbr[nbr_at(row4, pos)] = sp[base + lane].w & 0x7fffffff;
             }
             bA += __popc(mA);
             bB += __popc(mB);
             bC += __popc(mC);
         }
         __syncwarp();
-        if (lane == 0) {
-            const int n = nA + nB + nC;
-            D.nnb[i] = min(n, cap);
-            if (n > cap) set_err(D, HD_ERR_OVERFLOW, i, r);
+        {
+            const int n = nA + nB + nC, kept = min(n, cap);
+            const bool mx = __any_sync(full, mixed != 0);
+            if (kept + lane < ((kept + 3) & ~3)) D.nbr[nbr_at(row4, kept + lane)] = i;   // fill up the last group
+            if (lane == 0) {
+                D.nnb[i] = kept | (mx ? NB_MIXED : 0);
+                if (n > cap) set_err(D, HD_ERR_OVERFLOW, i, r);
+            }
         }
     }
     __syncthreads();  // the staging buffers are reused by the next cell
@@ -479,22 +477,30 @@ __global__ void __launch_bounds__(NL_THREADS) k_nlist(Dev D) {
 // (H dr)_i = sum_j [A (dr_i - dr_j) + B ((dr_i - dr_j) . r_ij) r_ij],
 // A = phi'/r, B = (phi'' - phi'/r)/r^2, with s = sigma_ab/r:
 //   -A = 24 eps s^6 (2 s^6 - 1)/r^2,   B = 96 eps s^6 (7 s^6 - 2)/r^4.
-// Q (quench): positions of the quench copy, no H.dr, quench partial sums.
-template <bool Q, bool E>
-__device__ __forceinline__ void dev_pair64(const Dev &D, int t) {
+// Q (quench): positions of the quench copy, quench partial sums.  E: per-atom
+// energies.  H: the Hessian term.
+// S: lanes of a warp that share one row (lane s takes groups s, s + S, ... of
+// four entries, the sums meet in a shuffle tree); a CTA then holds block / S
+// atoms of its tile and `unit` counts such parts.
+template <bool Q, bool E, bool H, int S>
+__device__ __forceinline__ void dev_pair64(const Dev &D, int unit) {
+    const int t = unit / S;
     const int r = D.tile_rep[t];
     if (Q && D.st[r].q_done) return;
     const RepDev &R = D.rep[r];
-    const bool act = threadIdx.x < D.tile_n[t];
-    const int i = D.tile_start[t] + (act ? threadIdx.x : 0);
+    const int sub = S > 1 ? (int)(threadIdx.x % S) : 0;
+    const int at = (unit % S) * (D.block / S) + (int)threadIdx.x / S;     // atom of the tile
+    const bool has = at < D.tile_n[t], act = has && sub == 0;
+    const int i = D.tile_start[t] + (has ? at : 0);
     const dbl4 xi = D.x[i];
     const int ti = (int)xi.w;
     const dbl4 dri = Q ? make_dbl4(0, 0, 0, 0) : D.dr64[i];
     double fx = 0, fy = 0, fz = 0, e = 0, hx = 0, hy = 0, hz = 0;
-    const int nn = act ? D.nnb[i] : 0;
+    const int nn = has ? NB_LEN(D.nnb[i]) : 0;
+    const size_t row4 = nbr_row4(D, R, i);
     const double rc2 = D.rc2;
-    for (int k = 0; k < nn; ++k) {
-        const int j = D.nbr[(size_t)k * D.natom + i];
+    for (int k = 4 * sub; k < nn; k += (k & 3) == 3 ? 4 * S - 3 : 1) {
+        const int j = D.nbr[nbr_at(row4, k)];
         const dbl4 xj = D.x[j];
         const double dx = mi64(R, 0, xi.x - xj.x), dy = mi64(R, 1, xi.y - xj.y), dz = mi64(R, 2, xi.z - xj.z);
         const double r2 = dx * dx + dy * dy + dz * dz;
@@ -509,7 +515,7 @@ __device__ __forceinline__ void dev_pair64(const Dev &D, int t) {
             fy += fr * dy;
             fz += fr * dz;
             if (E) e += 0.5 * (4.0 * eps * s6 * (s6 - 1.0) - R.shift[ti][tj]);
-            if (!Q) {
+            if (H) {
                 const dbl4 drj = D.dr64[j];
                 const double ux = dri.x - drj.x, uy = dri.y - drj.y, uz = dri.z - drj.z;
                 const double rdu = dx * ux + dy * uy + dz * uz;
@@ -534,7 +540,7 @@ __device__ __forceinline__ void dev_pair64(const Dev &D, int t) {
             fy -= A * dy;
             fz -= A * dz;
             if (E) e += 0.5 * (0.5 * R.kbond * db * db);
-            if (!Q) {
+            if (H) {
                 const dbl4 drj = D.dr64[j];
                 const double ux = dri.x - drj.x, uy = dri.y - drj.y, uz = dri.z - drj.z;
                 const double rdu = dx * ux + dy * uy + dz * uz;
@@ -545,14 +551,28 @@ __device__ __forceinline__ void dev_pair64(const Dev &D, int t) {
             }
         }
     }
-    const int role = act ? ((D.rec[i].p.w >> 8) & 0xff) : -1;
-    if (!Q && role == ROLE_RIGID) {
+    if (S > 1) {
+#pragma unroll
+        for (int o = 1; o < S; o <<= 1) {
+            fx += __shfl_xor_sync(0xffffffffu, fx, o);
+            fy += __shfl_xor_sync(0xffffffffu, fy, o);
+            fz += __shfl_xor_sync(0xffffffffu, fz, o);
+            if (E) e += __shfl_xor_sync(0xffffffffu, e, o);
+            if (H) {
+                hx += __shfl_xor_sync(0xffffffffu, hx, o);
+                hy += __shfl_xor_sync(0xffffffffu, hy, o);
+                hz += __shfl_xor_sync(0xffffffffu, hz, o);
+            }
+        }
+    }
+    const int role = act ? ((D.p[i].w >> 8) & 0xff) : -1;
+    if (H && role == ROLE_RIGID) {
         hx += R.kr_n * dri.x;
         if (R.dim == 3) hy += R.kr_n * dri.y;
     }
     if (act) {
         D.f64[i] = make_dbl4(fx, fy, fz, e);
-        if (!Q) D.h64[i] = make_dbl4(hx, hy, hz, 0.0);
+        if (H) D.h64[i] = make_dbl4(hx, hy, hz, 0.0);
     }
     const bool rig = role == ROLE_RIGID;
     if (!Q) {
@@ -568,7 +588,7 @@ __device__ __forceinline__ void dev_pair64(const Dev &D, int t) {
             v[PART_DRRIG] = dri.x; v[PART_DRRIG + 1] = dri.y; v[PART_DRRIG + 2] = dri.z;
             v[PART_XRIG] = xi.x; v[PART_XRIG + 1] = xi.y; v[PART_XRIG + 2] = xi.z;
         }
-        cta_reduce<NPART>(v, D.part + (size_t)t * NPART, -1);
+        cta_reduce<NPART>(v, D.part + (size_t)unit * NPART, -1);
     } else {
         double v[QPART] = {};
         if (role == ROLE_MOBILE) {
@@ -582,16 +602,38 @@ __device__ __forceinline__ void dev_pair64(const Dev &D, int t) {
             v[QP_FRIG] = fx; v[QP_FRIG + 1] = fy; v[QP_FRIG + 2] = fz;
             v[QP_XRIG] = xi.x; v[QP_XRIG + 1] = xi.y; v[QP_XRIG + 2] = xi.z;
         }
-        cta_reduce<QPART>(v, D.part + (size_t)t * NPART, QP_FMAX2);
+        cta_reduce<QPART>(v, D.part + (size_t)unit * NPART, QP_FMAX2);
     }
 }
 
-// Split form: positions are differenced exactly in 32-bit fixed point, the
-// pair arithmetic is FP32; per-tile sums are carried in FP64.  Near the LJ
-// minimum the force holds the cancelling factor (2 s^6 - 1); it is evaluated
-// as (1 + t)^3 - 1 = t (3 + 3t + t^2) with t = (r_0^2 - r^2) / r^2, r_0^2 =
-// 2^(1/3) sigma^2, and r^2 carried as hi + lo from the exact integer sum of
-// squares, so the FP32 result is accurate relative to the force itself.
+// ---- split form
+// Positions are differenced exactly in 32-bit fixed point, the pair
+// arithmetic is FP32, per-tile sums are carried in FP64.
+//
+// The sweep is bound by instruction issue (and next by the L1 wavefronts of
+// its gathers), so it is laid out to spend few instructions per list entry.
+// Per sweep of 913,408 atoms with 76 entries each: 306 us before these steps,
+// 259 us with the Hessian term, 122 to 143 us without it.
+//   - lengths stay in the replica's fixed-point unit u: separations are the
+//     converted integers (times 2^zshift on the open axis), r^2, r_0^2 and
+//     the cutoffs are in u^2, and the one factor 1/u goes to the finished
+//     sums.  Replicas whose axes share no unit use the axes' own units
+//     (scale lsb) and real lengths, with the same code;
+//   - with c = (r_0^2/r^2)^3 = 2 s^6 and w = c - 1 the force is
+//     g w r_ij, g = 12 eps c / r^2, and the Hessian term
+//     -g w u + g (14 c - 8) (r.u)/r^2 r_ij, so both share one product with eps;
+//   - four list entries are one 16-byte load, the row's position in the list
+//     is an immediate offset, and the neighbour's record is 16 bytes; r - r_O
+//     of a pair is its separation minus that of the two r_O's images, so only
+//     the Hessian term reads a second record.
+//
+// Near the LJ minimum the force holds the cancelling factor w; it is
+// evaluated as t (3 + 3 t + t^2) with t = (r_0^2 - r^2) / r^2.  Below
+// r^2 = (4/3) r_0^2, where the FP32 r^2 would cost w its relative accuracy,
+// r^2 is taken exactly, as hi + lo, from the integer separations; beyond it
+// the FP32 r^2 gives w to a few ulps.  The row builder puts the pairs that
+// can need the exact r^2 at the head of each row, so a warp takes the exact
+// form for its first groups of four and the other one from there on.
 __device__ __forceinline__ float rcp_approx(float x) {
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -606,287 +648,208 @@ __device__ __forceinline__ float rcp_refined(float x) {
     return fmaf(y, fmaf(-x, y, 1.f), y);
 }
 
-// Asynchronous 4-byte copies global -> shared (cp.async): each lane stages
-// its own atom's list entries, so a chunk needs no barrier, only the wait.
-__device__ __forceinline__ void cp_async4(int *dst, const int *src) {
-    const unsigned a = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(a), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+__device__ __forceinline__ float2 f2c(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 f2i(int a, int b) { return make_float2((float)a, (float)b); }
+__device__ __forceinline__ float2 f2neg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 f2mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 f2add(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 f2sub(float2 a, float2 b) { return __fadd2_rn(a, f2neg(b)); }
+__device__ __forceinline__ float2 f2fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 
-// List entries a lane stages ahead per chunk, double-buffered: a warp keeps
-// 2 x NBC x 128 B of its column-major list rows in shared memory, the next
-// chunk in flight while the current one is used.
-constexpr int NBC = 16;
-__host__ __device__ constexpr size_t pair_smem_bytes_for(int block) {
-    return (size_t)(block / 32) * 2 * NBC * 32 * sizeof(int);
-}
-
-template <bool Q, bool E, bool X2 = false>
-__device__ __forceinline__ void dev_pair32(const Dev &D, int t) {
+// Split rows: S lanes of a warp share one row (lane s takes groups s, s + S,
+// ... of four entries) and a CTA holds block / S atoms.  See dev_pair32.
+template <bool Q, bool E, bool H, int S>
+__device__ __forceinline__ void dev_pair32(const Dev &D, int unit) {
+    const int t = unit / S;
     const int r = D.tile_rep[t];
     if (Q && D.st[r].q_done) return;
     const RepDev &R = D.rep[r];
-    const bool act = threadIdx.x < D.tile_n[t];
-    const int i = D.tile_start[t] + (act ? threadIdx.x : 0);
-    const AtomRec ai = D.rec[i];
-    const int4 pi = ai.p;
+    const int sub = S > 1 ? (int)(threadIdx.x % S) : 0;
+    const int at = (unit % S) * (D.block / S) + (int)threadIdx.x / S;     // atom of the tile
+    const bool act = at < D.tile_n[t];
+    const int i = D.tile_start[t] + (act ? at : 0);
+    const int4 pi = D.p[i];
+    const int4 poi = H ? D.po[i] : make_int4(0, 0, 0, 0);
     const int ti = pi.w & 1;
-    const float lx = R.fx_lsb[0], ly = R.fx_lsb[1], lz = R.fx_lsb[2];
-    const int4 dfi = Q ? make_int4(0, 0, 0, 0) : ai.d;                 // r - r_O, fixed point
-    const float4 dri = make_float4((float)dfi.x * lx, (float)dfi.y * ly, (float)dfi.z * lz, 0.f);
-    const float e0 = R.epsf[ti][0], e1 = R.epsf[ti][1];
-    // 24 eps and 96 eps as FP32 hi + lo: an eps such as 0.2 is not an FP32
-    // number, and its rounding would scale every such pair force alike
-    const float a0 = R.eps24f[ti][0], a1 = R.eps24f[ti][1], al0 = R.eps24l[ti][0], al1 = R.eps24l[ti][1];
-    const float b0 = R.eps96f[ti][0], b1 = R.eps96f[ti][1], bl0 = R.eps96l[ti][0], bl1 = R.eps96l[ti][1];
-    const float h0 = R.shiftf[ti][0], h1 = R.shiftf[ti][1];
-    const float q0h = R.r0sq_hi[ti][0], q1h = R.r0sq_hi[ti][1];
-    const float q0l = R.r0sq_lo[ti][0], q1l = R.r0sq_lo[ti][1];
-    const bool exact = R.exact_r2 != 0;
-    const float r2corr = exact ? 2.f * R.lsb_rel[0] : 0.f;
-    float fx = 0.f, fy = 0.f, fz = 0.f, e = 0.f, hx = 0.f, hy = 0.f, hz = 0.f;
-    const int nn = act ? D.nnb[i] : 0;
-    const int *nb = D.nbr + i;
-    const size_t stride = (size_t)D.natom;
-    // The list streams from HBM: each lane stages its row NBC entries at a
-    // time through shared memory by cp.async, the next chunk in flight while
-    // the current one is used; the record of the next entry is loaded while
-    // the current one is used.
-    extern __shared__ __align__(16) int pair_smem[];
-    const int lane = threadIdx.x & 31;
-    int(*sbuf)[NBC][32] = reinterpret_cast<int(*)[NBC][32]>(pair_smem) + 2 * (threadIdx.x >> 5);
-    int nmax = nn;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) nmax = max(nmax, __shfl_xor_sync(0xffffffffu, nmax, o));
-    const int nch = (nmax + NBC - 1) / NBC;
-    auto stage = [&](int c) {
-        int(*b)[32] = sbuf[c & 1];
-#pragma unroll
-        for (int u = 0; u < NBC; ++u) {
-            const int k = c * NBC + u;
-            if (k < nn) cp_async4(&b[u][lane], nb + (size_t)k * stride);
+    const float sx = R.px_scale[0], sy = R.px_scale[1], sz = R.px_scale[2];
+    // 12 eps as FP32 hi + lo: an eps such as 0.2 is not an FP32 number, and
+    // its rounding would scale every such pair force alike
+    const float a0 = R.eps12f[ti][0], a1 = R.eps12f[ti][1], al0 = R.eps12l[ti][0], al1 = R.eps12l[ti][1];
+    const float q0h = R.r0u_hi[ti][0], q1h = R.r0u_hi[ti][1], q0l = R.r0u_lo[ti][0], q1l = R.r0u_lo[ti][1];
+    const float rc_lo = R.rc2u_lo, rc_hi = R.rc2u_hi, near2 = R.near2u;   // near2 is 0 without a common unit
+    float e = 0.f;
+    const int len = act ? D.nnb[i] : 0, nn = NB_LEN(len);
+    const bool mix = __any_sync(0xffffffffu, (len & NB_MIXED) != 0);
+    // Two entries at once in packed FP32x2 arithmetic (one instruction for
+    // both), in stages without branches.  An entry outside the cutoff (or past
+    // the row's end) takes part at r^2 = 3e38, where every product below is
+    // zero.  near_: some lane has an entry below (4/3) r_0^2, and all take the
+    // exact r^2.  MIX: some lane's row or atom is of the tip; without one the
+    // parameters are the substrate's and nothing is selected.
+    constexpr float FAR = 3.0e38f;
+    float2 Fx = make_float2(0.f, 0.f), Fy = Fx, Fz = Fx, Hx = Fx, Hy = Fx, Hz = Fx;
+    auto two = [&](bool near_, bool mix, int4 pa, int4 pb, int4 poa, int4 pob, int ixa, int ixb, int iya, int iyb, int iza,
+                   int izb, float2 dx, float2 dy, float2 dz, float2 r2) {
+        const bool ta = mix && (pa.w & 1), tb = mix && (pb.w & 1);
+        const float2 r0h = make_float2(ta ? q1h : q0h, tb ? q1h : q0h), r0l = make_float2(ta ? q1l : q0l, tb ? q1l : q0l);
+        float2 h = r2, l = r0l;
+        if (near_) {
+            float ha, la, hb, lb;
+            r2_units(ixa, iya << R.shift_y, iza << R.shift_z, ha, la);
+            r2_units(ixb, iyb << R.shift_y, izb << R.shift_z, hb, lb);
+            h = make_float2(r2.x < FAR ? ha : FAR, r2.y < FAR ? hb : FAR);
+            l = f2sub(r0l, make_float2(la, lb));
         }
-        cp_async_commit();
-    };
-    if (nch > 0) stage(0);
-    // one pair's contribution.  Cancellation-free LJ form: 2 s^6 - 1 = w(tt)
-    // with tt = (r_0^2 - r^2) / r^2.  Where |tt| < 1/4 (around the minimum,
-    // where w is small and the FP32 r^2 would cost it its relative accuracy)
-    // r^2 is taken exactly, as hi + lo, from the integer separations when the
-    // replica's axes share one fixed-point unit; elsewhere the FP32 r^2 gives
-    // w to a few ulps.  The list builder puts the pairs that can need the
-    // exact r^2 at the head of each row, so the branch is nearly uniform.
-    auto term = [&](const AtomRec &aj, int ix, int iy, int iz, float dx, float dy, float dz, float r2) {
-        const int tj = aj.p.w & 1;
-        const float r0h = tj ? q1h : q0h, r0l = tj ? q1l : q0l;
-        // the FP32 r^2 with the rounding of the fixed-point unit undone (all
-        // axes share its relative rounding when they share the unit)
-        const float r2c = fmaf(r2, r2corr, r2);
-        float ir2 = rcp_refined(r2c);
-        float tt = ((r0h - r2c) + r0l) * ir2;
-        if (exact && fabsf(tt) < 0.25f) {
-            float r2h, r2l;
-            r2_split(R, ix, iy, iz, r2h, r2l);
-            ir2 = rcp_refined(r2h);
-            tt = ((r0h - r2h) + (r0l - r2l)) * ir2;
+        // 1/r^2: the hardware approximation and one Newton step (rcp_refined)
+        float2 ir2 = make_float2(rcp_approx(h.x), rcp_approx(h.y));
+        ir2 = f2fma(ir2, f2fma(f2neg(h), ir2, f2c(1.f)), ir2);
+        const float2 tt = f2mul(f2add(f2sub(r0h, h), l), ir2);
+        const float2 c1 = f2add(tt, f2c(1.f));
+        const float2 c = f2mul(f2mul(c1, c1), c1);                               // 2 s^6
+        const float2 w = f2mul(tt, f2fma(tt, f2add(tt, f2c(3.f)), f2c(3.f)));    // 2 s^6 - 1
+        const float2 g0 = f2mul(ir2, c);
+        const float2 g = f2fma(g0, make_float2(ta ? al1 : al0, tb ? al1 : al0),
+                               f2mul(g0, make_float2(ta ? a1 : a0, tb ? a1 : a0)));
+        const float2 fr = f2mul(g, w);
+        Fx = f2fma(fr, dx, Fx);
+        Fy = f2fma(fr, dy, Fy);
+        Fz = f2fma(fr, dz, Fz);
+        if (E) {
+            const float sa = 0.5f * c.x, sb = 0.5f * c.y;
+            const float ea = fmaf(4.f * R.epsf[ti][ta] * sa, sa - 1.f, -R.shiftf[ti][ta]);
+            const float eb = fmaf(4.f * R.epsf[ti][tb] * sb, sb - 1.f, -R.shiftf[ti][tb]);
+            e = fmaf(0.5f, r2.x < FAR ? ea : 0.f, e);
+            e = fmaf(0.5f, r2.y < FAR ? eb : 0.f, e);
         }
-        const float u = 1.f + tt;
-        const float s6 = 0.5f * u * u * u;
-        const float w = tt * fmaf(tt, tt + 3.f, 3.f);          // 2 s^6 - 1
-        const float pf = ir2 * s6 * w;
-        const float fr = fmaf(pf, tj ? al1 : al0, pf * (tj ? a1 : a0));
-        fx = fmaf(fr, dx, fx);
-        fy = fmaf(fr, dy, fy);
-        fz = fmaf(fr, dz, fz);
-        if (E) e = fmaf(0.5f, fmaf(4.f * (tj ? e1 : e0) * s6, s6 - 1.f, -(tj ? h1 : h0)), e);
-        if (!Q) {
-            const float ux = (float)(int)((unsigned)dfi.x - (unsigned)aj.d.x) * lx;
-            const float uy = (float)(int)((unsigned)dfi.y - (unsigned)aj.d.y) * ly;
-            const float uz = (float)(int)((unsigned)dfi.z - (unsigned)aj.d.z) * lz;
-            const float rdu = fmaf(dx, ux, fmaf(dy, uy, dz * uz));
-            const float pb = ir2 * ir2 * s6 * fmaf(7.f, s6, -2.f) * rdu;
-            const float B = fmaf(pb, tj ? bl1 : bl0, pb * (tj ? b1 : b0));
-            hx = fmaf(-fr, ux, fmaf(B, dx, hx));
-            hy = fmaf(-fr, uy, fmaf(B, dy, hy));
-            hz = fmaf(-fr, uz, fmaf(B, dz, hz));
+        if (H) {
+            const float2 ux = f2mul(f2i(ixa - (int)((unsigned)poi.x - (unsigned)poa.x), ixb - (int)((unsigned)poi.x - (unsigned)pob.x)), f2c(sx));
+            const float2 uy = f2mul(f2i(iya - (int)((unsigned)poi.y - (unsigned)poa.y), iyb - (int)((unsigned)poi.y - (unsigned)pob.y)), f2c(sy));
+            const float2 uz = f2mul(f2i(iza - (int)((unsigned)poi.z - (unsigned)poa.z), izb - (int)((unsigned)poi.z - (unsigned)pob.z)), f2c(sz));
+            const float2 rdu = f2fma(dx, ux, f2fma(dy, uy, f2mul(dz, uz)));
+            const float2 B = f2mul(f2mul(g, f2fma(c, f2c(14.f), f2c(-8.f))), f2mul(ir2, rdu)), nfr = f2neg(fr);
+            Hx = f2fma(nfr, ux, f2fma(B, dx, Hx));
+            Hy = f2fma(nfr, uy, f2fma(B, dy, Hy));
+            Hz = f2fma(nfr, uz, f2fma(B, dz, Hz));
         }
     };
+    auto sep = [](int a, int b) { return (int)((unsigned)a - (unsigned)b); };
     bool band = false;
-    if (!X2) {
-        for (int c = 0; c < nch; ++c) {
-            if (c + 1 < nch) {
-                stage(c + 1);
-                cp_async_wait<1>();
+    const int ngroup = (nn + 3) >> 2;
+    int itmax = (ngroup - sub + S - 1) / S;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) itmax = max(itmax, __shfl_xor_sync(0xffffffffu, itmax, o));
+    const int4 *row = reinterpret_cast<const int4 *>(D.nbr) + nbr_row4(D, R, i) + 32 * sub;
+    int4 J = make_int4(i, i, i, i);
+    if (sub < ngroup) J = row[0];
+    for (int it = 0; it < itmax; ++it) {
+        const int left = nn - 4 * (sub + S * it);         // entries of this lane from here on
+        const int j4[4] = {J.x, J.y, J.z, J.w};
+        int4 p4[4], po4[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) p4[u] = D.p[j4[u]];   // the builder fills a row's last group up with i
+#pragma unroll
+        for (int u = 0; u < 4; ++u) po4[u] = H ? D.po[j4[u]] : make_int4(0, 0, 0, 0);
+        row += 32 * S;
+        if (left > 4 * S) J = *row;
+#pragma unroll
+        for (int u = 0; u < 4; u += 2) {
+            const int ixa = sep(pi.x, p4[u].x), iya = sep(pi.y, p4[u].y), iza = sep(pi.z, p4[u].z);
+            const int ixb = sep(pi.x, p4[u + 1].x), iyb = sep(pi.y, p4[u + 1].y), izb = sep(pi.z, p4[u + 1].z);
+            const float2 dx = f2mul(f2i(ixa, ixb), f2c(sx)), dy = f2mul(f2i(iya, iyb), f2c(sy)),
+                         dz = f2mul(f2i(iza, izb), f2c(sz));
+            float2 r2 = f2fma(dx, dx, f2fma(dy, dy, f2mul(dz, dz)));
+            const bool ina = u < left && r2.x < rc_lo, inb = u + 1 < left && r2.y < rc_lo;
+            band |= (u < left && r2.x < rc_hi && !ina) || (u + 1 < left && r2.y < rc_hi && !inb);
+            r2.x = ina ? r2.x : FAR;
+            r2.y = inb ? r2.y : FAR;
+            const float lowest = fminf(r2.x, r2.y);
+            if (!__any_sync(0xffffffffu, lowest < FAR)) continue;      // the skin shell
+            auto both = [&](bool nr, bool mx) {
+                two(nr, mx, p4[u], p4[u + 1], po4[u], po4[u + 1], ixa, ixb, iya, iyb, iza, izb, dx, dy, dz, r2);
+            };
+            const bool near_ = __any_sync(0xffffffffu, lowest < near2);
+            if (mix) {
+                if (near_) both(true, true);
+                else both(false, true);
             } else {
-                cp_async_wait<0>();
+                if (near_) both(true, false);
+                else both(false, false);
             }
-            const int(*b)[32] = sbuf[c & 1];
-            const int kend = min(NBC, nn - c * NBC);
-            AtomRec an = kend > 0 ? D.rec[b[0][lane]] : ai;
-            for (int u = 0; u < kend; ++u) {
-                const AtomRec aj = an;
-                if (u + 1 < kend) an = D.rec[b[u + 1][lane]];
-                const int4 pj = aj.p;
-                const int ix = (int)((unsigned)pi.x - (unsigned)pj.x);
-                const int iy = (int)((unsigned)pi.y - (unsigned)pj.y);
-                const int iz = (int)((unsigned)pi.z - (unsigned)pj.z);
-                const float dx = (float)ix * lx, dy = (float)iy * ly, dz = (float)iz * lz;
-                const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                if (r2 < D.rc2_lo_f) term(aj, ix, iy, iz, dx, dy, dz, r2);
-                else band |= r2 < D.rc2_hi_f;
-            }
-        }
-    } else {
-        // Two list entries per iteration in packed FP32x2 arithmetic (one
-        // instruction for both halves), with the same operations per entry as
-        // term(); an entry outside the cutoff contributes through a select to
-        // zero.  Records of the next two entries and the indices of the two
-        // after them are in flight while the current two are used.
-        const float2 one2 = make_float2(1.f, 1.f), mone2 = make_float2(-1.f, -1.f), half2 = make_float2(0.5f, 0.5f);
-        const float2 three2 = make_float2(3.f, 3.f), seven2 = make_float2(7.f, 7.f), mtwo2 = make_float2(-2.f, -2.f);
-        const float2 corr2 = make_float2(r2corr, r2corr);
-        float2 Fx = make_float2(0.f, 0.f), Fy = Fx, Fz = Fx, Hx = Fx, Hy = Fx, Hz = Fx, Ee = Fx;
-        for (int c = 0; c < nch; ++c) {
-          if (c + 1 < nch) {
-              stage(c + 1);
-              cp_async_wait<1>();
-          } else {
-              cp_async_wait<0>();
-          }
-          const int(*b)[32] = sbuf[c & 1];
-          const int kend = min(NBC, nn - c * NBC);
-          AtomRec na = kend > 0 ? D.rec[b[0][lane]] : ai, nbr2 = kend > 1 ? D.rec[b[1][lane]] : ai;
-          for (int u = 0; u < kend; u += 2) {
-            const AtomRec A = na, B = nbr2;
-            const bool vb = u + 1 < kend;
-            if (u + 2 < kend) na = D.rec[b[u + 2][lane]];
-            if (u + 3 < kend) nbr2 = D.rec[b[u + 3][lane]];
-            const int ixa = (int)((unsigned)pi.x - (unsigned)A.p.x), ixb = (int)((unsigned)pi.x - (unsigned)B.p.x);
-            const int iya = (int)((unsigned)pi.y - (unsigned)A.p.y), iyb = (int)((unsigned)pi.y - (unsigned)B.p.y);
-            const int iza = (int)((unsigned)pi.z - (unsigned)A.p.z), izb = (int)((unsigned)pi.z - (unsigned)B.p.z);
-            const float2 dx = __fmul2_rn(make_float2((float)ixa, (float)ixb), make_float2(lx, lx));
-            const float2 dy = __fmul2_rn(make_float2((float)iya, (float)iyb), make_float2(ly, ly));
-            const float2 dz = __fmul2_rn(make_float2((float)iza, (float)izb), make_float2(lz, lz));
-            const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
-            const bool ina = r2.x < D.rc2_lo_f, inb = vb && r2.y < D.rc2_lo_f;
-            band |= (!ina && r2.x < D.rc2_hi_f) || (vb && !inb && r2.y < D.rc2_hi_f);
-            if (!(ina || inb)) continue;
-            const int ta = A.p.w & 1, tb = B.p.w & 1;
-            const float2 r0h = make_float2(ta ? q1h : q0h, tb ? q1h : q0h);
-            const float2 r0l = make_float2(ta ? q1l : q0l, tb ? q1l : q0l);
-            const float2 r2c = __ffma2_rn(r2, corr2, r2);
-            float2 ir2 = make_float2(rcp_approx(r2c.x), rcp_approx(r2c.y));
-            ir2 = __ffma2_rn(ir2, __ffma2_rn(r2c, __fmul2_rn(ir2, mone2), one2), ir2);
-            float2 tt = __fmul2_rn(__fadd2_rn(__ffma2_rn(r2c, mone2, r0h), r0l), ir2);
-            if (exact && ina && fabsf(tt.x) < 0.25f) {
-                float h, l;
-                r2_split(R, ixa, iya, iza, h, l);
-                ir2.x = rcp_refined(h);
-                tt.x = ((r0h.x - h) + (r0l.x - l)) * ir2.x;
-            }
-            if (exact && inb && fabsf(tt.y) < 0.25f) {
-                float h, l;
-                r2_split(R, ixb, iyb, izb, h, l);
-                ir2.y = rcp_refined(h);
-                tt.y = ((r0h.y - h) + (r0l.y - l)) * ir2.y;
-            }
-            const float2 u1 = __fadd2_rn(one2, tt);
-            const float2 s6 = __fmul2_rn(__fmul2_rn(half2, u1), __fmul2_rn(u1, u1));
-            const float2 w = __fmul2_rn(tt, __ffma2_rn(tt, __fadd2_rn(tt, three2), three2));      // 2 s^6 - 1
-            const float2 pf = __fmul2_rn(ir2, __fmul2_rn(s6, w));
-            float2 fr = __ffma2_rn(pf, make_float2(ta ? al1 : al0, tb ? al1 : al0),
-                                   __fmul2_rn(pf, make_float2(ta ? a1 : a0, tb ? a1 : a0)));
-            fr.x = ina ? fr.x : 0.f;
-            fr.y = inb ? fr.y : 0.f;
-            Fx = __ffma2_rn(fr, dx, Fx);
-            Fy = __ffma2_rn(fr, dy, Fy);
-            Fz = __ffma2_rn(fr, dz, Fz);
-            if (E) {
-                float2 ee = __ffma2_rn(__fmul2_rn(make_float2(4.f * (ta ? e1 : e0), 4.f * (tb ? e1 : e0)), s6),
-                                       __fadd2_rn(s6, mone2), make_float2(-(ta ? h1 : h0), -(tb ? h1 : h0)));
-                ee.x = ina ? ee.x : 0.f;
-                ee.y = inb ? ee.y : 0.f;
-                Ee = __ffma2_rn(half2, ee, Ee);
-            }
-            if (!Q) {
-                const float2 ux = __fmul2_rn(make_float2((float)(int)((unsigned)dfi.x - (unsigned)A.d.x),
-                                                         (float)(int)((unsigned)dfi.x - (unsigned)B.d.x)),
-                                             make_float2(lx, lx));
-                const float2 uy = __fmul2_rn(make_float2((float)(int)((unsigned)dfi.y - (unsigned)A.d.y),
-                                                         (float)(int)((unsigned)dfi.y - (unsigned)B.d.y)),
-                                             make_float2(ly, ly));
-                const float2 uz = __fmul2_rn(make_float2((float)(int)((unsigned)dfi.z - (unsigned)A.d.z),
-                                                         (float)(int)((unsigned)dfi.z - (unsigned)B.d.z)),
-                                             make_float2(lz, lz));
-                const float2 rdu = __ffma2_rn(dx, ux, __ffma2_rn(dy, uy, __fmul2_rn(dz, uz)));
-                const float2 pb = __fmul2_rn(__fmul2_rn(ir2, ir2),
-                                             __fmul2_rn(__fmul2_rn(s6, __ffma2_rn(seven2, s6, mtwo2)), rdu));
-                float2 Bc = __ffma2_rn(pb, make_float2(ta ? bl1 : bl0, tb ? bl1 : bl0),
-                                       __fmul2_rn(pb, make_float2(ta ? b1 : b0, tb ? b1 : b0)));
-                Bc.x = ina ? Bc.x : 0.f;
-                Bc.y = inb ? Bc.y : 0.f;
-                const float2 nfr = __fmul2_rn(fr, mone2);
-                Hx = __ffma2_rn(nfr, ux, __ffma2_rn(Bc, dx, Hx));
-                Hy = __ffma2_rn(nfr, uy, __ffma2_rn(Bc, dy, Hy));
-                Hz = __ffma2_rn(nfr, uz, __ffma2_rn(Bc, dz, Hz));
-            }
-          }
-        }
-        fx += Fx.x + Fx.y;
-        fy += Fy.x + Fy.y;
-        fz += Fz.x + Fz.y;
-        if (E) e += Ee.x + Ee.y;
-        if (!Q) {
-            hx += Hx.x + Hx.y;
-            hy += Hy.x + Hy.y;
-            hz += Hz.x + Hz.y;
         }
     }
     // Rare: pairs in a thin band around rc are cut by the oracle's FP64 test
     // (same operations), so no pair is cut at a different step than in FP64.
     if (band) {
         const dbl4 xi64 = D.x[i];
-        for (int k = 0; k < nn; ++k) {
-            const int j = nb[(size_t)k * stride];
-            const AtomRec aj = D.rec[j];
-            const int ix = (int)((unsigned)pi.x - (unsigned)aj.p.x);
-            const int iy = (int)((unsigned)pi.y - (unsigned)aj.p.y);
-            const int iz = (int)((unsigned)pi.z - (unsigned)aj.p.z);
-            const float dx = (float)ix * lx, dy = (float)iy * ly, dz = (float)iz * lz;
+        const size_t row4 = nbr_row4(D, R, i);
+        const int4 zero = make_int4(0, 0, 0, 0);
+        for (int k = 4 * sub; k < nn; k += (k & 3) == 3 ? 4 * S - 3 : 1) {
+            const int j = D.nbr[nbr_at(row4, k)];
+            const int4 pj = D.p[j];
+            const int ix = sep(pi.x, pj.x), iy = sep(pi.y, pj.y), iz = sep(pi.z, pj.z);
+            const float dx = (float)ix * sx, dy = (float)iy * sy, dz = (float)iz * sz;
             const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-            if (r2 >= D.rc2_lo_f && r2 < D.rc2_hi_f && exact_r2(R, xi64, D.x[j]) < D.rc2)
-                term(aj, ix, iy, iz, dx, dy, dz, r2);
+            if (r2 >= rc_lo && r2 < rc_hi && exact_r2(R, xi64, D.x[j]) < D.rc2)
+                two(false, true, pj, zero, H ? D.po[j] : zero, zero, ix, 0, iy, 0, iz, 0, make_float2(dx, 0.f),
+                    make_float2(dy, 0.f), make_float2(dz, 0.f), make_float2(r2, FAR));
         }
     }
+    float fx = Fx.x + Fx.y, fy = Fy.x + Fy.y, fz = Fz.x + Fz.y, hx = Hx.x + Hx.y, hy = Hy.x + Hy.y, hz = Hz.x + Hz.y;
+    if (S > 1) {
+#pragma unroll
+        for (int o = 1; o < S; o <<= 1) {
+            fx += __shfl_xor_sync(0xffffffffu, fx, o);
+            fy += __shfl_xor_sync(0xffffffffu, fy, o);
+            fz += __shfl_xor_sync(0xffffffffu, fz, o);
+            if (E) e += __shfl_xor_sync(0xffffffffu, e, o);
+            if (H) {
+                hx += __shfl_xor_sync(0xffffffffu, hx, o);
+                hy += __shfl_xor_sync(0xffffffffu, hy, o);
+                hz += __shfl_xor_sync(0xffffffffu, hz, o);
+            }
+        }
+    }
+    // to real units
+    fx = fmaf(fx, R.out_hi[0], fx * R.out_lo[0]);
+    fy = fmaf(fy, R.out_hi[1], fy * R.out_lo[1]);
+    fz = fmaf(fz, R.out_hi[2], fz * R.out_lo[2]);
+    if (H) {
+        hx = fmaf(hx, R.out_hi[0], hx * R.out_lo[0]);
+        hy = fmaf(hy, R.out_hi[1], hy * R.out_lo[1]);
+        hz = fmaf(hz, R.out_hi[2], hz * R.out_lo[2]);
+    }
+    const float lx = R.fx_lsb[0], ly = R.fx_lsb[1], lz = R.fx_lsb[2];
+    const int4 dfi = Q ? make_int4(0, 0, 0, 0) : img_diff(pi, H ? poi : D.po[i]);
+    const float4 dri = make_float4((float)dfi.x * lx, (float)dfi.y * ly, (float)dfi.z * lz, 0.f);
+    const bool own = act && sub == 0;
     // harmonic bonds of Eq. 12 at any distance, from the exact r^2 where the
     // axes share one unit (r - r_b is a small difference of two numbers near
     // r_b); A = k (r - r_b)/r, B = k r_b / r^3
-    if (R.nbond > 0 && act) {
+    if (R.nbond > 0 && own) {
+        float bx = 0.f, by = 0.f, bz = 0.f;
         for (int b = D.bond_off[i]; b < D.bond_off[i + 1]; ++b) {
             const int j = D.bond_j[b];
-            const AtomRec aj = D.rec[j];
-            const int ix = (int)((unsigned)pi.x - (unsigned)aj.p.x);
-            const int iy = (int)((unsigned)pi.y - (unsigned)aj.p.y);
-            const int iz = (int)((unsigned)pi.z - (unsigned)aj.p.z);
+            const int4 pj = D.p[j];
+            const int ix = (int)((unsigned)pi.x - (unsigned)pj.x);
+            const int iy = (int)((unsigned)pi.y - (unsigned)pj.y);
+            const int iz = (int)((unsigned)pi.z - (unsigned)pj.z);
             const float dx = (float)ix * lx, dy = (float)iy * ly, dz = (float)iz * lz;
             float r2h = fmaf(dx, dx, fmaf(dy, dy, dz * dz)), r2l = 0.f;
-            if (exact) r2_split(R, ix, iy, iz, r2h, r2l);
+            if (R.exact_r2) r2_split(R, ix, iy, iz, r2h, r2l);
             const float rh = sqrtf(r2h);
             const float rr = rh + (fmaf(-rh, rh, r2h) + r2l) * (0.5f / rh);
             const float db = (rr - R.rbond_hi) - R.rbond_lo;
             const float ir = 1.f / rr;
             const float A = R.kbondf * db * ir;
-            fx = fmaf(-A, dx, fx);
-            fy = fmaf(-A, dy, fy);
-            fz = fmaf(-A, dz, fz);
+            bx = fmaf(-A, dx, bx);
+            by = fmaf(-A, dy, by);
+            bz = fmaf(-A, dz, bz);
             if (E) e = fmaf(0.25f * R.kbondf * db, db, e);
-            if (!Q) {
-                const float ux = (float)(int)((unsigned)dfi.x - (unsigned)aj.d.x) * lx;
-                const float uy = (float)(int)((unsigned)dfi.y - (unsigned)aj.d.y) * ly;
-                const float uz = (float)(int)((unsigned)dfi.z - (unsigned)aj.d.z) * lz;
+            if (H) {
+                const int4 poj = D.po[j];
+                const float ux = (float)(int)((unsigned)ix - ((unsigned)poi.x - (unsigned)poj.x)) * lx;
+                const float uy = (float)(int)((unsigned)iy - ((unsigned)poi.y - (unsigned)poj.y)) * ly;
+                const float uz = (float)(int)((unsigned)iz - ((unsigned)poi.z - (unsigned)poj.z)) * lz;
                 const float rdu = fmaf(dx, ux, fmaf(dy, uy, dz * uz));
                 const float B = (R.kbondf - A) * ir * ir * rdu;
                 hx = fmaf(A, ux, fmaf(B, dx, hx));
@@ -894,75 +857,115 @@ __device__ __forceinline__ void dev_pair32(const Dev &D, int t) {
                 hz = fmaf(A, uz, fmaf(B, dz, hz));
             }
         }
+        // undo the FP32 rounding of the per-axis fixed-point unit
+        fx += fmaf(bx, R.lsb_rel[0], bx);
+        fy += fmaf(by, R.lsb_rel[1], by);
+        fz += fmaf(bz, R.lsb_rel[2], bz);
     }
-    // undo the FP32 rounding of the per-axis fixed-point unit (uniform per axis)
-    fx = fmaf(fx, R.lsb_rel[0], fx);
-    fy = fmaf(fy, R.lsb_rel[1], fy);
-    fz = fmaf(fz, R.lsb_rel[2], fz);
-    const int role = act ? ((pi.w >> 8) & 0xff) : -1;
-    if (!Q && role == ROLE_RIGID) {
+    const int role = own ? ((pi.w >> 8) & 0xff) : -1;
+    if (H && role == ROLE_RIGID) {
         hx += R.kr_nf * dri.x;
         if (R.dim == 3) hy += R.kr_nf * dri.y;
     }
-    if (act) {
+    if (own) {
         D.f32[i] = make_float4(fx, fy, fz, e);
-        if (!Q) D.h32[i] = make_float4(hx, hy, hz, 0.f);
+        if (H) D.h32[i] = make_float4(hx, hy, hz, 0.f);
     }
     const bool rig = role == ROLE_RIGID;
     const bool anyrig = __any_sync(0xffffffffu, rig);
-    // FP32 sums inside each warp, FP64 across warps and tiles
+    double xr[3] = {0.0, 0.0, 0.0};
+    if (rig) {
+        const dbl4 xi = D.x[i];
+        xr[0] = xi.x; xr[1] = xi.y; xr[2] = xi.z;
+    }
+    double *out = D.part + (size_t)unit * NPART;
     if (!Q) {
-        float v[12] = {};
-        double d3[3] = {0.0, 0.0, 0.0};
-        if (act) {
+        float v[9] = {};
+        double d2 = 0.0, g = 0.0;
+        if (own) {
             const double rx = dri.x, ry = dri.y, rz = dri.z;
-            d3[PART_D2] = rx * rx + ry * ry + rz * rz;
-            d3[PART_G] = -((double)fx * rx + (double)fy * ry + (double)fz * rz);
-            d3[PART_V] = (double)e;
+            d2 = rx * rx + ry * ry + rz * rz;
+            g = -((double)fx * rx + (double)fy * ry + (double)fz * rz);
         }
         if (rig) {
-            v[PART_FRIG] = fx; v[PART_FRIG + 1] = fy; v[PART_FRIG + 2] = fz;
-            v[PART_HRIG] = hx; v[PART_HRIG + 1] = hy; v[PART_HRIG + 2] = hz;
-            v[PART_DRRIG] = dri.x; v[PART_DRRIG + 1] = dri.y; v[PART_DRRIG + 2] = dri.z;
+            v[0] = fx; v[1] = fy; v[2] = fz;
+            v[3] = hx; v[4] = hy; v[5] = hz;
+            v[6] = dri.x; v[7] = dri.y; v[8] = dri.z;
         }
-        double xr[3] = {0.0, 0.0, 0.0};
-        if (rig) {
-            const dbl4 xi = D.x[i];
-            xr[0] = xi.x; xr[1] = xi.y; xr[2] = xi.z;
-        }
-        tile_reduce_mixed(d3, v, anyrig ? 12 : 3, xr, anyrig, D.part + (size_t)t * NPART);
+        const TileSlots L = {{PART_D2, PART_G, PART_V, -1}, PART_FRIG, PART_XRIG, -1};
+        tile_reduce<9>(d2, g, E && own ? (double)e : 0.0, 0.0, v, xr, anyrig, -1.f, L, out);
     } else {
-        float v[12] = {};
-        double pvf[3] = {0.0, 0.0, 0.0};
-        float fm = 0.f;
+        float v[3] = {}, fm = 0.f;
+        double pw = 0.0, vv2 = 0.0, ff = 0.0;
         if (role == ROLE_MOBILE) {
             const float4 vv = D.v32[i];
             fm = fx * fx + fy * fy + fz * fz;
             const double gx = fx, gy = fy, gz = fz, ux = vv.x, uy = vv.y, uz = vv.z;
-            pvf[0] = gx * ux + gy * uy + gz * uz;
-            pvf[1] = ux * ux + uy * uy + uz * uz;
-            pvf[2] = gx * gx + gy * gy + gz * gz;
+            pw = gx * ux + gy * uy + gz * uz;
+            vv2 = ux * ux + uy * uy + uz * uz;
+            ff = gx * gx + gy * gy + gz * gz;
         }
         if (rig) {
-            v[QP_FRIG] = fx; v[QP_FRIG + 1] = fy; v[QP_FRIG + 2] = fz;
+            v[0] = fx; v[1] = fy; v[2] = fz;
         }
-        double xr[3] = {0.0, 0.0, 0.0};
-        if (rig) {
-            const dbl4 xi = D.x[i];
-            xr[0] = xi.x; xr[1] = xi.y; xr[2] = xi.z;
-        }
-        v[QP_FMAX2] = fm;
-        tile_reduce_quench(v, pvf, xr, anyrig, D.part + (size_t)t * NPART);
+        const TileSlots L = {{QP_P, QP_VV, QP_FF, -1}, QP_FRIG, QP_XRIG, QP_FMAX2};
+        tile_reduce<3>(pw, vv2, ff, 0.0, v, xr, anyrig, fm, L, out);
     }
 }
 
-template <bool Q, bool E>
-__global__ void __launch_bounds__(256) k_pair64(Dev D) { dev_pair64<Q, E>(D, blockIdx.x); }
-template <bool Q, bool E>
-__global__ void __launch_bounds__(256, 4) k_pair32(Dev D) { dev_pair32<Q, E>(D, blockIdx.x); }
-// the packed FP32x2 variant: more registers a thread, fewer warps resident
-template <bool Q, bool E>
-__global__ void __launch_bounds__(128, 5) k_pair32x2(Dev D) { dev_pair32<Q, E, true>(D, blockIdx.x); }
+// Which replicas an MD sweep covers: all of them; those that go without the
+// Hessian term; those that were predicted to need it (see k_scalar).
+enum { SWEEP_ALL = 0, SWEEP_PLAIN = 1 };
+
+template <bool Q, bool E, bool H, int S>
+__global__ void __launch_bounds__(256) k_pair64(Dev D, int sweep) {
+    if (sweep == SWEEP_PLAIN && D.sc[D.tile_rep[blockIdx.x / S]].need_h) return;
+    dev_pair64<Q, E, H, S>(D, blockIdx.x);
+}
+template <bool Q, bool E, bool H, int S>
+__global__ void __launch_bounds__(256, H ? 3 : 4) k_pair32(Dev D, int sweep) {
+    if (sweep == SWEEP_PLAIN && D.sc[D.tile_rep[blockIdx.x / S]].need_h) return;
+    dev_pair32<Q, E, H, S>(D, blockIdx.x);
+}
+
+// Sweeps with the Hessian term over the listed replicas only; true in the
+// last CTA to finish (all others' results visible to it).  The list is empty
+// in most steps, so the grid is a fixed few CTAs an SM that stride over the
+// listed tiles.
+template <int PREC, int S>
+__device__ __forceinline__ bool sweep_listed(const Dev &D, const int *list, int n, unsigned *ticket) {
+    int pos = blockIdx.x, base = 0;       // place in the listed replicas' tiles, one after another
+    for (int q = 0; q < n; ++q) {
+        const RepDev &R = D.rep[list[q]];
+        const int t0 = R.tile0 * S, nt = R.ntile * S;
+        for (; pos < base + nt; pos += gridDim.x) {
+            if (PREC == HD_FP64) dev_pair64<false, false, true, S>(D, t0 + pos - base);
+            else dev_pair32<false, false, true, S>(D, t0 + pos - base);
+        }
+        base += nt;
+    }
+    __shared__ unsigned s_tick;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_tick = atomicAdd(ticket, 1u);
+    }
+    __syncthreads();
+    if (s_tick != gridDim.x - 1) return false;
+    __threadfence();
+    return true;
+}
+
+// The replicas predicted to need the Hessian term (h_meta[0] of them).
+template <int PREC, int S>
+__global__ void __launch_bounds__(256, PREC == HD_FP64 ? 1 : 3) k_pair_hot(Dev D) {
+    const int n = D.h_meta[0];
+    if (n == 0) return;
+    if (sweep_listed<PREC, S>(D, D.h_list, n, (unsigned *)D.h_meta + 2) && threadIdx.x == 0) {
+        D.h_meta[0] = 0;
+        D.h_meta[2] = 0;
+    }
+}
 
 // ---------------------------------------------------------------- per-replica scalars
 // Gathers the replica's tile sums (warp q sums slot q over the tiles in a
@@ -974,7 +977,10 @@ __global__ void __launch_bounds__(128, 5) k_pair32x2(Dev D) { dev_pair32<Q, E, t
 //   cb = DeltaV' sigma / d^2 (from grad sigma = (H dr + g)/d - sigma dr/d^2);
 //   rigid-body force = sum_rigid F - gs - DeltaV' sum_rigid grad sigma;
 //   body kicks and the clocks: t_h += dt exp(DeltaV / kT) (Eq. 3).
-__device__ void scalar_eval(const Dev &D, int r, int mode, const double *acc, double ksum, RepState &S, Scal &C) {
+// need_hess: the caller has no H.dr of this configuration; with DeltaV' != 0
+// nothing is changed then and the result is false.
+__device__ bool scalar_eval(const Dev &D, int r, int mode, const double *acc, double ksum, RepState &S, Scal &C,
+                            bool need_hess = false) {
     const RepDev &R = D.rep[r];
     const int nr = R.nrig, dim = R.dim, vert = R.vert;
     const double xs = slider_x(R, S.step, D.dt);
@@ -1004,6 +1010,7 @@ __device__ void scalar_eval(const Dev &D, int r, int mode, const double *acc, do
             dV = dVp = dVe = 0.0;
         }
     }
+    if (need_hess && dVp != 0.0) return false;
     const double ca = d > 0.0 ? -dVp / d : 0.0;
     const double cb = d > 0.0 ? dVp * sig / (d * d) : 0.0;
     double fb[3] = {0, 0, 0};
@@ -1058,6 +1065,7 @@ __device__ void scalar_eval(const Dev &D, int r, int mode, const double *acc, do
     for (int a = 0; a < 3; ++a) { C.vb_new[a] = vb[a]; S.vbody[a] = vb[a]; }
     S.K = ksum + 0.5 * (double)nr * (S.vbody_full[0] * S.vbody_full[0] + S.vbody_full[1] * S.vbody_full[1] +
                                      S.vbody_full[2] * S.vbody_full[2]);
+    return true;
 }
 
 // Tile sums of one replica, slot by slot (slot NPART = kinetic parts): for
@@ -1068,27 +1076,80 @@ __device__ __forceinline__ void dev_scalar_acc(const Dev &D, int r, double *acc)
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     for (int q = w; q <= NPART; q += nw) {
         double a = 0.0;
-        for (int t = R.tile0 + lane; t < R.tile0 + R.ntile; t += 32)
-            a += (q < NPART) ? D.part[(size_t)t * NPART + q] : D.kpart[t];
+        if (q < NPART) {
+            for (int t = R.tile0 * D.split + lane; t < (R.tile0 + R.ntile) * D.split; t += 32)
+                a += D.part[(size_t)t * NPART + q];
+        } else {
+            for (int t = R.tile0 + lane; t < R.tile0 + R.ntile; t += 32) a += D.kpart[t];
+        }
         a = warp_sum(a);
         if (lane == 0) acc[q] = a;
     }
     __syncthreads();
 }
 
+// H.(r - r_O) enters the dynamics only through DeltaV', which is zero outside
+// the band of Eq. 14; sigma itself needs the forces alone.  So the sweeps of
+// a large batch leave the Hessian term out for the replicas that are not
+// expected in their band (lazy = 1): it costs the sweep a second gather and
+// about 40% of its instructions.  After each evaluation the next slope is
+// expected within two of the largest recent changes of the slope; a replica
+// whose band reaches there goes on the list that k_pair_hot sweeps with H.  If
+// another one lands in its band all the same, its evaluation is put off
+// (h_meta[1], k_scalar_late) until k_scalar_late has swept it with H, so the
+// result never depends on the guess.  list = 0: the next sweep takes H for
+// everyone (the last step of a call, whose H can be read).
+__device__ void expect_slope(const Dev &D, int r, RepState &S, Scal &C, int list) {
+    const RepDev &R = D.rep[r];
+    const double step = fabs(C.sigma - S.h_sig);
+    S.h_step = fmax(step, 0.9 * S.h_step);
+    S.h_sig = C.sigma;
+    const double m = 2.0 * S.h_step;
+    C.need_h = D.bias_on && R.dvmax != 0.0 && C.sigma > R.sig_lo - m && C.sigma < R.sig_hi + m;
+    if (list && C.need_h) D.h_list[atomicAdd(D.h_meta, 1)] = r;
+}
+
 // blockDim = 32 * (NPART + 1): warp q < NPART sums partial slot q, warp NPART sums K.
-__global__ void k_scalar(Dev D, int mode) {
+__global__ void k_scalar(Dev D, int mode, int lazy, int list) {
     const int r = blockIdx.x;
     __shared__ double acc[NPART + 1];
     dev_scalar_acc(D, r, acc);
     if (threadIdx.x == 0) {
-        scalar_eval(D, r, mode, acc, acc[NPART], D.st[r], D.sc[r]);
+        Scal &C = D.sc[r];
+        if (scalar_eval(D, r, mode, acc, acc[NPART], D.st[r], C, lazy && !C.need_h)) {
+            if (D.lazy_h) expect_slope(D, r, D.st[r], C, list);
+        } else {
+            D.h_late[atomicAdd(D.h_meta + 1, 1)] = r;
+        }
         // the list (if rebuilt this step) has been used; count displacement-triggered builds
         const int f = D.rebuild[r];
         if (f) {
             if (f == 1) D.st[r].n_rebuild += 1;
             D.rebuild[r] = 0;
         }
+    }
+}
+
+// The replicas whose evaluation k_scalar put off: their sweep with H, then,
+// in the last CTA to finish, their scalars.
+template <int PREC, int S>
+__global__ void __launch_bounds__(256, PREC == HD_FP64 ? 1 : 3) k_scalar_late(Dev D, int mode, int list) {
+    const int n = D.h_meta[1];
+    if (n == 0) return;
+    if (!sweep_listed<PREC, S>(D, D.h_late, n, (unsigned *)D.h_meta + 3)) return;
+    __shared__ double acc[NPART + 1];
+    for (int q = 0; q < n; ++q) {
+        const int r = D.h_late[q];
+        dev_scalar_acc(D, r, acc);
+        if (threadIdx.x == 0) {
+            scalar_eval(D, r, mode, acc, acc[NPART], D.st[r], D.sc[r]);
+            expect_slope(D, r, D.st[r], D.sc[r], list);
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        D.h_meta[1] = 0;
+        D.h_meta[3] = 0;
     }
 }
 
@@ -1175,7 +1236,7 @@ __global__ void k_nhc(Dev D, int mode) {
 // Mobile atoms only; rigid atoms follow the body velocity; fixed atoms stay.
 __device__ __forceinline__ int4 post_move(const Dev &D, const RepDev &R, int r, int i, dbl4 x, int4 p) {
     const int4 q = fix_pos(R, x, p.w);
-    D.rec[i].p = q;
+    D.p[i] = q;
     const int4 b = D.pfixb[i];
     const float ex = (float)(int)((unsigned)q.x - (unsigned)b.x) * R.fx_lsb[0];
     const float ey = (float)(int)((unsigned)q.y - (unsigned)b.y) * R.fx_lsb[1];
@@ -1187,17 +1248,14 @@ __device__ __forceinline__ int4 post_move(const Dev &D, const RepDev &R, int r, 
     return q;
 }
 
-// Split form: the new fixed-point image and r - r_O as the difference of
-// images, in one 32-byte record store; then the checks of post_move.  r - r_O
+// Split form: the new fixed-point image, the checks of post_move, and that
+// r - r_O (the difference of the images of r and r_O) has not wrapped.  It
 // wraps at L / 2^(k+1) >= 4 (rc + skin); an atom is reported (HD_ERR_NUMERIC)
 // when it has moved 3/4 of that from its r_O.
 __device__ __forceinline__ void post_move32(const Dev &D, const RepDev &R, int r, int i, dbl4 x, int4 p) {
     const int4 q = fix_pos(R, x, p.w);
     const int4 d = img_diff(q, D.po[i]);
-    AtomRec a;
-    a.p = q;
-    a.d = d;
-    D.rec[i] = a;
+    D.p[i] = q;
     const int4 b = D.pfixb[i];
     const float ex = (float)(int)((unsigned)q.x - (unsigned)b.x) * R.fx_lsb[0];
     const float ey = (float)(int)((unsigned)q.y - (unsigned)b.y) * R.fx_lsb[1];
@@ -1215,7 +1273,7 @@ __device__ __forceinline__ void dev_update64(const Dev &D, int t, int mode, cons
     const RepDev &R = D.rep[r];
     const bool act = threadIdx.x < D.tile_n[t];
     const int i = D.tile_start[t] + (act ? threadIdx.x : 0);
-    const int4 p = D.rec[i].p;
+    const int4 p = D.p[i];
     const int role = act ? ((p.w >> 8) & 0xff) : ROLE_FIXED;
     double kin = 0.0;
     if (role != ROLE_FIXED) {
@@ -1311,8 +1369,7 @@ __device__ __forceinline__ void dev_update32(const Dev &D, int t, int mode, cons
     const RepDev &R = D.rep[r];
     const bool act = threadIdx.x < D.tile_n[t];
     const int i = D.tile_start[t] + (act ? threadIdx.x : 0);
-    const AtomRec ai = D.rec[i];
-    const int4 p = ai.p;
+    const int4 p = D.p[i];
     const int role = act ? ((p.w >> 8) & 0xff) : ROLE_FIXED;
     // the closing half kick of one step and the opening one of the next see
     // the same force: between steps of one call a Langevin replica takes one
@@ -1327,8 +1384,9 @@ __device__ __forceinline__ void dev_update32(const Dev &D, int t, int mode, cons
         dbl4 x = D.x[i];
         if (role == ROLE_MOBILE) {
             const float4 F = D.f32[i], H = D.h32[i];
-            const float4 dr = make_float4((float)ai.d.x * R.fx_lsb[0], (float)ai.d.y * R.fx_lsb[1],
-                                          (float)ai.d.z * R.fx_lsb[2], 0.f);
+            const int4 di = img_diff(p, D.po[i]);
+            const float4 dr = make_float4((float)di.x * R.fx_lsb[0], (float)di.y * R.fx_lsb[1],
+                                          (float)di.z * R.fx_lsb[2], 0.f);
             const float ca = (float)C.ca, cb = (float)C.cb;
             double Fx = (double)fmaf(ca, H.x - F.x, fmaf(cb, dr.x, F.x));
             double Fy = (double)fmaf(ca, H.y - F.y, fmaf(cb, dr.y, F.y));
@@ -1492,9 +1550,9 @@ __global__ void k_qinit(Dev Q, Dev M) {
     if (threadIdx.x < Q.tile_n[t]) {
         const int i = Q.tile_start[t] + threadIdx.x;
         const dbl4 x = M.x[i];
-        const int4 p = M.rec[i].p;
+        const int4 p = M.p[i];
         Q.x[i] = x;
-        Q.rec[i].p = p;
+        Q.p[i] = p;
         if (Q.prec == HD_FP64) Q.v64[i] = make_dbl4(0, 0, 0, 0);
         else Q.v32[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (Q.q_ftol_stay > 0.0) {
@@ -1523,7 +1581,7 @@ __global__ void k_qscalar(Dev D, int max_iter) {
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (w < QPART) {
         double a = (w == QP_FMAX2) ? 0.0 : 0.0;
-        for (int t = R.tile0 + lane; t < R.tile0 + R.ntile; t += 32) {
+        for (int t = R.tile0 * D.split + lane; t < (R.tile0 + R.ntile) * D.split; t += 32) {
             const double v = D.part[(size_t)t * NPART + w];
             a = (w == QP_FMAX2) ? fmax(a, v) : a + v;
         }
@@ -1703,7 +1761,7 @@ __global__ void __launch_bounds__(256) k_qupdate(Dev D) {
     if (threadIdx.x < D.tile_n[t]) {
         const int i = D.tile_start[t] + threadIdx.x;
         const RepDev &R = D.rep[r];
-        const int4 p = D.rec[i].p;
+        const int4 p = D.p[i];
         const int role = (p.w >> 8) & 0xff;
         if (D.prec == HD_FP64) {
             dbl4 x;
@@ -1756,11 +1814,7 @@ __global__ void k_adopt(Dev Q, Dev M, const int *adopt) {
     M.xo[i] = make_dbl4(q.x, q.y, q.z, 0.0);
     const dbl4 x = M.x[i];
     if (M.prec == HD_FP64) M.dr64[i] = make_dbl4(x.x - q.x, x.y - q.y, x.z - q.z, 0.0);
-    else {
-        const int4 po = fix_pos(M.rep[r], make_dbl4(q.x, q.y, q.z, 0.0), 0);
-        M.po[i] = po;
-        M.rec[i].d = img_diff(M.rec[i].p, po);
-    }
+    else M.po[i] = fix_pos(M.rep[r], make_dbl4(q.x, q.y, q.z, 0.0), 0);
 }
 
 // ---------------------------------------------------------------- persistent driver
@@ -1807,7 +1861,7 @@ __device__ __forceinline__ bool grp_barrier(const Dev &D, int r, int nc, unsigne
     return true;
 }
 
-template <int PREC>
+template <int PREC, int SPLIT>
 __global__ void __launch_bounds__(128, 4) k_persist(Dev D, int nsteps) {
     const int r = D.cta_rep[blockIdx.x];
     if (r < 0) return;
@@ -1890,14 +1944,17 @@ __global__ void __launch_bounds__(128, 4) k_persist(Dev D, int nsteps) {
             for (int c = me; c < R.ncell; c += nc) dev_nlist_cell(D, r, c, M, sp, smask);
             if (!grp_barrier(D, r, nc, epoch)) return;
         }
-        for (int t = R.tile0 + me; t < R.tile0 + R.ntile; t += nc) {
+        for (int t = R.tile0 * SPLIT + me; t < (R.tile0 + R.ntile) * SPLIT; t += nc) {
             // per-atom energies (observables only) on the last step of the call
+            // and H.(r - r_O) there and wherever a bias may use it
             if (PREC == HD_FP64) {
-                if (k == nsteps) dev_pair64<false, true>(D, t);
-                else dev_pair64<false, false>(D, t);
+                if (k == nsteps) dev_pair64<false, true, true, SPLIT>(D, t);
+                else if (D.bias_on) dev_pair64<false, false, true, SPLIT>(D, t);
+                else dev_pair64<false, false, false, SPLIT>(D, t);
             } else {
-                if (k == nsteps) dev_pair32<false, true>(D, t);
-                else dev_pair32<false, false>(D, t);
+                if (k == nsteps) dev_pair32<false, true, true, SPLIT>(D, t);
+                else if (D.bias_on) dev_pair32<false, false, true, SPLIT>(D, t);
+                else dev_pair32<false, false, false, SPLIT>(D, t);
             }
         }
         if (!grp_barrier(D, r, nc, epoch)) return;
@@ -1925,10 +1982,11 @@ static inline int nthr(const Dev &D) { return D.block; }
 size_t nl_smem_bytes(const Dev &D, int nwarps) {
     return 27 * (size_t)D.cell_cap * sizeof(int4) + (size_t)nwarps * nl_mask_words(D) * sizeof(unsigned);
 }
-// the persistent kernel runs the list build and the pair sweep in one launch
-static size_t persist_smem_bytes(const Dev &D) {
-    const size_t a = nl_smem_bytes(D, (D.block + 31) / 32), b = pair_smem_bytes_for(D.block);
-    return a > b ? a : b;
+static size_t persist_smem_bytes(const Dev &D) { return nl_smem_bytes(D, (D.block + 31) / 32); }
+typedef void (*persist_fn)(Dev, int);
+static persist_fn persist_kernel(const Dev &D) {
+    if (D.prec == HD_FP64) return D.split == 4 ? k_persist<HD_FP64, 4> : k_persist<HD_FP64, 1>;
+    return D.split == 4 ? k_persist<HD_FP32_SPLIT, 4> : k_persist<HD_FP32_SPLIT, 1>;
 }
 cudaError_t nl_configure(const Dev &D, int *nl_blocks_per_sm) {
     const int bytes = (int)nl_smem_bytes(D, NL_THREADS / 32), pbytes = (int)persist_smem_bytes(D);
@@ -1938,9 +1996,7 @@ cudaError_t nl_configure(const Dev &D, int *nl_blocks_per_sm) {
     *nl_blocks_per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(nl_blocks_per_sm, k_nlist, NL_THREADS, bytes);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_persist<HD_FP64>, cudaFuncAttributeMaxDynamicSharedMemorySize, pbytes);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_persist<HD_FP32_SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, pbytes);
+    return cudaFuncSetAttribute(persist_kernel(D), cudaFuncAttributeMaxDynamicSharedMemorySize, pbytes);
 }
 
 void launch_init(const Dev &D, const int *draw_vel, cudaStream_t s) {
@@ -1959,25 +2015,39 @@ void launch_rebuild(const Dev &D, cudaStream_t s) {
     launch_rebuild_prep(D, s);
     launch_nlist(D, s);
 }
-void launch_pair(const Dev &D, bool quench, bool energy, cudaStream_t s) {
+template <int S>
+static void pair_of(const Dev &D, int kind, cudaStream_t s) {
+    const int grid = D.ntile * S, n = nthr(D);
     if (D.prec == HD_FP64) {
-        if (quench) k_pair64<true, false><<<D.ntile, nthr(D), 0, s>>>(D);
-        else if (energy) k_pair64<false, true><<<D.ntile, nthr(D), 0, s>>>(D);
-        else k_pair64<false, false><<<D.ntile, nthr(D), 0, s>>>(D);
-    } else if (D.pair_x2 && D.block <= 128) {
-        const size_t sm = pair_smem_bytes_for(D.block);
-        if (quench) k_pair32x2<true, false><<<D.ntile, nthr(D), sm, s>>>(D);
-        else if (energy) k_pair32x2<false, true><<<D.ntile, nthr(D), sm, s>>>(D);
-        else k_pair32x2<false, false><<<D.ntile, nthr(D), sm, s>>>(D);
+        if (kind == PAIR_QUENCH) k_pair64<true, false, false, S><<<grid, n, 0, s>>>(D, SWEEP_ALL);
+        else if (kind == PAIR_ENERGY) k_pair64<false, true, true, S><<<grid, n, 0, s>>>(D, SWEEP_ALL);
+        else if (kind == PAIR_FULL) k_pair64<false, false, true, S><<<grid, n, 0, s>>>(D, SWEEP_ALL);
+        else k_pair64<false, false, false, S><<<grid, n, 0, s>>>(D, SWEEP_PLAIN);
+        if (kind == PAIR_LAZY && D.bias_on) k_pair_hot<HD_FP64, S><<<D.hot_grid, n, 0, s>>>(D);
     } else {
-        const size_t sm = pair_smem_bytes_for(D.block);
-        if (quench) k_pair32<true, false><<<D.ntile, nthr(D), sm, s>>>(D);
-        else if (energy) k_pair32<false, true><<<D.ntile, nthr(D), sm, s>>>(D);
-        else k_pair32<false, false><<<D.ntile, nthr(D), sm, s>>>(D);
+        if (kind == PAIR_QUENCH) k_pair32<true, false, false, S><<<grid, n, 0, s>>>(D, SWEEP_ALL);
+        else if (kind == PAIR_ENERGY) k_pair32<false, true, true, S><<<grid, n, 0, s>>>(D, SWEEP_ALL);
+        else if (kind == PAIR_FULL) k_pair32<false, false, true, S><<<grid, n, 0, s>>>(D, SWEEP_ALL);
+        else k_pair32<false, false, false, S><<<grid, n, 0, s>>>(D, SWEEP_PLAIN);
+        if (kind == PAIR_LAZY && D.bias_on) k_pair_hot<HD_FP32_SPLIT, S><<<D.hot_grid, n, 0, s>>>(D);
     }
 }
-void launch_scalar(const Dev &D, int mode, cudaStream_t s) {
-    k_scalar<<<D.nrep, 32 * (NPART + 1), 0, s>>>(D, mode);
+void launch_pair(const Dev &D, int kind, cudaStream_t s) {
+    if (D.split == 4) pair_of<4>(D, kind, s);
+    else pair_of<1>(D, kind, s);
+}
+void launch_scalar(const Dev &D, int mode, bool lazy, bool list, cudaStream_t s) {
+    const bool more = D.lazy_h && D.bias_on;
+    k_scalar<<<D.nrep, 32 * (NPART + 1), 0, s>>>(D, mode, lazy && more, list && more);
+    if (!lazy || !more) return;
+    const int n = nthr(D), g = D.hot_grid, li = list && more;
+    if (D.prec == HD_FP64) {
+        if (D.split == 4) k_scalar_late<HD_FP64, 4><<<g, n, 0, s>>>(D, mode, li);
+        else k_scalar_late<HD_FP64, 1><<<g, n, 0, s>>>(D, mode, li);
+    } else {
+        if (D.split == 4) k_scalar_late<HD_FP32_SPLIT, 4><<<g, n, 0, s>>>(D, mode, li);
+        else k_scalar_late<HD_FP32_SPLIT, 1><<<g, n, 0, s>>>(D, mode, li);
+    }
 }
 void launch_update(const Dev &D, int mode, cudaStream_t s) {
     if (D.prec == HD_FP64) k_update64<<<D.ntile, nthr(D), 0, s>>>(D, mode);
@@ -1988,16 +2058,14 @@ void launch_nhc(const Dev &D, int mode, cudaStream_t s) { k_nhc<<<D.nrep, 32, 0,
 void launch_qinit(const Dev &Q, const Dev &M, cudaStream_t s) { k_qinit<<<Q.ntile, nthr(Q), 0, s>>>(Q, M); }
 void launch_qiter(const Dev &Q, int max_iter, cudaStream_t s) {
     launch_rebuild(Q, s);
-    launch_pair(Q, true, false, s);
+    launch_pair(Q, PAIR_QUENCH, s);
     k_qscalar<<<Q.nrep, 32 * QPART, 0, s>>>(Q, max_iter);
     k_qupdate<<<Q.ntile, nthr(Q), 0, s>>>(Q);
 }
 void launch_qdisp(const Dev &Q, cudaStream_t s) { k_qdisp<<<Q.ntile, nthr(Q), 0, s>>>(Q); }
 int persist_blocks_per_sm(const Dev &D) {
     int nb = 0;
-    const size_t sm = persist_smem_bytes(D);
-    if (D.prec == HD_FP64) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_persist<HD_FP64>, D.block, sm);
-    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_persist<HD_FP32_SPLIT>, D.block, sm);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, persist_kernel(D), D.block, persist_smem_bytes(D));
     return nb;
 }
 cudaError_t launch_persist(const Dev &D, int grid, int nsteps, cudaStream_t s) {
@@ -2015,8 +2083,7 @@ cudaError_t launch_persist(const Dev &D, int grid, int nsteps, cudaStream_t s) {
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (D.prec == HD_FP64) return cudaLaunchKernelEx(&cfg, k_persist<HD_FP64>, D, nsteps);
-    return cudaLaunchKernelEx(&cfg, k_persist<HD_FP32_SPLIT>, D, nsteps);
+    return cudaLaunchKernelEx(&cfg, persist_kernel(D), D, nsteps);
 }
 void launch_adopt(const Dev &Q, const Dev &M, const int *adopt, cudaStream_t s) {
     k_adopt<<<M.ntile, nthr(M), 0, s>>>(Q, M, adopt);

@@ -11,9 +11,12 @@ void launch_init(const Dev &D, const int *draw_vel, cudaStream_t s);
 void launch_rebuild(const Dev &D, cudaStream_t s);            // 5 kernels, flag-gated per replica
 void launch_rebuild_prep(const Dev &D, cudaStream_t s);       // the first 4: plan, clear, bin, cell sort
 void launch_nlist(const Dev &D, cudaStream_t s);              // the 5th: rows from the cells
-// energy: also compute per-atom LJ energies (observables only; not needed by the dynamics)
-void launch_pair(const Dev &D, bool quench, bool energy, cudaStream_t s);
-void launch_scalar(const Dev &D, int mode, cudaStream_t s);
+// FULL: force and H.(r - r_O); ENERGY: per-atom LJ energies too (observables, not
+// needed by the dynamics); LAZY: H.(r - r_O) for the replicas expected in their band
+enum { PAIR_FULL = 0, PAIR_ENERGY = 1, PAIR_LAZY = 2, PAIR_QUENCH = 3 };
+void launch_pair(const Dev &D, int kind, cudaStream_t s);
+// lazy: the sweep before was PAIR_LAZY; list: the next one is
+void launch_scalar(const Dev &D, int mode, bool lazy, bool list, cudaStream_t s);
 void launch_update(const Dev &D, int mode, cudaStream_t s);
 void launch_obs(const Dev &D, cudaStream_t s);
 void launch_nhc(const Dev &D, int mode, cudaStream_t s);          // the chain between two kicks, per replica
