@@ -206,6 +206,9 @@ bool make_plan(const hd_replica_desc *reps, int n_rep, const hd_params *p, Plan 
             const double u = R.fx_scale[a] != 0.0 ? 1.0 / R.fx_scale[a] : 0.0;
             R.lsb_rel[a] = R.fx_lsb[a] != 0.f ? (float)((u - (double)R.fx_lsb[a]) / (double)R.fx_lsb[a]) : 0.f;
         }
+        R.nl_local = 1;
+        for (int a = 0; a < 3; ++a)
+            if (R.periodic[a] && R.nc[a] < 4) R.nl_local = 0;
         R.ncell = R.nc[0] * R.nc[1] * R.nc[2];
         R.cell0 = (int)ncell;
         R.wg0 = P.nwg;

@@ -101,6 +101,7 @@ struct RepDev {
     float rc2u_lo, rc2u_hi, near2u;      // rc^2 (1 -+ 2^-20); the exact r^2 is taken below near2u = (4/3) r_0^2
     float r0u_hi[2][2], r0u_lo[2][2];    // r_0^2 = 2^(1/3) sigma_ab^2 (LJ minimum, squared) as hi + lo
     float eps12f[2][2], eps12l[2][2];    // 12 eps_ab as hi + lo
+    int nl_local;                // every periodic axis has four cells or more (see k_nlist)
     float rA2f;                  // list class A (first shell): FP32 r^2 below this at build time
     float kbondf;                // Eq. 12 bonds: stiffness (FP32)
     double kbond, rbond;         // Eq. 12 bonds: stiffness, rest length

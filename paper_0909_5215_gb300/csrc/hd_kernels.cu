@@ -18,6 +18,15 @@
 
 namespace hd {
 
+// ---------------------------------------------------------------- packed FP32x2
+__device__ __forceinline__ float2 f2c(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 f2i(int a, int b) { return make_float2((float)a, (float)b); }
+__device__ __forceinline__ float2 f2neg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 f2mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 f2add(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 f2sub(float2 a, float2 b) { return __fadd2_rn(a, f2neg(b)); }
+__device__ __forceinline__ float2 f2fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+
 // ---------------------------------------------------------------- reductions
 // Sums NV per-thread values over the CTA in a fixed order and writes them to
 // out[0..NV).  Slot `maxslot` (if >= 0) is reduced with max instead of +.
@@ -262,36 +271,152 @@ __global__ void __launch_bounds__(128) k_cellsort(Dev D) {
 // (rc + skin)^2.  One CTA builds the rows of one cell's atoms.  It first
 // stages the candidates of the cell's stencil (the 27, or 9 in 2-D,
 // surrounding cells in ascending cell order, each cell's atoms ascending) in
-// shared memory: index and fixed-point position.  Then one warp per atom of
-// the cell walks the staged candidates 32 at a time.  An FP32 test on the
-// exact integer differences decides all but a thin band around the radius,
-// where the oracle's FP64 test is repeated operation for operation.  Each
-// accepted j gets a class, kept in shared memory:
-//   A (first shell) FP32 r^2 < rA^2, the pairs that can come within the
-//                   range where the pair sweep takes the exact r^2;
-//   B               the rest of the pairs within rc at build time;
-//   C (skin shell)  the rest of the row.
+// shared memory.  Then one warp per atom of the cell takes two passes.
+//
+// 1. All candidates (~675 in a dense 3-D crystal, of which ~76 are neighbours),
+//    64 at a time: the FP32 distance, one compare, and the place of each
+//    accepted candidate goes to the warp's buffer, packed by ballot.  This is
+//    where the instructions are, so positions are staged as FP32 offsets from
+//    the cell's centre (three packed subtractions and three packed products
+//    per 64) and nothing else is decided here.  An offset is the exact integer
+//    difference of the images, rounded: r^2 is good to ~1e-6, far inside the
+//    2^-12 wide band that pass 2 decides exactly.  A periodic axis of three
+//    cells or one has no such offsets (a neighbour may be nearer around the
+//    box); a replica with one stages the images and subtracts those.
+// 2. The accepted ones: the atom itself leaves, the thin band around the
+//    radius takes the oracle's FP64 test operation for operation, and each j
+//    gets a class: A (first shell) FP32 r^2 < rA^2, the pairs that can come
+//    within the range where the pair sweep takes the exact r^2; B the rest of
+//    the pairs within rc at build time; C (skin shell) the rest of the row.
+//
 // The row is then written as A | B | C, each block in candidate order, so the
 // lanes of the pair sweep leave the first shell, and later the cutoff, at
-// nearly the same k.  The row order is a deterministic function of the cell
-// lists (sorted by k_cellsort); reads return each row ascending in j.
-// ballot masks per warp of the list build: three per 32 staged candidates
-__host__ __device__ inline int nl_mask_words(const Dev &D) { return 3 * ((27 * D.cell_cap + 31) / 32); }
+// nearly the same k; a lane writes a group of four.  The row order is a
+// deterministic function of the cell lists (sorted by k_cellsort); reads
+// return each row ascending in j.
+//
+// Bound by instruction issue and the latency of the staging.
 // Row-build CTA: 8 warps share one staged stencil (the cell's atoms split among them).
 constexpr int NL_THREADS = 256;
+// Accepted candidates a warp holds between the passes: the longest row and
+// room for the atom itself and the band's candidates that pass 2 takes out.
+constexpr int NL_BUF = 256;
 
 struct NlSmem {
     int nst, tot, kc;
-    int cell[27], off[28];
+    int cell[27], off[28], centre[3];
 };
 
-__device__ __forceinline__ void dev_nlist_cell(const Dev &D, int r, int c, NlSmem &M, int4 *sp,
-                                               unsigned *smask) {
+// Shared memory of a row-build CTA: the staged candidates (x, y, z as FP32
+// offsets or images; slot, top bit its type), then per warp the accepted
+// candidates and the row.
+__host__ __device__ inline int nl_cand(const Dev &D) { return (27 * D.cell_cap + 63) / 64 * 64; }
+__host__ __device__ inline size_t nl_warp_bytes(const Dev &D) { return NL_BUF * 2 + (size_t)D.ngrp * sizeof(int4); }
+struct NlStage {
+    float *x, *y, *z;
+    int *j;
+    char *warp;
+};
+
+template <bool LOCAL>
+__device__ __forceinline__ void dev_nlist_rows(const Dev &D, const RepDev &R, int r, int m, const NlSmem &M, const NlStage &T) {
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const unsigned below = (1u << lane) - 1u;
+    const int tot = M.tot, cap = D.maxnb;
+    const float lx = R.fx_lsb[0], ly = R.fx_lsb[1], lz = R.fx_lsb[2], rA2 = R.rA2f;
+    const float lo = D.rl2_lo_f, hi = D.rl2_hi_f, rc2 = D.rc2_lo_f;
+    unsigned short *buf = reinterpret_cast<unsigned short *>(T.warp + w * nl_warp_bytes(D));
+    int *row = reinterpret_cast<int *>(buf + NL_BUF);
+    // difference of two staged coordinates
+    auto diff = [](float a, float b, float l) {
+        return LOCAL ? a - b : (float)(int)(__float_as_uint(a) - __float_as_uint(b)) * l;
+    };
+    for (int a = w; a < m; a += nw) {
+        const int slot = M.off[M.kc] + a;
+        const float xi = T.x[slot], yi = T.y[slot], zi = T.z[slot];
+        const int i = T.j[slot] & 0x7fffffff;
+        int cnt = 0;
+        for (int base = 0; base < tot; base += 64) {
+            const int q = base + 2 * lane;
+            const float2 xj = *reinterpret_cast<const float2 *>(T.x + q), yj = *reinterpret_cast<const float2 *>(T.y + q),
+                         zj = *reinterpret_cast<const float2 *>(T.z + q);
+            float2 dx, dy, dz;
+            if (LOCAL) {
+                dx = f2sub(f2c(xi), xj);
+                dy = f2sub(f2c(yi), yj);
+                dz = f2sub(f2c(zi), zj);
+            } else {
+                dx = make_float2(diff(xi, xj.x, lx), diff(xi, xj.y, lx));
+                dy = make_float2(diff(yi, yj.x, ly), diff(yi, yj.y, ly));
+                dz = make_float2(diff(zi, zj.x, lz), diff(zi, zj.y, lz));
+            }
+            const float2 r2 = f2fma(dx, dx, f2fma(dy, dy, f2mul(dz, dz)));
+            // offsets past the last candidate are far away; images are not
+            const bool ina = r2.x < hi && (LOCAL || q < tot), inb = r2.y < hi && (LOCAL || q + 1 < tot);
+            const unsigned ma = __ballot_sync(full, ina), mb = __ballot_sync(full, inb);
+            int at = cnt + __popc(ma & below) + __popc(mb & below);
+            if (ina && at < NL_BUF) buf[at] = (unsigned short)q;
+            at += ina;
+            if (inb && at < NL_BUF) buf[at] = (unsigned short)(q + 1);
+            cnt += __popc(ma) + __popc(mb);
+        }
+        const int have = min(cnt, NL_BUF);
+        __syncwarp();
+        int nA = 0, nB = 0, nC = 0;
+        unsigned mixed = (unsigned)T.j[slot] >> 31;
+        for (int base = 0; base < have; base += 32) {
+            int cl = 3;
+            const int e = base + lane;
+            const int q = e < have ? buf[e] : slot;
+            if (q != slot) {
+                const int jt = T.j[q], j = jt & 0x7fffffff;
+                const float dx = diff(xi, T.x[q], lx), dy = diff(yi, T.y[q], ly), dz = diff(zi, T.z[q], lz);
+                const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+                if (r2 < lo || exact_r2(R, D.x[i], D.x[j]) < D.rl2) {
+                    cl = r2 < rA2 ? 0 : (r2 < rc2 ? 1 : 2);
+                    mixed |= (unsigned)jt >> 31;
+                }
+            }
+            if (e < have) buf[e] = (unsigned short)(q | (cl << 14));
+            nA += __popc(__ballot_sync(full, cl == 0));
+            nB += __popc(__ballot_sync(full, cl == 1));
+            nC += __popc(__ballot_sync(full, cl == 2));
+        }
+        __syncwarp();
+        const int n = nA + nB + nC, kept = min(n, cap);
+        int bA = 0, bB = nA, bC = nA + nB;
+        for (int base = 0; base < have; base += 32) {
+            const int e = base + lane;
+            const int v = e < have ? buf[e] : 3 << 14, cl = v >> 14;
+            const unsigned mA = __ballot_sync(full, cl == 0), mB = __ballot_sync(full, cl == 1),
+                           mC = __ballot_sync(full, cl == 2);
+            const int pos = cl == 0 ? bA + __popc(mA & below) : (cl == 1 ? bB + __popc(mB & below) : bC + __popc(mC & below));
+            if (cl < 3 && pos < cap) row[pos] = T.j[v & 0x3fff] & 0x7fffffff;
+            bA += __popc(mA);
+            bB += __popc(mB);
+            bC += __popc(mC);
+        }
+        if (kept + lane < ((kept + 3) & ~3)) row[kept + lane] = i;     // fill up the last group
+        __syncwarp();
+        const size_t row4 = nbr_row4(D, R, i);
+        for (int g = lane; g < (kept + 3) >> 2; g += 32)
+            reinterpret_cast<int4 *>(D.nbr)[row4 + 32 * (size_t)g] = reinterpret_cast<const int4 *>(row)[g];
+        const bool mx = __any_sync(full, mixed != 0);
+        if (lane == 0) {
+            D.nnb[i] = kept | (mx ? NB_MIXED : 0);
+            if (n > cap || cnt > NL_BUF) set_err(D, HD_ERR_OVERFLOW, i, r);
+        }
+        __syncwarp();
+    }
+}
+
+__device__ __forceinline__ void dev_nlist_cell(const Dev &D, int r, int c, NlSmem &M, const NlStage &T) {
     const RepDev &R = D.rep[r];
     const int cell0 = R.cell0 + c;
     const int m = min(D.cell_cnt[cell0], D.cell_cap);
     if (m == 0) return;  // uniform: every thread reads the same count
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     if (w == 0) {
         // lane k < 27: stencil cell (k % 3, k / 3 % 3, k / 9) of the per-axis
         // lists, each list ascending (a periodic wrap puts nc-1 after 0 and 1)
@@ -345,12 +470,21 @@ __device__ __forceinline__ void dev_nlist_cell(const Dev &D, int r, int c, NlSme
             M.tot = incl;
             M.nst = nst;
         }
+        // the cell's centre in the fixed-point image
+        if (lane < 3) {
+            const int ca = lane == 0 ? ci[0] : (lane == 1 ? ci[1] : ci[2]);
+            const double x = R.periodic[lane] ? (ca + 0.5) * (R.L[lane] / R.nc[lane]) : R.cell_lo + (ca + 0.5) / R.cell_inv_w;
+            M.centre[lane] = R.periodic[lane] || lane == R.vert ? fix_coord(R, lane, x) : 0;
+        }
     }
     __syncthreads();
     // stage the stencil: every thread takes candidates idx, idx + blockDim, ...,
     // four at a time so that their loads are in flight together
     {
         const int tot = M.tot, nst = M.nst;
+        const bool local = R.nl_local != 0;
+        const float lx = R.fx_lsb[0], ly = R.fx_lsb[1], lz = R.fx_lsb[2];
+        const int cx = M.centre[0], cy = M.centre[1], cz = M.centre[2];
         for (int base = threadIdx.x; base < tot; base += 4 * blockDim.x) {
             int jj[4];
 #pragma unroll
@@ -373,102 +507,45 @@ __device__ __forceinline__ void dev_nlist_cell(const Dev &D, int r, int c, NlSme
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int idx = base + u * blockDim.x;
-                // w: the candidate's slot, top bit its type
-                if (idx < tot) sp[idx] = make_int4(pp[u].x, pp[u].y, pp[u].z, jj[u] | (pp[u].w << 31));
-            }
-        }
-    }
-    __syncthreads();
-    const int tot = M.tot, cap = D.maxnb;
-    const unsigned full = 0xffffffffu;
-    const float lx = R.fx_lsb[0], ly = R.fx_lsb[1], lz = R.fx_lsb[2];
-    // per warp: three ballot masks (classes A, B, C) per 32 candidates
-    unsigned *msk = smask + (size_t)w * nl_mask_words(D);
-    for (int a = w; a < m; a += nw) {
-        const int slot = M.off[M.kc] + a;
-        const int4 pi = sp[slot];
-        const int i = pi.w & 0x7fffffff;
-        const size_t row4 = nbr_row4(D, R, i);
-        unsigned mixed = (unsigned)pi.w >> 31;
-        int nA = 0, nB = 0, nC = 0;
-        // pass 1: classify every candidate, count the classes
-        for (int base = 0; base < tot; base += 32) {
-            const int q = base + lane;
-            int cl = 0;
-            if (q < tot) {
-                const int4 pj = sp[q];
-                const int j = pj.w & 0x7fffffff;
-                if (j != i) {
-                    const float dx = (float)(int)((unsigned)pi.x - (unsigned)pj.x) * lx;
-                    const float dy = (float)(int)((unsigned)pi.y - (unsigned)pj.y) * ly;
-                    const float dz = (float)(int)((unsigned)pi.z - (unsigned)pj.z) * lz;
-                    const float r2 = dx * dx + dy * dy + dz * dz;
-                    bool in;
-                    if (r2 < D.rl2_lo_f) in = true;
-                    else if (r2 >= D.rl2_hi_f) in = false;
-                    else in = exact_r2(R, D.x[i], D.x[j]) < D.rl2;
-                    if (in) {
-                        cl = r2 < R.rA2f ? 1 : (r2 < D.rc2_lo_f ? 2 : 3);
-                        mixed |= (unsigned)pj.w >> 31;
-                    }
+                if (idx < tot) {
+                    const int4 p = pp[u];
+                    const int ox = (int)((unsigned)p.x - (unsigned)cx), oy = (int)((unsigned)p.y - (unsigned)cy),
+                              oz = (int)((unsigned)p.z - (unsigned)cz);
+                    T.x[idx] = local ? (float)ox * lx : __int_as_float(p.x);
+                    T.y[idx] = local ? (float)oy * ly : __int_as_float(p.y);
+                    T.z[idx] = local ? (float)oz * lz : __int_as_float(p.z);
+                    T.j[idx] = jj[u] | (p.w << 31);      // top bit: the type
                 }
             }
-            const unsigned mA = __ballot_sync(full, cl == 1), mB = __ballot_sync(full, cl == 2),
-                           mC = __ballot_sync(full, cl == 3);
-            if (lane == 0) {
-                msk[3 * (base >> 5)] = mA;
-                msk[3 * (base >> 5) + 1] = mB;
-                msk[3 * (base >> 5) + 2] = mC;
-            }
-            nA += __popc(mA);
-            nB += __popc(mB);
-            nC += __popc(mC);
         }
-        __syncwarp();
-        // pass 2: write the row as A | B | C, each block in candidate order
-        int bA = 0, bB = nA, bC = nA + nB;
-        const unsigned below = (1u << lane) - 1u, bit = 1u << lane;
-        for (int base = 0; base < tot; base += 32) {
-            const unsigned mA = msk[3 * (base >> 5)], mB = msk[3 * (base >> 5) + 1], mC = msk[3 * (base >> 5) + 2];
-            const int cl = (mA & bit) ? 1 : ((mB & bit) ? 2 : ((mC & bit) ? 3 : 0));
-            if (cl) {
-                const int pos = cl == 1 ? bA + __popc(mA & below) : (cl == 2 ? bB + __popc(mB & below)
-                                                                             : bC + __popc(mC & below));
-                if (pos < cap) D.nbr[nbr_at(row4, pos)] = sp[base + lane].w & 0x7fffffff;
-            }
-            bA += __popc(mA);
-            bB += __popc(mB);
-            bC += __popc(mC);
-        }
-        __syncwarp();
-        {
-            const int n = nA + nB + nC, kept = min(n, cap);
-            const bool mx = __any_sync(full, mixed != 0);
-            if (kept + lane < ((kept + 3) & ~3)) D.nbr[nbr_at(row4, kept + lane)] = i;   // fill up the last group
-            if (lane == 0) {
-                D.nnb[i] = kept | (mx ? NB_MIXED : 0);
-                if (n > cap) set_err(D, HD_ERR_OVERFLOW, i, r);
-            }
-        }
+        // the last 64 are read whole
+        for (int idx = tot + threadIdx.x; idx < (tot + 63) / 64 * 64; idx += blockDim.x) T.x[idx] = T.y[idx] = T.z[idx] = 1e18f;
     }
+    __syncthreads();
+    if (R.nl_local) dev_nlist_rows<true>(D, R, r, m, M, T);
+    else dev_nlist_rows<false>(D, R, r, m, M, T);
     __syncthreads();  // the staging buffers are reused by the next cell
 }
 
-__device__ __forceinline__ void nl_smem_carve(const Dev &D, char *base, int4 *&sp, unsigned *&smask) {
-    sp = reinterpret_cast<int4 *>(base);
-    smask = reinterpret_cast<unsigned *>(base + (size_t)27 * D.cell_cap * sizeof(int4));
+__device__ __forceinline__ NlStage nl_smem_carve(const Dev &D, char *base) {
+    const int n = nl_cand(D);
+    NlStage T;
+    T.x = reinterpret_cast<float *>(base);
+    T.y = T.x + n;
+    T.z = T.y + n;
+    T.j = reinterpret_cast<int *>(T.z + n);
+    T.warp = reinterpret_cast<char *>(T.j + n);
+    return T;
 }
 
 __global__ void __launch_bounds__(NL_THREADS) k_nlist(Dev D) {
     extern __shared__ __align__(16) char nl_smem[];
     __shared__ NlSmem M;
-    int4 *sp;
-    unsigned *smask;
-    nl_smem_carve(D, nl_smem, sp, smask);
+    const NlStage T = nl_smem_carve(D, nl_smem);
     const int n = D.rb_meta[0], total = D.rb_meta[1];
     for (int idx = blockIdx.x; idx < total; idx += gridDim.x) {
         const int k = rb_find(D.rb_off, n, idx);
-        dev_nlist_cell(D, D.rb_list[k], idx - D.rb_off[k], M, sp, smask);
+        dev_nlist_cell(D, D.rb_list[k], idx - D.rb_off[k], M, T);
     }
 }
 
@@ -647,14 +724,6 @@ __device__ __forceinline__ float rcp_refined(float x) {
     const float y = rcp_approx(x);
     return fmaf(y, fmaf(-x, y, 1.f), y);
 }
-
-__device__ __forceinline__ float2 f2c(float a) { return make_float2(a, a); }
-__device__ __forceinline__ float2 f2i(int a, int b) { return make_float2((float)a, (float)b); }
-__device__ __forceinline__ float2 f2neg(float2 a) { return make_float2(-a.x, -a.y); }
-__device__ __forceinline__ float2 f2mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 f2add(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 f2sub(float2 a, float2 b) { return __fadd2_rn(a, f2neg(b)); }
-__device__ __forceinline__ float2 f2fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 
 // Split rows: S lanes of a warp share one row (lane s takes groups s, s + S,
 // ... of four entries) and a CTA holds block / S atoms.  See dev_pair32.
@@ -1874,9 +1943,7 @@ __global__ void __launch_bounds__(128, 4) k_persist(Dev D, int nsteps) {
     __shared__ int s_flag;
     __shared__ NlSmem M;
     extern __shared__ __align__(16) char nl_smem[];
-    int4 *sp;
-    unsigned *smask;
-    nl_smem_carve(D, nl_smem, sp, smask);
+    const NlStage T = nl_smem_carve(D, nl_smem);
     if (threadIdx.x == 0) {
         S = D.st[r];
         C = D.sc[r];
@@ -1941,7 +2008,7 @@ __global__ void __launch_bounds__(128, 4) k_persist(Dev D, int nsteps) {
                 if (leader) D.rebuild[r] = 0;
             }
             // rows are built cell by cell, so a CTA's tiles take rows other CTAs wrote
-            for (int c = me; c < R.ncell; c += nc) dev_nlist_cell(D, r, c, M, sp, smask);
+            for (int c = me; c < R.ncell; c += nc) dev_nlist_cell(D, r, c, M, T);
             if (!grp_barrier(D, r, nc, epoch)) return;
         }
         for (int t = R.tile0 * SPLIT + me; t < (R.tile0 + R.ntile) * SPLIT; t += nc) {
@@ -1976,11 +2043,9 @@ __global__ void __launch_bounds__(128, 4) k_persist(Dev D, int nsteps) {
 // ---------------------------------------------------------------- launchers
 static inline int nthr(const Dev &D) { return D.block; }
 
-// Dynamic shared memory of the list build: positions, indices and classes
-// of up to 27 cells of cell_cap candidates (classes: one byte per candidate
-// for each of the warps of a 128-thread CTA).
+// Dynamic shared memory of the list build.
 size_t nl_smem_bytes(const Dev &D, int nwarps) {
-    return 27 * (size_t)D.cell_cap * sizeof(int4) + (size_t)nwarps * nl_mask_words(D) * sizeof(unsigned);
+    return (size_t)nl_cand(D) * 16 + nwarps * nl_warp_bytes(D);
 }
 static size_t persist_smem_bytes(const Dev &D) { return nl_smem_bytes(D, (D.block + 31) / 32); }
 typedef void (*persist_fn)(Dev, int);
