@@ -271,7 +271,11 @@ bool make_plan(const hd_replica_desc *reps, int n_rep, const hd_params *p, Plan 
                 R.sig2f[a][b] = (float)(sig * sig);
                 R.shiftf[a][b] = (float)R.shift[a][b];
                 const double r0sq = std::cbrt(2.0) * sig * sig;   // LJ minimum 2^(1/6) sigma, squared
-                R.r0u_hi[a][b] = (float)(r0sq * pu2);
+                {   // 20 bits, so that its difference from any r^2 up to rc^2 is exact
+                    int e;
+                    const double m = std::frexp(r0sq * pu2, &e);
+                    R.r0u_hi[a][b] = (float)std::ldexp(std::floor(std::ldexp(m, 20)), e - 20);
+                }
                 R.r0u_lo[a][b] = (float)(r0sq * pu2 - (double)R.r0u_hi[a][b]);
                 R.eps12f[a][b] = (float)(12.0 * eps);
                 R.eps12l[a][b] = (float)(12.0 * eps - (double)R.eps12f[a][b]);
@@ -915,7 +919,7 @@ hd_status hd_create(const hd_replica_desc *reps, int n_rep, const hd_params *p, 
     // Leave the Hessian term out of the sweeps where it is not used: always
     // without a bias; with one, where the sweep is long enough to pay for the
     // two launches more (~5 us) that a step then takes.  Measured per sweep with
-    // and without it: 259 and ~150 us at 913,408 atoms (split form), 54 and 49
+    // and without it: 259 and 122 to 143 us at 913,408 atoms (split form), 54 and 49
     // at 121,000, where the launches cost what it saves; 514 and 327 us at
     // 57,088 in the FP64 form, whose pipe the term fills.  The eigenvalue bias
     // keeps the plain order.

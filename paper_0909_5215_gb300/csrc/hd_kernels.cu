@@ -772,7 +772,10 @@ __device__ __forceinline__ void dev_pair32(const Dev &D, int unit) {
         // 1/r^2: the hardware approximation and one Newton step (rcp_refined)
         float2 ir2 = make_float2(rcp_approx(h.x), rcp_approx(h.y));
         ir2 = f2fma(ir2, f2fma(f2neg(h), ir2, f2c(1.f)), ir2);
-        const float2 tt = f2mul(f2add(f2sub(r0h, h), l), ir2);
+        // r0h holds 20 bits, so r0h - h is exact whatever the distance; the rest
+        // joins by a product: added to r0h - h it would round off alike in every
+        // pair (1.8e-7 of each force beyond 1.6 sigma, all of one sign)
+        const float2 tt = f2fma(l, ir2, f2mul(f2sub(r0h, h), ir2));
         const float2 c1 = f2add(tt, f2c(1.f));
         const float2 c = f2mul(f2mul(c1, c1), c1);                               // 2 s^6
         const float2 w = f2mul(tt, f2fma(tt, f2add(tt, f2c(3.f)), f2c(3.f)));    // 2 s^6 - 1
