@@ -237,6 +237,8 @@ bool make_plan(const hd_replica_desc *reps, int n_rep, const hd_params *p, Plan 
         // interaction constants (Eq. 9 with the shift at rc)
         R.kT = d.kT;
         R.beta = 1.0 / d.kT;
+        R.inv_nrig = nrig > 0 ? 1.0 / nrig : 0.0;
+        R.boost_max = std::exp(d.dvmax / d.kT);
         R.c_ou = std::exp(-d.gamma * p->dt);
         R.s_ou = std::sqrt((1.0 - R.c_ou * R.c_ou) * d.kT);
         R.c_ouf = (float)R.c_ou;
@@ -582,7 +584,11 @@ void fill_dev(hd_ctx *c) {
     D.cell_cap = P.cell_cap;
     D.ncell = P.ncell;
     D.max_cells = 0;
-    for (const RepDev &R : P.rep) D.max_cells = std::max(D.max_cells, R.ncell);
+    D.max_parts = 0;
+    for (const RepDev &R : P.rep) {
+        D.max_cells = std::max(D.max_cells, R.ncell);
+        D.max_parts = std::max(D.max_parts, R.ntile * P.split);
+    }
     D.prec = P.prec;
     D.block = P.block;
     D.ngrp = (P.maxnb + 3) / 4;
@@ -1025,6 +1031,7 @@ hd_status hd_set_bias(hd_ctx *c, const double *bias) {
     for (int r = 0; r < c->P.nrep; ++r) {
         if (!(bias[4 * r + 3] >= 1.0)) return fail(c, HD_ERR_ARG, "replica %d: m must be >= 1", r);
         c->P.rep[r].dvmax = bias[4 * r];
+        c->P.rep[r].boost_max = std::exp(bias[4 * r] / c->P.rep[r].kT);
         c->P.rep[r].sig_lo = bias[4 * r + 1];
         c->P.rep[r].sig_hi = bias[4 * r + 2];
         c->P.rep[r].m_exp = (int)bias[4 * r + 3];

@@ -70,6 +70,7 @@ struct RepDev {
     int cell0, ncell, vert, wg0;          // wg0: first 32-atom block of the list
     int nc[3], periodic[3];
     double L[3], invL[3];
+    double inv_nrig, boost_max;  // 1 / n_rig (0 without a rigid layer), exp(dvmax / kT)
     double kT, beta, c_ou, s_ou, kspring, fnormal, slider[2];
     double v_slide;              // continuous sliding: x_S = slider[0] + (step - slide_step0) (v_slide dt)
     long long slide_step0;       // step count of the configuration at which slider[0] was set
@@ -147,6 +148,7 @@ struct Scal {
 
 struct Dev {
     int nrep, ntile, natom, maxnb, cell_cap, ncell, prec, bias_on, block;
+    int max_parts;               // largest number of tile parts of one replica
     int ngrp, split;             // groups of four per list row; lanes that share a row of the pair sweep (1 or 4)
     int q_method, max_cells;        // max_cells: largest cell count of one replica
     double dt, rc2, rl2, half_skin2, q_ftol, q_step, q_theta;

@@ -1051,22 +1051,35 @@ __global__ void __launch_bounds__(256, PREC == HD_FP64 ? 1 : 3) k_pair_hot(Dev D
 //   body kicks and the clocks: t_h += dt exp(DeltaV / kT) (Eq. 3).
 // need_hess: the caller has no H.dr of this configuration; with DeltaV' != 0
 // nothing is changed then and the result is false.
+//
+// One warp evaluates it (every lane calls; S and C may be in shared or global
+// memory): lane a < 3 holds axis a.  The chain of FP64 operations is all of
+// its time, so it is kept short: one square root and one division (1/d), the
+// other quotients by reciprocals that the host set, the exponential only
+// inside the band (its value at DeltaV_max is the host's, at 0 it is 1).  With
+// one thread for all of it, 22 divisions one after another, a step of 16 x 421
+// atoms in one launch took 30.8 us; it takes 19.3 now, and the kernel of 8 x
+// 1,983 atoms 13 us where it took 21.
 __device__ bool scalar_eval(const Dev &D, int r, int mode, const double *acc, double ksum, RepState &S, Scal &C,
                             bool need_hess = false) {
+    const unsigned full = 0xffffffffu;
     const RepDev &R = D.rep[r];
-    const int nr = R.nrig, dim = R.dim, vert = R.vert;
-    const double xs = slider_x(R, S.step, D.dt);
-    double xT[3] = {0, 0, 0}, gs[3] = {0, 0, 0};
-    if (nr > 0) {
-        for (int a = 0; a < 3; ++a) xT[a] = acc[PART_XRIG + a] / (double)nr;
-        gs[0] = R.kspring * (xT[0] - xs);
-        if (dim == 3) gs[1] = R.kspring * (xT[1] - R.slider[1]);
-        gs[vert] = R.fnormal;
-    }
-    double G = acc[PART_G];
-    if (nr > 0) G += (gs[0] * acc[PART_DRRIG] + gs[1] * acc[PART_DRRIG + 1] + gs[2] * acc[PART_DRRIG + 2]) / (double)nr;
-    const double d = sqrt(acc[PART_D2]);
-    const double sig = d > 0.0 ? G / d : 0.0;
+    const int lane = threadIdx.x & 31, a = lane < 3 ? lane : 2;
+    const int dim = R.dim, vert = R.vert;
+    const bool rig = R.nrig > 0, mine = lane < 3;
+    const double inr = R.inv_nrig, h = D.dt, k = R.kspring, fn = R.fnormal;
+    const long long step = S.step;
+    const double vb0 = S.vbody[a], xs = slider_x(R, step, h);
+    const bool spring = a == 0 || (a == 1 && dim == 3);           // else the load, on the vertical axis
+    const double xT = rig ? acc[PART_XRIG + a] * inr : 0.0;
+    const double off = xT - (a == 0 ? xs : R.slider[1]);
+    const double gs = !rig ? 0.0 : (a == vert ? fn : (spring ? k * off : 0.0));
+    auto sum3 = [&](double v) { return (__shfl_sync(full, v, 0) + __shfl_sync(full, v, 1)) + __shfl_sync(full, v, 2); };
+    const double gd = sum3(gs * acc[PART_DRRIG + a]);
+    const double ext = sum3(!rig ? 0.0 : (a == vert ? fn * xT : (spring ? 0.5 * k * off * off : 0.0)));
+    const double G = acc[PART_G] + (rig ? gd * inr : 0.0);
+    const double d = sqrt(acc[PART_D2]), id = d > 0.0 ? 1.0 / d : 0.0;
+    const double sig = G * id;
     double dV = 0.0, dVp = 0.0, dVe = 0.0, d1 = 0.0, d2 = 0.0;
     if (D.bias_on) dv1(R, sig, dV, dVp);
     d1 = dV;
@@ -1083,79 +1096,97 @@ __device__ bool scalar_eval(const Dev &D, int r, int mode, const double *acc, do
         }
     }
     if (need_hess && dVp != 0.0) return false;
-    const double ca = d > 0.0 ? -dVp / d : 0.0;
-    const double cb = d > 0.0 ? dVp * sig / (d * d) : 0.0;
-    double fb[3] = {0, 0, 0};
-    if (nr > 0)
-        for (int a = 0; a < 3; ++a) {
-            const double grig = -acc[PART_FRIG + a] + gs[a];
-            const double srig = d > 0.0 ? (acc[PART_HRIG + a] + grig) / d - sig * acc[PART_DRRIG + a] / (d * d) : 0.0;
-            fb[a] = acc[PART_FRIG + a] - gs[a] - dVp * srig;
-        }
-    if (dVe != 0.0 && nr > 0) {
+    const double ca = -dVp * id, cb = dVp * sig * (id * id);
+    double fb = 0.0;
+    if (rig) {
+        const double F = acc[PART_FRIG + a];
+        const double srig = (acc[PART_HRIG + a] + (gs - F)) * id - sig * acc[PART_DRRIG + a] * (id * id);
+        fb = F - gs - (dVp != 0.0 ? dVp * srig : 0.0);
+    }
+    if (dVe != 0.0 && rig) {
         // the rigid layer's share of -dDeltaV/depsilon grad epsilon, summed per tile
-        for (int a = 0; a < 3; ++a) {
-            double e = 0.0;
-            for (int t = R.tile0; t < R.tile0 + R.ntile; ++t) e += D.epart[(size_t)t * 4 + a];
-            fb[a] -= dVe * e;
-        }
+        double e = 0.0;
+        for (int t = R.tile0; t < R.tile0 + R.ntile; ++t) e += D.epart[(size_t)t * 4 + a];
+        fb -= dVe * e;
     }
-    C.ce = -dVe;
-    C.dV1 = d1;
-    C.dV2 = d2;
-    double ext = 0.0;
-    if (nr > 0) {
-        ext = 0.5 * R.kspring * (xT[0] - xs) * (xT[0] - xs);
-        if (dim == 3) ext += 0.5 * R.kspring * (xT[1] - R.slider[1]) * (xT[1] - R.slider[1]);
-        ext += R.fnormal * xT[vert];
-    }
-    C.d = d; C.sigma = sig; C.dV = dV; C.dVp = dVp; C.G = G;
-    C.Vlj = acc[PART_V];
-    C.V = acc[PART_V] + ext;
-    C.FR = R.kspring * (xs - xT[0]);
-    C.xS = xs;
-    C.ca = ca; C.cb = cb;
-    for (int a = 0; a < 3; ++a) { C.xT[a] = xT[a]; C.fbody[a] = fb[a]; }
-    // clocks and the rigid body
-    const double h = D.dt;
-    double vb[3] = {S.vbody[0], S.vbody[1], S.vbody[2]};
+    // the rigid body
+    const double kick = rig && a < dim ? 0.5 * h * fb * inr : 0.0;
+    double vb = vb0, vfull = S.vbody_full[a];
     if (mode & MODE_CLOSE) {
-        if (nr > 0)
-            for (int a = 0; a < dim; ++a) vb[a] += 0.5 * h * fb[a] / (double)nr;
-        for (int a = 0; a < 3; ++a) S.vbody_full[a] = vb[a];
+        vb += kick;
+        vfull = vb;
     }
-    for (int a = 0; a < 3; ++a) C.vb_mid[a] = vb[a];
-    C.step_cur = S.step;
-    if (mode & MODE_OPEN) {
-        S.t_h += h * exp(dV / R.kT);
-        S.t_md += h;
-        S.step += 1;
-        S.n_dv[dV <= 0.0 ? 0 : (dV >= R.dvmax ? 2 : 1)] += 1;
-        if (nr > 0)
-            for (int a = 0; a < dim; ++a) vb[a] += 0.5 * h * fb[a] / (double)nr;
+    const double vmid = vb;
+    if (mode & MODE_OPEN) vb += kick;
+    const double v2 = sum3(vfull * vfull);
+    double boost = 1.0;
+    if (mode & MODE_OPEN) boost = dV == 0.0 ? 1.0 : (dV == R.dvmax ? R.boost_max : exp(dV * R.beta));
+    __syncwarp();                       // every lane has read S
+    if (mine) {
+        C.xT[a] = xT;
+        C.fbody[a] = fb;
+        C.vb_mid[a] = vmid;
+        C.vb_new[a] = vb;
+        S.vbody[a] = vb;
+        S.vbody_full[a] = vfull;
     }
-    for (int a = 0; a < 3; ++a) { C.vb_new[a] = vb[a]; S.vbody[a] = vb[a]; }
-    S.K = ksum + 0.5 * (double)nr * (S.vbody_full[0] * S.vbody_full[0] + S.vbody_full[1] * S.vbody_full[1] +
-                                     S.vbody_full[2] * S.vbody_full[2]);
+    if (lane == 0) {
+        C.ce = -dVe;
+        C.dV1 = d1;
+        C.dV2 = d2;
+        C.d = d; C.sigma = sig; C.dV = dV; C.dVp = dVp; C.G = G;
+        C.Vlj = acc[PART_V];
+        C.V = acc[PART_V] + ext;
+        C.FR = k * (xs - xT);
+        C.xS = xs;
+        C.ca = ca; C.cb = cb;
+        C.step_cur = step;
+        if (mode & MODE_OPEN) {
+            // Eq. 3
+            S.t_h += h * boost;
+            S.t_md += h;
+            S.step = step + 1;
+            S.n_dv[dV <= 0.0 ? 0 : (dV >= R.dvmax ? 2 : 1)] += 1;
+        }
+        S.K = ksum + 0.5 * (double)R.nrig * v2;
+    }
+    __syncwarp();
     return true;
 }
 
-// Tile sums of one replica, slot by slot (slot NPART = kinetic parts): for
-// each slot, lane l adds tiles l, l+32, ... in order, then a fixed warp
-// tree; the result does not depend on which warp of which CTA computes it.
+// Sums of one replica's tile parts into acc[0..NPART) and of its kinetic parts
+// into acc[NPART].  A warp reads two parts (256 bytes) at a time, lane l slot
+// l % 16, and every warp takes every nw-th pair, so the loads are coalesced and
+// each lane adds its own slot; the warps' sums meet in shared memory in warp
+// order.  The order is a function of the block size alone.  MAXSLOT is reduced
+// with max (-1: none).
+template <int MAXSLOT>
 __device__ __forceinline__ void dev_scalar_acc(const Dev &D, int r, double *acc) {
+    __shared__ double sm[17][NPART + 1];
     const RepDev &R = D.rep[r];
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int q = w; q <= NPART; q += nw) {
-        double a = 0.0;
-        if (q < NPART) {
-            for (int t = R.tile0 * D.split + lane; t < (R.tile0 + R.ntile) * D.split; t += 32)
-                a += D.part[(size_t)t * NPART + q];
-        } else {
-            for (int t = R.tile0 + lane; t < R.tile0 + R.ntile; t += 32) a += D.kpart[t];
-        }
-        a = warp_sum(a);
-        if (lane == 0) acc[q] = a;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5, slot = lane & 15;
+    const int p0 = R.tile0 * D.split, np = R.ntile * D.split;
+    const bool mx = slot == MAXSLOT;
+    double v = 0.0, k = 0.0;
+    const double *p = D.part + (size_t)p0 * NPART;
+    for (int t = 2 * w + (lane >> 4); t < np; t += 2 * nw) {
+        const double x = p[(size_t)t * NPART + slot];
+        v = mx ? fmax(v, x) : v + x;
+    }
+    const double o = __shfl_down_sync(0xffffffffu, v, 16);
+    v = mx ? fmax(v, o) : v + o;
+    if (MAXSLOT < 0) {
+        for (int t = (int)threadIdx.x; t < R.ntile; t += blockDim.x) k += D.kpart[R.tile0 + t];
+        k = warp_sum(k);
+    }
+    if (lane < NPART) sm[w][lane] = v;
+    if (lane == 0) sm[w][NPART] = k;
+    __syncthreads();
+    if (threadIdx.x <= NPART) {
+        const int q = threadIdx.x;
+        double s = sm[0][q];
+        for (int m = 1; m < nw; ++m) s = q == MAXSLOT ? fmax(s, sm[m][q]) : s + sm[m][q];
+        acc[q] = s;
     }
     __syncthreads();
 }
@@ -1181,23 +1212,26 @@ __device__ void expect_slope(const Dev &D, int r, RepState &S, Scal &C, int list
     if (list && C.need_h) D.h_list[atomicAdd(D.h_meta, 1)] = r;
 }
 
-// blockDim = 32 * (NPART + 1): warp q < NPART sums partial slot q, warp NPART sums K.
-__global__ void k_scalar(Dev D, int mode, int lazy, int list) {
+// threads of a scalar kernel's CTA: what its replica's tile sums can use
+static inline int sc_threads(const Dev &D) { return D.max_parts > 256 ? 512 : 256; }
+constexpr int SC_MAX = 512;
+
+__global__ void __launch_bounds__(SC_MAX) k_scalar(Dev D, int mode, int lazy, int list) {
     const int r = blockIdx.x;
     __shared__ double acc[NPART + 1];
-    dev_scalar_acc(D, r, acc);
-    if (threadIdx.x == 0) {
+    dev_scalar_acc<-1>(D, r, acc);
+    if (threadIdx.x < 32) {
         Scal &C = D.sc[r];
-        if (scalar_eval(D, r, mode, acc, acc[NPART], D.st[r], C, lazy && !C.need_h)) {
-            if (D.lazy_h) expect_slope(D, r, D.st[r], C, list);
-        } else {
-            D.h_late[atomicAdd(D.h_meta + 1, 1)] = r;
-        }
-        // the list (if rebuilt this step) has been used; count displacement-triggered builds
-        const int f = D.rebuild[r];
-        if (f) {
-            if (f == 1) D.st[r].n_rebuild += 1;
-            D.rebuild[r] = 0;
+        const bool done = scalar_eval(D, r, mode, acc, acc[NPART], D.st[r], C, lazy && !C.need_h);
+        if (threadIdx.x == 0) {
+            if (!done) D.h_late[atomicAdd(D.h_meta + 1, 1)] = r;
+            else if (D.lazy_h) expect_slope(D, r, D.st[r], C, list);
+            // the list (if rebuilt this step) has been used; count displacement-triggered builds
+            const int f = D.rebuild[r];
+            if (f) {
+                if (f == 1) D.st[r].n_rebuild += 1;
+                D.rebuild[r] = 0;
+            }
         }
     }
 }
@@ -1212,10 +1246,10 @@ __global__ void __launch_bounds__(256, PREC == HD_FP64 ? 1 : 3) k_scalar_late(De
     __shared__ double acc[NPART + 1];
     for (int q = 0; q < n; ++q) {
         const int r = D.h_late[q];
-        dev_scalar_acc(D, r, acc);
-        if (threadIdx.x == 0) {
+        dev_scalar_acc<-1>(D, r, acc);
+        if (threadIdx.x < 32) {
             scalar_eval(D, r, mode, acc, acc[NPART], D.st[r], D.sc[r]);
-            expect_slope(D, r, D.st[r], D.sc[r], list);
+            if (threadIdx.x == 0) expect_slope(D, r, D.st[r], D.sc[r], list);
         }
         __syncthreads();
     }
@@ -1640,7 +1674,7 @@ __global__ void k_qinit(Dev Q, Dev M) {
 
 // Convergence test and FIRE bookkeeping (reading of Bitzek et al. 2006: mix
 // with the alpha of this step, then grow/shrink dt and alpha).
-__global__ void k_qscalar(Dev D, int max_iter) {
+__global__ void __launch_bounds__(SC_MAX) k_qscalar(Dev D, int max_iter) {
     const int r = blockIdx.x;
     const RepDev &R = D.rep[r];
     RepState &S = D.st[r];
@@ -1649,25 +1683,16 @@ __global__ void k_qscalar(Dev D, int max_iter) {
     __syncthreads();
     if (threadIdx.x == 0) D.rebuild[r] = 0;
     if (S.q_done) return;
-    __shared__ double acc[QPART];
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (w < QPART) {
-        double a = (w == QP_FMAX2) ? 0.0 : 0.0;
-        for (int t = R.tile0 * D.split + lane; t < (R.tile0 + R.ntile) * D.split; t += 32) {
-            const double v = D.part[(size_t)t * NPART + w];
-            a = (w == QP_FMAX2) ? fmax(a, v) : a + v;
-        }
-        a = (w == QP_FMAX2) ? warp_max(a) : warp_sum(a);
-        if (lane == 0) acc[w] = a;
-    }
-    __syncthreads();
+    __shared__ double acc[NPART + 1];
+    dev_scalar_acc<QP_FMAX2>(D, r, acc);
     if (threadIdx.x != 0) return;
+    const double inr = R.inv_nrig;
     const int nr = R.nrig, dim = R.dim;
     double fb[3] = {0, 0, 0};
     double fm2 = acc[QP_FMAX2];
     if (nr > 0) {
         double xT[3], gs[3] = {0, 0, 0};
-        for (int a = 0; a < 3; ++a) xT[a] = acc[QP_XRIG + a] / (double)nr;
+        for (int a = 0; a < 3; ++a) xT[a] = acc[QP_XRIG + a] * inr;
         gs[0] = R.kspring * (xT[0] - slider_x(R, S.step, D.dt));   // the slider stands still during a quench
         if (dim == 3) gs[1] = R.kspring * (xT[1] - R.slider[1]);
         gs[R.vert] = R.fnormal;
@@ -1698,16 +1723,16 @@ __global__ void k_qscalar(Dev D, int max_iter) {
             for (int a = 0; a < dim; ++a) {
                 pw += fb[a] * S.q_vb[a];
                 vv += (double)nr * S.q_vb[a] * S.q_vb[a];
-                ff += fb[a] * fb[a] / (double)nr;
+                ff += fb[a] * fb[a] * inr;
             }
         double alpha = S.q_alpha, dt = S.q_dt;
         double vb[3] = {S.q_vb[0], S.q_vb[1], S.q_vb[2]};
         if (pw > 0.0) {
-            const double mix = ff > 0.0 ? alpha * sqrt(vv) / sqrt(ff) : 0.0;
+            const double mix = ff > 0.0 ? alpha * sqrt(vv / ff) : 0.0;
             C.q_mix = mix;
             C.q_zero = 0;
             if (nr > 0)
-                for (int a = 0; a < dim; ++a) vb[a] = (1.0 - alpha) * vb[a] + mix * fb[a] / (double)nr;
+                for (int a = 0; a < dim; ++a) vb[a] = (1.0 - alpha) * vb[a] + mix * fb[a] * inr;
             S.q_npos += 1;
             if (S.q_npos > 5) {
                 dt = dt * 1.1 < 10.0 * D.q_step ? dt * 1.1 : 10.0 * D.q_step;
@@ -1726,7 +1751,7 @@ __global__ void k_qscalar(Dev D, int max_iter) {
         S.q_alpha = alpha;
         S.q_dt = dt;
         if (nr > 0)
-            for (int a = 0; a < dim; ++a) vb[a] += dt * fb[a] / (double)nr;
+            for (int a = 0; a < dim; ++a) vb[a] += dt * fb[a] * inr;
         for (int a = 0; a < 3; ++a) { S.q_vb[a] = vb[a]; C.q_vb[a] = vb[a]; }
     }
     S.q_iter += 1;
@@ -1954,9 +1979,9 @@ __global__ void __launch_bounds__(128, 4) k_persist(Dev D, int nsteps) {
     __syncthreads();
     unsigned epoch = 0;
     auto scalars = [&](int mode) {
-        dev_scalar_acc(D, r, acc);
+        dev_scalar_acc<-1>(D, r, acc);
+        if (threadIdx.x < 32) scalar_eval(D, r, mode, acc, acc[NPART], S, C);
         if (threadIdx.x == 0) {
-            scalar_eval(D, r, mode, acc, acc[NPART], S, C);
             if (leader) {
                 D.st[r] = S;
                 D.sc[r] = C;
@@ -1973,7 +1998,7 @@ __global__ void __launch_bounds__(128, 4) k_persist(Dev D, int nsteps) {
     // the chain between the kicks (every CTA evaluates it alike from the
     // replica's kinetic sums)
     auto chain = [&](int mode) {
-        dev_scalar_acc(D, r, acc);
+        dev_scalar_acc<-1>(D, r, acc);
         if (threadIdx.x == 0) {
             nhc_eval(D, r, mode, acc[NPART], S, C);
             if (leader) {
@@ -2106,7 +2131,7 @@ void launch_pair(const Dev &D, int kind, cudaStream_t s) {
 }
 void launch_scalar(const Dev &D, int mode, bool lazy, bool list, cudaStream_t s) {
     const bool more = D.lazy_h && D.bias_on;
-    k_scalar<<<D.nrep, 32 * (NPART + 1), 0, s>>>(D, mode, lazy && more, list && more);
+    k_scalar<<<D.nrep, sc_threads(D), 0, s>>>(D, mode, lazy && more, list && more);
     if (!lazy || !more) return;
     const int n = nthr(D), g = D.hot_grid, li = list && more;
     if (D.prec == HD_FP64) {
@@ -2127,7 +2152,7 @@ void launch_qinit(const Dev &Q, const Dev &M, cudaStream_t s) { k_qinit<<<Q.ntil
 void launch_qiter(const Dev &Q, int max_iter, cudaStream_t s) {
     launch_rebuild(Q, s);
     launch_pair(Q, PAIR_QUENCH, s);
-    k_qscalar<<<Q.nrep, 32 * QPART, 0, s>>>(Q, max_iter);
+    k_qscalar<<<Q.nrep, sc_threads(Q), 0, s>>>(Q, max_iter);
     k_qupdate<<<Q.ntile, nthr(Q), 0, s>>>(Q);
 }
 void launch_qdisp(const Dev &Q, cudaStream_t s) { k_qdisp<<<Q.ntile, nthr(Q), 0, s>>>(Q); }
