@@ -8,9 +8,12 @@
 namespace hd {
 
 void launch_init(const Dev &D, const int *draw_vel, cudaStream_t s);
-void launch_rebuild(const Dev &D, cudaStream_t s);            // 5 kernels, flag-gated per replica
-void launch_rebuild_prep(const Dev &D, cudaStream_t s);       // the first 4: plan, clear, bin, cell sort
-void launch_nlist(const Dev &D, cudaStream_t s);              // the 5th: rows from the cells
+// replicas whose rebuild plan each CTA of the binning makes in its shared memory; with
+// more of them a kernel of its own makes it first
+constexpr int PLAN_MAX = 4000;
+void launch_rebuild(const Dev &D, cudaStream_t s);            // 3 kernels, flag-gated per replica
+void launch_rebuild_prep(const Dev &D, cudaStream_t s);       // the first 2: plan and bin, cell sort
+void launch_nlist(const Dev &D, cudaStream_t s);              // the 3rd: rows from the cells
 // FULL: force and H.(r - r_O); ENERGY: per-atom LJ energies too (observables, not
 // needed by the dynamics); LAZY: H.(r - r_O) for the replicas expected in their band
 enum { PAIR_FULL = 0, PAIR_ENERGY = 1, PAIR_LAZY = 2, PAIR_QUENCH = 3 };
@@ -22,7 +25,7 @@ void launch_obs(const Dev &D, cudaStream_t s);
 void launch_nhc(const Dev &D, int mode, cudaStream_t s);          // the chain between two kicks, per replica
 void launch_eig(const Dev &D, cudaStream_t s);                    // epsilon (Lanczos) and grad epsilon (hd_eig.cu)
 void launch_qinit(const Dev &Q, const Dev &M, cudaStream_t s);
-void launch_qiter(const Dev &Q, int max_iter, cudaStream_t s);  // 8 kernels
+void launch_qiter(const Dev &Q, int max_iter, cudaStream_t s);  // 6 kernels
 void launch_qdisp(const Dev &Q, cudaStream_t s);
 void launch_adopt(const Dev &Q, const Dev &M, const int *adopt, cudaStream_t s);
 size_t nl_smem_bytes(const Dev &D, int nwarps);                  // dynamic shared memory of the list build
