@@ -1927,18 +1927,36 @@ __global__ void __launch_bounds__(256) k_qupdate(Dev D) {
 // Largest displacement of the quenched copy from r_O per replica (minimum
 // image, FP64, the oracle's operation order); stored as the bits of the
 // non-negative double so that an integer max is the FP64 max.
-__global__ void k_qdisp(Dev Q) {
+// One atomic per CTA: with one per atom the 14,272 of a replica ran one after
+// another (508 us for 64 of them).  Below half a box the nearest integer to
+// d / L is 0 and the division, which the FP64 pipe takes ten instructions for,
+// is left out.
+__global__ void __launch_bounds__(256) k_qdisp(Dev Q) {
+    __shared__ unsigned long long most;
     const int t = blockIdx.x, r = Q.tile_rep[t];
-    if (threadIdx.x >= Q.tile_n[t]) return;
-    const int i = Q.tile_start[t] + threadIdx.x;
-    const RepDev &R = Q.rep[r];
-    const dbl4 a = Q.x[i], b = Q.xo[i];
-    double d0 = a.x - b.x, d1 = a.y - b.y, d2 = a.z - b.z;
-    if (R.periodic[0]) d0 = __dsub_rn(d0, __dmul_rn(R.L[0], rint(__ddiv_rn(d0, R.L[0]))));
-    if (R.periodic[1]) d1 = __dsub_rn(d1, __dmul_rn(R.L[1], rint(__ddiv_rn(d1, R.L[1]))));
-    if (R.periodic[2]) d2 = __dsub_rn(d2, __dmul_rn(R.L[2], rint(__ddiv_rn(d2, R.L[2]))));
-    const double m = __dadd_rn(__dadd_rn(__dmul_rn(d0, d0), __dmul_rn(d1, d1)), __dmul_rn(d2, d2));
-    atomicMax(Q.qdisp + r, (unsigned long long)__double_as_longlong(m));
+    if (threadIdx.x == 0) most = 0ull;
+    __syncthreads();
+    unsigned long long bits = 0ull;
+    if (threadIdx.x < Q.tile_n[t]) {
+        const int i = Q.tile_start[t] + threadIdx.x;
+        const RepDev &R = Q.rep[r];
+        const dbl4 a = Q.x[i], b = Q.xo[i];
+        auto image = [&](int ax, double d) {
+            if (!R.periodic[ax] || fabs(d) < 0.499 * R.L[ax]) return d;
+            return __dsub_rn(d, __dmul_rn(R.L[ax], rint(__ddiv_rn(d, R.L[ax]))));
+        };
+        const double d0 = image(0, a.x - b.x), d1 = image(1, a.y - b.y), d2 = image(2, a.z - b.z);
+        const double m = __dadd_rn(__dadd_rn(__dmul_rn(d0, d0), __dmul_rn(d1, d1)), __dmul_rn(d2, d2));
+        bits = (unsigned long long)__double_as_longlong(m);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long u = __shfl_xor_sync(0xffffffffu, bits, o);
+        bits = u > bits ? u : bits;
+    }
+    if ((threadIdx.x & 31) == 0) atomicMax(&most, bits);
+    __syncthreads();
+    if (threadIdx.x == 0) atomicMax(Q.qdisp + r, most);
 }
 
 // r_O <- quenched copy for replicas with adopt[r] != 0; refresh r - r_O.
