@@ -24,7 +24,7 @@ constexpr size_t ALIGN = 256;
 
 struct Plan {
     int nrep = 0, natom = 0, ntile = 0, maxnb = 0, cell_cap = 0, ncell = 0, block = 128, prec = 0;
-    int nwg = 0, split = 1;
+    int nwg = 0, lanes = 1, split = 1;
     std::vector<RepDev> rep;
     std::vector<int> tile_rep, tile_start, tile_n;
     // storage order: atoms of a replica are held cell-major (cells of the
@@ -381,7 +381,15 @@ bool make_plan(const hd_replica_desc *reps, int n_rep, const hd_params *p, Plan 
     // atoms: 34.5 us a sweep with 1, 20.9 with 4; 8 x 113 atoms, FP64, one
     // launch: 66.6 and 47.7 us a step); beyond that the split only adds work
     // (57,088 atoms FP64: 513 us with 1, 570 with 4).
-    P.split = P.natom / 32 < 152 * 8 ? 4 : 1;
+    P.lanes = P.split = P.natom / 32 < 152 * 8 ? 4 : 1;
+    // The persistent launch cuts tiles into smaller units while SMs are idle:
+    // 8 atoms (one warp) up to 4,864 atoms, 16 up to 9,728 (4 CTAs an SM).
+    if (p->driver == HD_DRIVER_PERSISTENT && P.lanes == 4)
+        for (int w = 8; w <= 16; w *= 2)
+            if (P.block % w == 0 && P.block / w > P.split && P.natom <= 608 * w) {
+                P.split = P.block / w;
+                break;
+            }
     // layout
     const size_t N = P.natom, T = P.ntile, R = P.nrep;
     const size_t v4 = P.prec == HD_FP64 ? sizeof(dbl4) : sizeof(float4);
@@ -394,7 +402,7 @@ bool make_plan(const hd_replica_desc *reps, int n_rep, const hd_params *p, Plan 
     P.o_tn = take(cur, T * 4);
     P.o_part = take(cur, T * P.split * NPART * 8);
     P.o_qpart = take(cur, T * P.split * NPART * 8);
-    P.o_kpart = take(cur, T * 8);
+    P.o_kpart = take(cur, T * P.split * 8);
     P.o_x = take(cur, N * sizeof(dbl4));
     P.o_xo = take(cur, N * sizeof(dbl4));
     P.o_xq = take(cur, N * sizeof(dbl4));
@@ -592,7 +600,9 @@ void fill_dev(hd_ctx *c) {
     D.prec = P.prec;
     D.block = P.block;
     D.ngrp = (P.maxnb + 3) / 4;
+    D.lanes = P.lanes;
     D.split = P.split;
+    D.ksplit = 1;
     D.rep = at<RepDev>(b, P.o_rep);
     D.st = at<RepState>(b, P.o_st);
     D.sc = at<Scal>(b, P.o_sc);
@@ -658,7 +668,7 @@ void fill_dev(hd_ctx *c) {
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
         D.nl_grid = nsm * 4;
-        D.hot_grid = std::min(P.ntile * P.split, nsm * std::max(1, 768 / P.block));   // what is resident at once
+        D.hot_grid = std::min(P.ntile * P.split, nsm * std::max(1, 768 / (P.block / P.split * P.lanes)));   // what is resident at once
     }
     // quench view: the copy of the positions and its own velocity, force,
     // fixed-point image, rebuild flags and tile sums
@@ -983,6 +993,10 @@ hd_status hd_create(const hd_replica_desc *reps, int n_rep, const hd_params *p, 
     int *d_draw = at<int>(c->ws, P.o_drawvel);
     CK(cudaMemcpyAsync(d_draw, draw.data(), P.nrep * 4, cudaMemcpyHostToDevice, c->s));
     CK(cudaMemcpyAsync(c->D.rebuild, two.data(), P.nrep * 4, cudaMemcpyHostToDevice, c->s));
+    if (p->driver == HD_DRIVER_PERSISTENT && setup_persistent(c)) {
+        c->driver = HD_DRIVER_PERSISTENT;
+        c->D.ksplit = c->Q.ksplit = P.split;
+    }
     launch_init(c->D, d_draw, c->s);
     launch_rebuild(c->D, c->s);
     launch_pair(c->D, PAIR_ENERGY, c->s);
@@ -998,7 +1012,6 @@ hd_status hd_create(const hd_replica_desc *reps, int n_rep, const hd_params *p, 
     c->qconv.assign(P.nrep, 0);
     c->step0.resize(P.nrep);
     for (int r = 0; r < P.nrep; ++r) c->step0[r] = reps[r].step0;
-    if (p->driver == HD_DRIVER_PERSISTENT && setup_persistent(c)) c->driver = HD_DRIVER_PERSISTENT;
     return check_device(c);
 }
 

@@ -149,7 +149,9 @@ struct Scal {
 struct Dev {
     int nrep, ntile, natom, maxnb, cell_cap, ncell, prec, bias_on, block;
     int max_parts;               // largest number of tile parts of one replica
-    int ngrp, split;             // groups of four per list row; lanes that share a row of the pair sweep (1 or 4)
+    int ngrp;                    // groups of four per list row
+    int lanes, split;            // lanes that share a row of the pair sweep (1 or 4); units a tile is cut into
+    int ksplit;                  // slots of the kinetic sums per tile (split in the persistent driver, else 1)
     int q_method, max_cells;        // max_cells: largest cell count of one replica
     double dt, rc2, rl2, half_skin2, q_ftol, q_step, q_theta;
     double q_ftol_stay, q_keep2;    // quench: early stop inside the basin (0: off), (theta/2)^2
@@ -170,7 +172,7 @@ struct Dev {
     int *cellid, *nnb, *nbr, *cell_cnt, *cell_atoms;
     int *rebuild;                // per replica: list rebuild requested
     int *err;                    // [0] first error code, [1] atom, [2] replica
-    unsigned int *bar;           // per replica barrier counters (persistent driver)
+    unsigned int *bar;           // per replica 64-bit barrier counters (persistent driver)
     unsigned long long *qdisp;   // per replica max |x_q - r_O|^2 (bits of the double)
     unsigned long long *qgate;   // per replica max |x_q - r_O|^2 of the current quench iterate
     const int *orig;             // per slot: index of the atom in its replica's input

@@ -218,12 +218,6 @@ __device__ __forceinline__ void dev_bin_atom(const Dev &D, int r, int i) {
     else set_err(D, HD_ERR_OVERFLOW, i, r);
     D.pfixb[i] = p;
 }
-// tile form, for the persistent driver (which rebuilds one replica at a time)
-__device__ __forceinline__ void dev_bin(const Dev &D, int t) {
-    const int r = D.tile_rep[t];
-    if (!D.rebuild[r] || threadIdx.x >= D.tile_n[t]) return;
-    dev_bin_atom(D, r, D.tile_start[t] + threadIdx.x);
-}
 // planned: the plan is in global memory already (k_rebuild_plan, for batches
 // whose plan does not fit a CTA's shared memory).
 __global__ void __launch_bounds__(256) k_bin(Dev D, bool planned) {
@@ -593,16 +587,16 @@ __global__ void __launch_bounds__(NL_THREADS) k_nlist(Dev D) {
 // Q (quench): positions of the quench copy, quench partial sums.  E: per-atom
 // energies.  H: the Hessian term.
 // S: lanes of a warp that share one row (lane s takes groups s, s + S, ... of
-// four entries, the sums meet in a shuffle tree); a CTA then holds block / S
-// atoms of its tile and `unit` counts such parts.
+// four entries, the sums meet in a shuffle tree).  A tile is cut into D.split
+// units of block / split atoms, one CTA each, of S threads an atom.
 template <bool Q, bool E, bool H, int S>
 __device__ __forceinline__ void dev_pair64(const Dev &D, int unit) {
-    const int t = unit / S;
+    const int t = unit / D.split;
     const int r = D.tile_rep[t];
     if (Q && D.st[r].q_done) return;
     const RepDev &R = D.rep[r];
     const int sub = S > 1 ? (int)(threadIdx.x % S) : 0;
-    const int at = (unit % S) * (D.block / S) + (int)threadIdx.x / S;     // atom of the tile
+    const int at = (unit % D.split) * (D.block / D.split) + (int)threadIdx.x / S;     // atom of the tile
     const bool has = at < D.tile_n[t], act = has && sub == 0;
     const int i = D.tile_start[t] + (has ? at : 0);
     const dbl4 xi = D.x[i];
@@ -761,16 +755,15 @@ __device__ __forceinline__ float rcp_refined(float x) {
     return fmaf(y, fmaf(-x, y, 1.f), y);
 }
 
-// Split rows: S lanes of a warp share one row (lane s takes groups s, s + S,
-// ... of four entries) and a CTA holds block / S atoms.  See dev_pair32.
+// S, unit: as in dev_pair64.
 template <bool Q, bool E, bool H, int S>
 __device__ __forceinline__ void dev_pair32(const Dev &D, int unit) {
-    const int t = unit / S;
+    const int t = unit / D.split;
     const int r = D.tile_rep[t];
     if (Q && D.st[r].q_done) return;
     const RepDev &R = D.rep[r];
     const int sub = S > 1 ? (int)(threadIdx.x % S) : 0;
-    const int at = (unit % S) * (D.block / S) + (int)threadIdx.x / S;     // atom of the tile
+    const int at = (unit % D.split) * (D.block / D.split) + (int)threadIdx.x / S;     // atom of the tile
     const bool act = at < D.tile_n[t];
     const int i = D.tile_start[t] + (act ? at : 0);
     const int4 pi = D.p[i];
@@ -1027,12 +1020,12 @@ enum { SWEEP_ALL = 0, SWEEP_PLAIN = 1 };
 
 template <bool Q, bool E, bool H, int S>
 __global__ void __launch_bounds__(256) k_pair64(Dev D, int sweep) {
-    if (sweep == SWEEP_PLAIN && D.sc[D.tile_rep[blockIdx.x / S]].need_h) return;
+    if (sweep == SWEEP_PLAIN && D.sc[D.tile_rep[blockIdx.x / D.split]].need_h) return;
     dev_pair64<Q, E, H, S>(D, blockIdx.x);
 }
 template <bool Q, bool E, bool H, int S>
 __global__ void __launch_bounds__(256, H ? 3 : 4) k_pair32(Dev D, int sweep) {
-    if (sweep == SWEEP_PLAIN && D.sc[D.tile_rep[blockIdx.x / S]].need_h) return;
+    if (sweep == SWEEP_PLAIN && D.sc[D.tile_rep[blockIdx.x / D.split]].need_h) return;
     dev_pair32<Q, E, H, S>(D, blockIdx.x);
 }
 
@@ -1045,7 +1038,7 @@ __device__ __forceinline__ bool sweep_listed(const Dev &D, const int *list, int 
     int pos = blockIdx.x, base = 0;       // place in the listed replicas' tiles, one after another
     for (int q = 0; q < n; ++q) {
         const RepDev &R = D.rep[list[q]];
-        const int t0 = R.tile0 * S, nt = R.ntile * S;
+        const int t0 = R.tile0 * D.split, nt = R.ntile * D.split;
         for (; pos < base + nt; pos += gridDim.x) {
             if (PREC == HD_FP64) dev_pair64<false, false, true, S>(D, t0 + pos - base);
             else dev_pair32<false, false, true, S>(D, t0 + pos - base);
@@ -1205,14 +1198,21 @@ __device__ __forceinline__ void dev_scalar_acc(const Dev &D, int r, double *acc)
     const bool mx = slot == MAXSLOT;
     double v = 0.0, k = 0.0;
     const double *p = D.part + (size_t)p0 * NPART;
-    for (int t = 2 * w + (lane >> 4); t < np; t += 2 * nw) {
-        const double x = p[(size_t)t * NPART + slot];
-        v = mx ? fmax(v, x) : v + x;
+    // eight loads in flight: a warp alone (the smallest units) would wait for each
+    for (int t = 2 * w + (lane >> 4); t < np; t += 16 * nw) {
+        double x[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) x[u] = t + 2 * nw * u < np ? p[(size_t)(t + 2 * nw * u) * NPART + slot] : 0.0;
+#pragma unroll
+        for (int h = 4; h > 0; h >>= 1)
+#pragma unroll
+            for (int u = 0; u < h; ++u) x[u] = mx ? fmax(x[u], x[u + h]) : x[u] + x[u + h];
+        v = mx ? fmax(v, x[0]) : v + x[0];
     }
     const double o = __shfl_down_sync(0xffffffffu, v, 16);
     v = mx ? fmax(v, o) : v + o;
     if (MAXSLOT < 0) {
-        for (int t = (int)threadIdx.x; t < R.ntile; t += blockDim.x) k += D.kpart[R.tile0 + t];
+        for (int t = (int)threadIdx.x; t < R.ntile * D.ksplit; t += blockDim.x) k += D.kpart[R.tile0 * D.ksplit + t];
         k = warp_sum(k);
     }
     if (lane < NPART) sm[w][lane] = v;
@@ -1302,7 +1302,7 @@ __global__ void k_obs(Dev D) {
     const RepDev &R = D.rep[r];
     RepState &S = D.st[r];
     double a = 0.0;
-    for (int t = R.tile0 + (int)threadIdx.x; t < R.tile0 + R.ntile; t += 32) a += D.kpart[t];
+    for (int t = (int)threadIdx.x; t < R.ntile * D.ksplit; t += 32) a += D.kpart[R.tile0 * D.ksplit + t];
     a = warp_sum(a);
     if (threadIdx.x == 0)
         S.K = a + 0.5 * (double)R.nrig * (S.vbody_full[0] * S.vbody_full[0] + S.vbody_full[1] * S.vbody_full[1] +
@@ -1367,7 +1367,7 @@ __global__ void k_nhc(Dev D, int mode) {
     const int r = blockIdx.x;
     const RepDev &R = D.rep[r];
     double a = 0.0;
-    for (int t = R.tile0 + (int)threadIdx.x; t < R.tile0 + R.ntile; t += 32) a += D.kpart[t];
+    for (int t = (int)threadIdx.x; t < R.ntile * D.ksplit; t += 32) a += D.kpart[R.tile0 * D.ksplit + t];
     a = warp_sum(a);
     if (threadIdx.x == 0) nhc_eval(D, r, mode, a, D.st[r], D.sc[r]);
 }
@@ -1377,14 +1377,14 @@ __global__ void k_nhc(Dev D, int mode) {
 //   CLOSE: v += dt/2 F_tot                      (end of the previous step)
 //   OPEN:  v += dt/2 F_tot; x += dt/2 v; v = c v + s xi; x += dt/2 v
 // Mobile atoms only; rigid atoms follow the body velocity; fixed atoms stay.
-__device__ __forceinline__ int4 post_move(const Dev &D, const RepDev &R, int r, int i, dbl4 x, int4 p) {
+__device__ __forceinline__ int4 post_move(const Dev &D, const RepDev &R, int r, int i, dbl4 x, int4 p, int *moved) {
     const int4 q = fix_pos(R, x, p.w);
     D.p[i] = q;
     const int4 b = D.pfixb[i];
     const float ex = (float)(int)((unsigned)q.x - (unsigned)b.x) * R.fx_lsb[0];
     const float ey = (float)(int)((unsigned)q.y - (unsigned)b.y) * R.fx_lsb[1];
     const float ez = (float)(int)((unsigned)q.z - (unsigned)b.z) * R.fx_lsb[2];
-    if (ex * ex + ey * ey + ez * ez > D.half_skin2_f) D.rebuild[r] = 1;
+    if (ex * ex + ey * ey + ez * ez > D.half_skin2_f) *moved = 1;
     const double zv = R.vert == 2 ? x.z : x.y;
     if (!(fabs(zv - R.fx_origin[R.vert]) < R.open_lim) || !isfinite(x.x) || !isfinite(x.y) || !isfinite(x.z))
         set_err(D, HD_ERR_NUMERIC, i, r);
@@ -1395,7 +1395,7 @@ __device__ __forceinline__ int4 post_move(const Dev &D, const RepDev &R, int r, 
 // r - r_O (the difference of the images of r and r_O) has not wrapped.  It
 // wraps at L / 2^(k+1) >= 4 (rc + skin); an atom is reported (HD_ERR_NUMERIC)
 // when it has moved 3/4 of that from its r_O.
-__device__ __forceinline__ void post_move32(const Dev &D, const RepDev &R, int r, int i, dbl4 x, int4 p) {
+__device__ __forceinline__ void post_move32(const Dev &D, const RepDev &R, int r, int i, dbl4 x, int4 p, int *moved) {
     const int4 q = fix_pos(R, x, p.w);
     const int4 d = img_diff(q, D.po[i]);
     D.p[i] = q;
@@ -1403,7 +1403,7 @@ __device__ __forceinline__ void post_move32(const Dev &D, const RepDev &R, int r
     const float ex = (float)(int)((unsigned)q.x - (unsigned)b.x) * R.fx_lsb[0];
     const float ey = (float)(int)((unsigned)q.y - (unsigned)b.y) * R.fx_lsb[1];
     const float ez = (float)(int)((unsigned)q.z - (unsigned)b.z) * R.fx_lsb[2];
-    if (ex * ex + ey * ey + ez * ez > D.half_skin2_f) D.rebuild[r] = 1;
+    if (ex * ex + ey * ey + ez * ez > D.half_skin2_f) *moved = 1;
     const double zv = R.vert == 2 ? x.z : x.y;
     const int lim = 3 << 29;
     if (!(fabs(zv - R.fx_origin[R.vert]) < R.open_lim) || !isfinite(x.x) || !isfinite(x.y) || !isfinite(x.z) ||
@@ -1411,11 +1411,28 @@ __device__ __forceinline__ void post_move32(const Dev &D, const RepDev &R, int r
         set_err(D, HD_ERR_NUMERIC, i, r);
 }
 
-__device__ __forceinline__ void dev_update64(const Dev &D, int t, int mode, const Scal &C) {
+// The atoms a CTA updates: a tile of the per-phase kernels; a unit of the
+// persistent launch (block / split atoms, with more threads than that), whose
+// kinetic sum has its own slot.  *moved is set where an atom has moved half the
+// skin since the last list build: the replica's flag, or the CTA's own.
+struct UpdateSpan {
+    int t, first, n, slot, r;
+    int *moved;
+};
+__device__ __forceinline__ UpdateSpan update_tile(const Dev &D, int t) {
     const int r = D.tile_rep[t];
+    return {t, D.tile_start[t], D.tile_n[t], t * D.ksplit, r, D.rebuild + r};
+}
+__device__ __forceinline__ UpdateSpan update_unit(const Dev &D, int unit, int *moved) {
+    const int t = unit / D.split, w = D.block / D.split, o = (unit % D.split) * w;
+    return {t, D.tile_start[t] + o, min(w, max(0, D.tile_n[t] - o)), unit, D.tile_rep[t], moved};
+}
+
+__device__ __forceinline__ void dev_update64(const Dev &D, const UpdateSpan &U, int mode, const Scal &C) {
+    const int r = U.r;
     const RepDev &R = D.rep[r];
-    const bool act = threadIdx.x < D.tile_n[t];
-    const int i = D.tile_start[t] + (act ? threadIdx.x : 0);
+    const bool act = (int)threadIdx.x < U.n;
+    const int i = U.first + (act ? threadIdx.x : 0);
     const int4 p = D.p[i];
     const int role = act ? ((p.w >> 8) & 0xff) : ROLE_FIXED;
     double kin = 0.0;
@@ -1494,24 +1511,24 @@ __device__ __forceinline__ void dev_update64(const Dev &D, int t, int mode, cons
             D.x[i] = x;
             const dbl4 xo = D.xo[i];
             D.dr64[i] = make_dbl4(x.x - xo.x, x.y - xo.y, x.z - xo.z, 0.0);
-            post_move(D, R, r, i, x, p);
+            post_move(D, R, r, i, x, p, U.moved);
         }
     }
     if (mode & (MODE_CLOSE | MODE_KIN | MODE_SCALE)) {
         double v1[1] = {kin};
-        cta_reduce<1>(v1, D.kpart + t, -1);
+        cta_reduce<1>(v1, D.kpart + U.slot, -1);
     }
 }
 
-__device__ __forceinline__ void dev_update32(const Dev &D, int t, int mode, const Scal &C) {
+__device__ __forceinline__ void dev_update32(const Dev &D, const UpdateSpan &U, int mode, const Scal &C) {
     // split form: FP32 forces, FP64 velocities and positions (FP32 velocities
     // would round every kick and thermostat step at 2^-24 of |v|, which after
     // 100 steps puts sigma and the boosted clock beyond 1e-6 of FP64); r - r_O
     // from the fixed-point images of r and r_O
-    const int r = D.tile_rep[t];
+    const int r = U.r;
     const RepDev &R = D.rep[r];
-    const bool act = threadIdx.x < D.tile_n[t];
-    const int i = D.tile_start[t] + (act ? threadIdx.x : 0);
+    const bool act = (int)threadIdx.x < U.n;
+    const int i = U.first + (act ? threadIdx.x : 0);
     const int4 p = D.p[i];
     const int role = act ? ((p.w >> 8) & 0xff) : ROLE_FIXED;
     // the closing half kick of one step and the opening one of the next see
@@ -1604,21 +1621,20 @@ __device__ __forceinline__ void dev_update32(const Dev &D, int t, int mode, cons
         D.v64[i] = v;
         if (mode & MODE_OPEN) {
             D.x[i] = x;
-            post_move32(D, R, r, i, x, p);
+            post_move32(D, R, r, i, x, p, U.moved);
         }
     }
     if ((mode & (MODE_CLOSE | MODE_KIN | MODE_SCALE)) && !fused) {
-        double v1[1] = {(double)warp_sum(kin)};
-        if ((threadIdx.x & 31) != 0) v1[0] = 0.0;
-        cta_reduce<1>(v1, D.kpart + t, -1);
+        double v1[1] = {(double)kin};    // FP64 sums: how atoms share warps must not show in K
+        cta_reduce<1>(v1, D.kpart + U.slot, -1);
     }
 }
 
 __global__ void __launch_bounds__(256) k_update64(Dev D, int mode) {
-    dev_update64(D, blockIdx.x, mode, D.sc[D.tile_rep[blockIdx.x]]);
+    dev_update64(D, update_tile(D, blockIdx.x), mode, D.sc[D.tile_rep[blockIdx.x]]);
 }
 __global__ void __launch_bounds__(256) k_update32(Dev D, int mode) {
-    dev_update32(D, blockIdx.x, mode, D.sc[D.tile_rep[blockIdx.x]]);
+    dev_update32(D, update_tile(D, blockIdx.x), mode, D.sc[D.tile_rep[blockIdx.x]]);
 }
 
 // ---------------------------------------------------------------- quench
@@ -1843,7 +1859,7 @@ __device__ __forceinline__ dbl4 qmove(const Dev &D, const RepDev &R, const Scal 
         }
     }
     D.x[i] = x;
-    *img = post_move(D, R, r, i, x, p);
+    *img = post_move(D, R, r, i, x, p, D.rebuild + r);
     return x;
 }
 
@@ -1882,7 +1898,7 @@ __device__ __forceinline__ int4 qmove32(const Dev &D, const RepDev &R, const Sca
         if (three) x.z += C.q_dt * C.q_vb[2];
     }
     D.x[i] = x;
-    return post_move(D, R, r, i, x, p);
+    return post_move(D, R, r, i, x, p, D.rebuild + r);
 }
 
 __global__ void __launch_bounds__(256) k_qupdate(Dev D) {
@@ -1973,96 +1989,117 @@ __global__ void k_adopt(Dev Q, Dev M, const int *adopt) {
 
 // ---------------------------------------------------------------- persistent driver
 // One launch steps every replica n times.  Replica r owns CTAs
-// [pg_first[r], pg_first[r] + pg_count[r]); each CTA takes the replica's
-// tiles round robin and runs the same per-tile phases as the per-phase
+// [pg_first[r], pg_first[r] + pg_count[r]); each takes the replica's units
+// (see dev_pair64) round robin and runs the same phases as the per-phase
 // kernels; the compiler may contract multiply-adds differently where a phase
-// is inlined here, so the two drivers agree to rounding.  Phases of one
-// replica are separated by that replica's own barrier: a counter in global
-// memory (reset before each launch) that CTAs increment and poll.  Polling
-// is bounded: after ~2^24 polls the CTA records HD_ERR_TIMEOUT, raises the
-// abort word err[3], and every CTA leaves at its next barrier.  The launch
-// is cooperative, so all CTAs are resident.  A one-CTA replica uses only
-// __syncthreads().
-__device__ __forceinline__ bool grp_barrier(const Dev &D, int r, int nc, unsigned &epoch) {
+// is inlined here, so the two drivers agree to rounding.
+//
+// Small replicas are what this driver is for, and a step of theirs is latency:
+// two barriers, the sweep of a row, the scalars and the update.  So a unit is
+// small (8 atoms where the batch leaves SMs idle: an FP64 sweep is bound by
+// the FP64 pipe of the SMs it is on), a CTA updates the atoms it sweeps, states
+// go to global memory at the end of the call only, and a barrier carries the
+// flag that a list is due.  Against a tile's threads, separate flags and
+// fences a step of 16 x 421 atoms takes 16.2 us in place of 18.7, of 8 x 113 in
+// the FP64 form 33.2 in place of 36.5.
+//
+// Phases of one replica are separated by that replica's own barrier: a 64-bit
+// counter in global memory (reset before each launch) whose low half counts
+// arrivals and whose high half counts CTAs that saw an atom move half the skin
+// in the update before.  An arrival releases the CTA's writes, the poll
+// acquires the others'.  Polling is bounded: after ~2^24 polls the CTA records
+// HD_ERR_TIMEOUT, raises the abort word err[3], and every CTA leaves at its
+// next barrier.  The launch is cooperative, so all CTAs are resident.  A
+// one-CTA replica uses only __syncthreads().
+struct GrpBar {
+    unsigned epoch, moved;       // barriers passed; high half of the counter at the last one
+    bool due;                    // a CTA arrived with `moved` since then
+};
+__device__ __forceinline__ bool grp_barrier(const Dev &D, int r, int nc, GrpBar &B, int *s_moved) {
     __shared__ int s_ok;
+    __shared__ unsigned s_hi;
     __syncthreads();
-    if (nc > 1) {
-        if (threadIdx.x == 0) {
-            int ok = 1;
-            __threadfence();
-            const unsigned target = (epoch + 1u) * (unsigned)nc;
+    if (threadIdx.x == 0) {
+        int ok = 1;
+        const unsigned mine = s_moved && *s_moved ? 1u : 0u;
+        unsigned hi = B.moved + mine;
+        if (s_moved) *s_moved = 0;
+        if (nc > 1) {
+            unsigned long long *ctr = reinterpret_cast<unsigned long long *>(D.bar) + r;
+            const unsigned target = (B.epoch + 1u) * (unsigned)nc;
             // test hook: one CTA of replica fault_rep skips its first arrival
-            const bool skip = D.fault_rep == r && epoch == 0 && blockIdx.x == (unsigned)D.pg_first[r];
-            if (!skip) atomicAdd(D.bar + r, 1u);
+            const bool skip = D.fault_rep == r && B.epoch == 0 && blockIdx.x == (unsigned)D.pg_first[r];
+            const unsigned long long add = ((unsigned long long)mine << 32) | 1ull;
+            if (!skip) asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(ctr), "l"(add) : "memory");
             unsigned polls = 0;
-            while (*((volatile unsigned *)(D.bar + r)) < target) {
-                if (*((volatile int *)(D.err + 3)) != 0) { ok = 0; break; }
-                if (++polls > (1u << 24)) {
-                    set_err(D, HD_ERR_TIMEOUT, -1, r);
-                    atomicExch(D.err + 3, 1);
-                    ok = 0;
-                    break;
+            unsigned long long v;
+            for (;;) {
+                asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(ctr) : "memory");
+                if ((unsigned)v >= target) break;
+                if ((++polls & 63u) == 0) {
+                    if (*((volatile int *)(D.err + 3)) != 0) { ok = 0; break; }
+                    if (polls > (1u << 24)) {
+                        set_err(D, HD_ERR_TIMEOUT, -1, r);
+                        atomicExch(D.err + 3, 1);
+                        ok = 0;
+                        break;
+                    }
+                    __nanosleep(64);
                 }
-                __nanosleep(64);
             }
-            __threadfence();
-            s_ok = ok;
+            hi = (unsigned)(v >> 32);
         }
-        __syncthreads();
-        if (!s_ok) return false;
+        s_hi = hi;
+        s_ok = ok;
     }
-    ++epoch;
-    return true;
+    __syncthreads();
+    ++B.epoch;
+    // at the other barriers the high half may already hold the next update's
+    if (s_moved) {
+        B.due = s_hi != B.moved;
+        B.moved = s_hi;
+    }
+    return s_ok != 0;
 }
 
-template <int PREC, int SPLIT>
+template <int PREC, int S>
 __global__ void __launch_bounds__(128, 4) k_persist(Dev D, int nsteps) {
     const int r = D.cta_rep[blockIdx.x];
     if (r < 0) return;
     const RepDev &R = D.rep[r];
     const int nc = D.pg_count[r], me = blockIdx.x - D.pg_first[r];
+    const int u0 = R.tile0 * D.split + me, u1 = (R.tile0 + R.ntile) * D.split;
     const bool leader = me == 0;
-    __shared__ RepState S;
+    __shared__ RepState St;
     __shared__ Scal C;
     __shared__ double acc[NPART + 1];
-    __shared__ int s_flag;
+    __shared__ int s_moved;
     __shared__ NlSmem M;
     extern __shared__ __align__(16) char nl_smem[];
     const NlStage T = nl_smem_carve(D, nl_smem);
     if (threadIdx.x == 0) {
-        S = D.st[r];
+        St = D.st[r];
         C = D.sc[r];
+        s_moved = D.rebuild[r] != 0;
     }
     __syncthreads();
-    unsigned epoch = 0;
+    GrpBar B = {0u, 0u, false};
     auto scalars = [&](int mode) {
         dev_scalar_acc<-1>(D, r, acc);
-        if (threadIdx.x < 32) scalar_eval(D, r, mode, acc, acc[NPART], S, C);
-        if (threadIdx.x == 0) {
-            if (leader) {
-                D.st[r] = S;
-                D.sc[r] = C;
-            }
-        }
+        if (threadIdx.x < 32) scalar_eval(D, r, mode, acc, acc[NPART], St, C);
         __syncthreads();
     };
     auto update = [&](int mode) {
-        for (int t = R.tile0 + me; t < R.tile0 + R.ntile; t += nc) {
-            if (PREC == HD_FP64) dev_update64(D, t, mode, C);
-            else dev_update32(D, t, mode, C);
+        for (int u = u0; u < u1; u += nc) {
+            if (PREC == HD_FP64) dev_update64(D, update_unit(D, u, &s_moved), mode, C);
+            else dev_update32(D, update_unit(D, u, &s_moved), mode, C);
         }
     };
     // the chain between the kicks (every CTA evaluates it alike from the
     // replica's kinetic sums)
     auto chain = [&](int mode) {
         dev_scalar_acc<-1>(D, r, acc);
-        if (threadIdx.x == 0) {
-            nhc_eval(D, r, mode, acc[NPART], S, C);
-            if (leader) {
-                D.st[r] = S;
-                D.sc[r] = C;
-            }
-        }
+        if (threadIdx.x == 0) nhc_eval(D, r, mode, acc[NPART], St, C);
         __syncthreads();
     };
     const bool nhc = D.any_nhc != 0;
@@ -2070,59 +2107,56 @@ __global__ void __launch_bounds__(128, 4) k_persist(Dev D, int nsteps) {
     scalars(MODE_OPEN);
     if (nhc) chain(MODE_OPEN);
     update(nhc ? (MODE_OPEN | MODE_NHC) : MODE_OPEN);
-    if (!grp_barrier(D, r, nc, epoch)) return;
+    if (!grp_barrier(D, r, nc, B, &s_moved)) return;
     for (int k = 1; k <= nsteps; ++k) {
-        if (threadIdx.x == 0) s_flag = *((volatile int *)(D.rebuild + r));
-        __syncthreads();
-        const int flag = s_flag;
-        if (flag) {
-            for (int t = R.tile0 + me; t < R.tile0 + R.ntile; t += nc) dev_bin(D, t);
-            if (!grp_barrier(D, r, nc, epoch)) return;
+        if (B.due) {
+            for (int i = R.atom0 + me * blockDim.x + threadIdx.x; i < R.atom0 + R.n; i += nc * blockDim.x) dev_bin_atom(D, r, i);
+            if (!grp_barrier(D, r, nc, B, nullptr)) return;
             {
                 const int wib = threadIdx.x >> 5, nwb = blockDim.x >> 5;
                 int *buf = reinterpret_cast<int *>(nl_smem) + wib * D.cell_cap;
                 for (int c = me * nwb + wib; c < R.ncell; c += nc * nwb) dev_cellsort_warp(D, R, c, buf);
                 __syncthreads();
             }
-            if (!grp_barrier(D, r, nc, epoch)) return;
-            // every CTA has read the flag before the first barrier above
-            if (threadIdx.x == 0) {
-                if (flag == 1) S.n_rebuild += 1;
-                if (leader) D.rebuild[r] = 0;
-            }
-            // rows are built cell by cell, so a CTA's tiles take rows other CTAs wrote
+            if (!grp_barrier(D, r, nc, B, nullptr)) return;
+            if (threadIdx.x == 0) St.n_rebuild += 1;
+            // rows are built cell by cell, so a CTA's units take rows other CTAs wrote
             for (int c = me; c < R.ncell; c += nc) dev_nlist_cell(D, r, c, M, T);
-            if (!grp_barrier(D, r, nc, epoch)) return;
+            if (!grp_barrier(D, r, nc, B, nullptr)) return;
             // the counts go back to zero for the next binning, whoever does it
             for (int c = me * blockDim.x + threadIdx.x; c < R.ncell; c += nc * blockDim.x) D.cell_cnt[R.cell0 + c] = 0;
         }
-        for (int t = R.tile0 * SPLIT + me; t < (R.tile0 + R.ntile) * SPLIT; t += nc) {
+        for (int u = u0; u < u1; u += nc) {
             // per-atom energies (observables only) on the last step of the call
             // and H.(r - r_O) there and wherever a bias may use it
             if (PREC == HD_FP64) {
-                if (k == nsteps) dev_pair64<false, true, true, SPLIT>(D, t);
-                else if (D.bias_on) dev_pair64<false, false, true, SPLIT>(D, t);
-                else dev_pair64<false, false, false, SPLIT>(D, t);
+                if (k == nsteps) dev_pair64<false, true, true, S>(D, u);
+                else if (D.bias_on) dev_pair64<false, false, true, S>(D, u);
+                else dev_pair64<false, false, false, S>(D, u);
             } else {
-                if (k == nsteps) dev_pair32<false, true, true, SPLIT>(D, t);
-                else if (D.bias_on) dev_pair32<false, false, true, SPLIT>(D, t);
-                else dev_pair32<false, false, false, SPLIT>(D, t);
+                if (k == nsteps) dev_pair32<false, true, true, S>(D, u);
+                else if (D.bias_on) dev_pair32<false, false, true, S>(D, u);
+                else dev_pair32<false, false, false, S>(D, u);
             }
         }
-        if (!grp_barrier(D, r, nc, epoch)) return;
+        if (!grp_barrier(D, r, nc, B, nullptr)) return;
         const int mode = k < nsteps ? (MODE_CLOSE | MODE_OPEN) : MODE_CLOSE;
         scalars(mode);
         if (!nhc) {
             update(mode);
         } else {
             update(MODE_CLOSE);
-            if (!grp_barrier(D, r, nc, epoch)) return;
+            if (!grp_barrier(D, r, nc, B, nullptr)) return;
             chain(mode);
             update((mode & MODE_OPEN) ? (MODE_OPEN | MODE_NHC) : MODE_SCALE);
         }
-        if (!grp_barrier(D, r, nc, epoch)) return;
+        if (!grp_barrier(D, r, nc, B, &s_moved)) return;
     }
-    if (leader && threadIdx.x == 0) D.st[r] = S;
+    if (leader && threadIdx.x == 0) {
+        D.st[r] = St;
+        D.sc[r] = C;
+        D.rebuild[r] = 0;
+    }
 }
 
 // ---------------------------------------------------------------- launchers
@@ -2132,11 +2166,13 @@ static inline int nthr(const Dev &D) { return D.block; }
 size_t nl_smem_bytes(const Dev &D, int nwarps) {
     return (size_t)nl_cand(D) * 16 + nwarps * nl_warp_bytes(D);
 }
-static size_t persist_smem_bytes(const Dev &D) { return nl_smem_bytes(D, (D.block + 31) / 32); }
+// threads of a CTA of the pair sweep and of the persistent launch: its unit's atoms times the lanes of a row
+static int unit_threads(const Dev &D) { return D.block / D.split * D.lanes; }
+static size_t persist_smem_bytes(const Dev &D) { return nl_smem_bytes(D, (unit_threads(D) + 31) / 32); }
 typedef void (*persist_fn)(Dev, int);
 static persist_fn persist_kernel(const Dev &D) {
-    if (D.prec == HD_FP64) return D.split == 4 ? k_persist<HD_FP64, 4> : k_persist<HD_FP64, 1>;
-    return D.split == 4 ? k_persist<HD_FP32_SPLIT, 4> : k_persist<HD_FP32_SPLIT, 1>;
+    if (D.prec == HD_FP64) return D.lanes == 4 ? k_persist<HD_FP64, 4> : k_persist<HD_FP64, 1>;
+    return D.lanes == 4 ? k_persist<HD_FP32_SPLIT, 4> : k_persist<HD_FP32_SPLIT, 1>;
 }
 cudaError_t nl_configure(const Dev &D, int *nl_blocks_per_sm) {
     const int bytes = (int)nl_smem_bytes(D, NL_THREADS / 32), pbytes = (int)persist_smem_bytes(D);
@@ -2167,7 +2203,7 @@ void launch_rebuild(const Dev &D, cudaStream_t s) {
 }
 template <int S>
 static void pair_of(const Dev &D, int kind, cudaStream_t s) {
-    const int grid = D.ntile * S, n = nthr(D);
+    const int grid = D.ntile * D.split, n = unit_threads(D);
     if (D.prec == HD_FP64) {
         if (kind == PAIR_QUENCH) k_pair64<true, false, false, S><<<grid, n, 0, s>>>(D, SWEEP_ALL);
         else if (kind == PAIR_ENERGY) k_pair64<false, true, true, S><<<grid, n, 0, s>>>(D, SWEEP_ALL);
@@ -2183,19 +2219,19 @@ static void pair_of(const Dev &D, int kind, cudaStream_t s) {
     }
 }
 void launch_pair(const Dev &D, int kind, cudaStream_t s) {
-    if (D.split == 4) pair_of<4>(D, kind, s);
+    if (D.lanes == 4) pair_of<4>(D, kind, s);
     else pair_of<1>(D, kind, s);
 }
 void launch_scalar(const Dev &D, int mode, bool lazy, bool list, cudaStream_t s) {
     const bool more = D.lazy_h && D.bias_on;
     k_scalar<<<D.nrep, sc_threads(D), 0, s>>>(D, mode, lazy && more, list && more);
     if (!lazy || !more) return;
-    const int n = nthr(D), g = D.hot_grid, li = list && more;
+    const int n = unit_threads(D), g = D.hot_grid, li = list && more;
     if (D.prec == HD_FP64) {
-        if (D.split == 4) k_scalar_late<HD_FP64, 4><<<g, n, 0, s>>>(D, mode, li);
+        if (D.lanes == 4) k_scalar_late<HD_FP64, 4><<<g, n, 0, s>>>(D, mode, li);
         else k_scalar_late<HD_FP64, 1><<<g, n, 0, s>>>(D, mode, li);
     } else {
-        if (D.split == 4) k_scalar_late<HD_FP32_SPLIT, 4><<<g, n, 0, s>>>(D, mode, li);
+        if (D.lanes == 4) k_scalar_late<HD_FP32_SPLIT, 4><<<g, n, 0, s>>>(D, mode, li);
         else k_scalar_late<HD_FP32_SPLIT, 1><<<g, n, 0, s>>>(D, mode, li);
     }
 }
@@ -2215,17 +2251,17 @@ void launch_qiter(const Dev &Q, int max_iter, cudaStream_t s) {
 void launch_qdisp(const Dev &Q, cudaStream_t s) { k_qdisp<<<Q.ntile, nthr(Q), 0, s>>>(Q); }
 int persist_blocks_per_sm(const Dev &D) {
     int nb = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, persist_kernel(D), D.block, persist_smem_bytes(D));
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, persist_kernel(D), unit_threads(D), persist_smem_bytes(D));
     return nb;
 }
 cudaError_t launch_persist(const Dev &D, int grid, int nsteps, cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(D.bar, 0, sizeof(unsigned) * D.nrep, s);
+    cudaError_t e = cudaMemsetAsync(D.bar, 0, sizeof(unsigned long long) * D.nrep, s);
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(D.err + 3, 0, sizeof(int), s);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(D.block);
+    cfg.blockDim = dim3(unit_threads(D));
     cfg.dynamicSmemBytes = persist_smem_bytes(D);
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
