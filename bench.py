@@ -57,7 +57,7 @@ def parse():
     ap.add_argument("--driver", default="auto", choices=["auto", "kernels", "persistent"])
     ap.add_argument("--block", type=int, default=0)
     ap.add_argument("--pair-kernel", type=int, default=0, choices=[0, 1],
-                    help="split form with --driver kernels: 0 scalar, 1 packed FP32x2 pair sweep")
+                    help="kept: the split form has one pair sweep, packed FP32x2, either way")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-fp64-compare", action="store_true")
     ap.add_argument("--cpu-seconds", type=float, default=12.0)
@@ -416,9 +416,9 @@ def run_ours(args):
     # algorithmic bytes per atom-step: every unique pair's index once (half
     # list, 2 nnb), position and velocity read and written, r_O read, type
     # and role (98 B split: FP64 r, FP32 v; 122 B FP64 form); the full list
-    # this kernel streams moves 4 nnb + the records and results (100 / 196 B)
+    # a force sweep streams moves 4 nnb + the records and results (52 / 132 B)
     bytes_per_atom = 2.0 * nnb + (98 if split else 122)
-    streamed_per_atom = 4.0 * nnb + (4 + 16 + 16 + 16 + 16 + 32 if split else 4 + 32 + 32 + 32 + 32 + 64)
+    streamed_per_atom = 4.0 * nnb + (4 + 16 + 16 + 16 if split else 4 + 32 + 32 + 32 + 32)
     traffic = committed_traffic(split)
     peaks = {}
     try:
@@ -430,8 +430,7 @@ def run_ours(args):
         achieved = bytes_per_atom * natoms / (pair_ms * 1e-3) / 1e9
         roof = {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
                 "traffic": traffic,
-                "kernel": ("k_pair32x2<false,false>" if b.params.pair_kernel == 1 else "k_pair32<false,false>")
-                if split else "k_pair64<false,false>",
+                "kernel": "k_pair32 (k_pair_hot included)" if split else "k_pair64 (k_pair_hot included)",
                 "algorithmic_bytes_per_atom": bytes_per_atom, "mean_neighbours": nnb,
                 "streamed_bytes_per_atom": streamed_per_atom,
                 "streamed_frac": streamed_per_atom * natoms / (pair_ms * 1e-3) / 1e9 / hbm,
@@ -497,8 +496,7 @@ def run_ours(args):
                            args.quench_ftol, args.quench_stay, args.quench_iters),
                        "driver": {1: "kernels", 2: "persistent"}.get(b.info()["driver"], "kernels"),
                        "block": (b.tuned or {}).get("block") or args.block or 128,
-                       "pair_kernel": {0: "scalar", 1: "packed FP32x2"}[(b.tuned or {}).get("pair_kernel",
-                                                                                              args.pair_kernel)],
+                       "pair_kernel": "packed FP32x2",
                        "autotune": b.tuned,
                        "precision": "split: FP32 pair/bias arithmetic, FP64 positions, sums, clocks" if split
                        else "FP64 throughout", "l2": "inputs larger than L2 (%.0f MB workspace)" % (

@@ -17,7 +17,8 @@ import os
 
 from . import hd
 
-# (driver, tile size, pair-sweep variant: 0 scalar, 1 packed FP32x2)
+# (driver, tile size, hd_params.pair_kernel: kept for callers that set it; both
+# values run the same sweep)
 CANDIDATES = [(hd.HD_DRIVER_KERNELS, 128, 0), (hd.HD_DRIVER_KERNELS, 64, 0), (hd.HD_DRIVER_KERNELS, 256, 0),
               (hd.HD_DRIVER_KERNELS, 128, 1), (hd.HD_DRIVER_KERNELS, 64, 1),
               (hd.HD_DRIVER_PERSISTENT, 128, 0), (hd.HD_DRIVER_PERSISTENT, 64, 0)]
@@ -25,7 +26,7 @@ DEFAULT = (hd.HD_DRIVER_KERNELS, 128, 0)
 
 
 def candidates(params):
-    """The packed pair sweep exists in the split form only."""
+    """pair_kernel 1 is offered in the split form only."""
     return [c for c in CANDIDATES if c[2] == 0 or params.prec == hd.HD_FP32_SPLIT]
 
 
