@@ -1944,7 +1944,7 @@ __global__ void __launch_bounds__(256) k_qupdate(Dev D) {
 // image, FP64, the oracle's operation order); stored as the bits of the
 // non-negative double so that an integer max is the FP64 max.
 // One atomic per CTA: with one per atom the 14,272 of a replica ran one after
-// another (508 us for 64 of them).  Below half a box the nearest integer to
+// another (508 us for 64 of them; 26 now).  Below half a box the nearest integer to
 // d / L is 0 and the division, which the FP64 pipe takes ten instructions for,
 // is left out.
 __global__ void __launch_bounds__(256) k_qdisp(Dev Q) {
