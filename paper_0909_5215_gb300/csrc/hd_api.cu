@@ -252,16 +252,6 @@ bool make_plan(const hd_replica_desc *reps, int n_rep, const hd_params *p, Plan 
         R.dvmax = d.dvmax;
         R.sig_lo = d.sig_lo;
         R.sig_hi = d.sig_hi;
-        // pair sweep: lengths in the common unit u (px = 1, times 2^zshift on the
-        // open axis; 1/u^2 = pu2) or, without one, in real lengths (px = lsb)
-        const double unit = R.exact_r2 ? 1.0 / R.fx_scale[0] : 1.0, pu2 = 1.0 / (unit * unit);
-        double near2 = 0.0;
-        for (int a = 0; a < 3; ++a) {
-            const double out = R.exact_r2 ? 1.0 / unit : 1.0 + (double)R.lsb_rel[a];
-            R.px_scale[a] = R.exact_r2 ? (float)(1 << (a == 1 ? R.shift_y : a == 2 ? R.shift_z : 0)) : R.fx_lsb[a];
-            R.out_hi[a] = (float)out;
-            R.out_lo[a] = (float)(out - (double)R.out_hi[a]);
-        }
         for (int a = 0; a < 2; ++a)
             for (int b = 0; b < 2; ++b) {
                 const double eps = d.eps[a][b], sig = d.sig[a][b];
@@ -273,28 +263,16 @@ bool make_plan(const hd_replica_desc *reps, int n_rep, const hd_params *p, Plan 
                 R.sig2f[a][b] = (float)(sig * sig);
                 R.shiftf[a][b] = (float)R.shift[a][b];
                 const double r0sq = std::cbrt(2.0) * sig * sig;   // LJ minimum 2^(1/6) sigma, squared
-                {   // 20 bits, so that its difference from any r^2 up to rc^2 is exact
-                    int e;
-                    const double m = std::frexp(r0sq * pu2, &e);
-                    R.r0u_hi[a][b] = (float)std::ldexp(std::floor(std::ldexp(m, 20)), e - 20);
-                }
-                R.r0u_lo[a][b] = (float)(r0sq * pu2 - (double)R.r0u_hi[a][b]);
+                R.r0sq_hi[a][b] = (float)r0sq;
+                R.r0sq_lo[a][b] = (float)(r0sq - (double)R.r0sq_hi[a][b]);
                 R.eps12f[a][b] = (float)(12.0 * eps);
                 R.eps12l[a][b] = (float)(12.0 * eps - (double)R.eps12f[a][b]);
-                near2 = std::max(near2, r0sq * 4.0 / 3.0);
-                // the pair sweep takes the exact r^2 where r^2 < (4/3) r_0^2; class A
-                // of the list holds the pairs within that radius plus 0.1 sigma at
-                // build time
+                // the pair sweep takes the exact r^2 where |r_0^2 - r^2| < r^2 / 4,
+                // i.e. r^2 < (4/3) r_0^2; class A of the list holds the pairs within
+                // that radius plus 0.1 sigma at build time
                 const double rA = std::sqrt(r0sq * 4.0 / 3.0) + 0.1 * sig;
                 R.rA2f = std::max(R.rA2f, (float)(rA * rA));
             }
-        // FP32 r^2 of the split sweep is within ~3e-7 (relative) of the oracle's
-        // FP64 r^2 (fixed-point rounding of positions plus FP32 rounding); the
-        // band decided in FP64 is 2^-20 ~ 9.5e-7 wide on each side
-        const double rc2u = p->rc * p->rc * pu2;
-        R.rc2u_lo = (float)(rc2u * (1.0 - 1.0 / 1048576.0));
-        R.rc2u_hi = (float)(rc2u * (1.0 + 1.0 / 1048576.0));
-        R.near2u = R.exact_r2 ? std::min((float)(near2 * pu2), R.rc2u_lo) : 0.f;
         R.kr_n = nrig > 0 ? d.k_spring / nrig : 0.0;
         R.kr_nf = (float)R.kr_n;
         // eigenvalue bias: Lanczos steps at most, capped at the dimension of the
@@ -697,7 +675,11 @@ void set_scalars(Dev &D, const hd_params *p) {
     D.half_skin2 = 0.25 * p->skin * p->skin;
     D.rl2_lo_f = (float)(D.rl2 * (1.0 - 1.0 / 4096.0));
     D.rl2_hi_f = (float)(D.rl2 * (1.0 + 1.0 / 4096.0));
+    // FP32 r^2 of the split sweep is within ~3e-7 (relative) of the oracle's
+    // FP64 r^2 (fixed-point rounding of positions plus FP32 rounding); the
+    // band decided in FP64 is 2^-20 ~ 9.5e-7 wide on each side
     D.rc2_lo_f = (float)(D.rc2 * (1.0 - 1.0 / 1048576.0));
+    D.rc2_hi_f = (float)(D.rc2 * (1.0 + 1.0 / 1048576.0));
     D.half_skin2_f = (float)(D.half_skin2 * (1.0 - 1e-4));
     D.seed_lo = (uint32_t)p->seed;
     D.seed_hi = (uint32_t)(p->seed >> 32);

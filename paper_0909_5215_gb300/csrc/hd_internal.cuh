@@ -94,13 +94,7 @@ struct RepDev {
     int exact_r2, zshift, shift_y, shift_z;
     float u2_42, u2_21, u2_0, u2lo_42;     // u^2 2^42, u^2 2^21, u^2 (FP32) and the low part of u^2 2^42
     float lsb_rel[3];            // (unit - fl32(unit)) / fl32(unit) per axis
-    // pair sweep: lengths in the common unit u where the axes share one
-    // (exact_r2), else in the axes' own units; separations are integer x
-    // px_scale, the finished sums are multiplied by out = hi + lo (1/u, or the
-    // rounding of lsb undone)
-    float px_scale[3], out_hi[3], out_lo[3];
-    float rc2u_lo, rc2u_hi, near2u;      // rc^2 (1 -+ 2^-20); the exact r^2 is taken below near2u = (4/3) r_0^2
-    float r0u_hi[2][2], r0u_lo[2][2];    // r_0^2 = 2^(1/3) sigma_ab^2 (LJ minimum, squared) as hi + lo
+    float r0sq_hi[2][2], r0sq_lo[2][2];  // r_0^2 = 2^(1/3) sigma_ab^2 (LJ minimum, squared) as hi + lo
     float eps12f[2][2], eps12l[2][2];    // 12 eps_ab as hi + lo
     int nl_local;                // every periodic axis has four cells or more (see k_nlist)
     float rA2f;                  // list class A (first shell): FP32 r^2 below this at build time
@@ -156,7 +150,7 @@ struct Dev {
     double dt, rc2, rl2, half_skin2, q_ftol, q_step, q_theta;
     double q_ftol_stay, q_keep2;    // quench: early stop inside the basin (0: off), (theta/2)^2
     float rl2_lo_f, rl2_hi_f, half_skin2_f;
-    float rc2_lo_f;              // rc^2 (1 - 2^-20): list class B ends here
+    float rc2_lo_f, rc2_hi_f;    // rc^2 (1 -+ 2^-20): band decided in FP64 (list class B ends at the lower one)
     uint32_t seed_lo, seed_hi;
     const RepDev *rep;
     RepState *st;
@@ -339,19 +333,6 @@ __device__ __forceinline__ void r2_split(const RepDev &R, int ix, int iy, int iz
     hi = a + b;
     const float eb = (a - hi) + b;
     lo = (ea + eb) + fmaf(f0, R.u2_0, f2 * R.u2lo_42);
-}
-
-// The same in units of u^2 (the pieces' weights are powers of two, so only
-// the two sums round).
-__device__ __forceinline__ void r2_units(int ix, int iy, int iz, float &hi, float &lo) {
-    unsigned long long q = (unsigned long long)((long long)ix * (long long)ix);
-    q += (unsigned long long)((long long)iy * (long long)iy);
-    q += (unsigned long long)((long long)iz * (long long)iz);
-    const float f0 = exact_f23((unsigned int)q & 0x1FFFFFu);
-    const float b = exact_f23((unsigned int)(q >> 21) & 0x1FFFFFu) * 2097152.f;
-    const float a = exact_f23((unsigned int)(q >> 42)) * 4398046511104.f;
-    hi = a + b;
-    lo = ((a - hi) + b) + f0;
 }
 
 // Row lengths: the flag says that the row or its atom holds a tip atom.

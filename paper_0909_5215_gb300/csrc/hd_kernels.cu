@@ -318,6 +318,9 @@ __global__ void __launch_bounds__(128) k_cellsort(Dev D) {
 //    gets a class: A (first shell) FP32 r^2 < rA^2, the pairs that can come
 //    within the range where the pair sweep takes the exact r^2; B the rest of
 //    the pairs within rc at build time; C (skin shell) the rest of the row.
+//    The class decides the place in the row, and with it the order in which
+//    the sweep adds up forces, so next to its two bounds it is taken from the
+//    images themselves: it must not depend on which cell's centre was near.
 //
 // The row is then written as A | B | C, each block in candidate order, so the
 // lanes of the pair sweep leave the first shell, and later the cutoff, at
@@ -347,6 +350,13 @@ struct NlStage {
     int *j;
     char *warp;
 };
+
+// FP32 r^2 of two images, from their exact integer differences
+__device__ __forceinline__ float img_r2(const RepDev &R, int4 a, int4 b) {
+    const int4 d = img_diff(a, b);
+    const float dx = (float)d.x * R.fx_lsb[0], dy = (float)d.y * R.fx_lsb[1], dz = (float)d.z * R.fx_lsb[2];
+    return dx * dx + dy * dy + dz * dz;
+}
 
 template <bool LOCAL>
 __device__ __forceinline__ void dev_nlist_rows(const Dev &D, const RepDev &R, int r, int m, const NlSmem &M, const NlStage &T) {
@@ -402,8 +412,9 @@ __device__ __forceinline__ void dev_nlist_rows(const Dev &D, const RepDev &R, in
             if (q != slot) {
                 const int jt = T.j[q], j = jt & 0x7fffffff;
                 const float dx = diff(xi, T.x[q], lx), dy = diff(yi, T.y[q], ly), dz = diff(zi, T.z[q], lz);
-                const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+                float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
                 if (r2 < lo || exact_r2(R, D.x[i], D.x[j]) < D.rl2) {
+                    if (fabsf(r2 - rA2) < rA2 * 0x1p-16f || fabsf(r2 - rc2) < rc2 * 0x1p-16f) r2 = img_r2(R, D.p[i], D.p[j]);
                     cl = r2 < rA2 ? 0 : (r2 < rc2 ? 1 : 2);
                     mixed |= (unsigned)jt >> 31;
                 }
@@ -717,43 +728,53 @@ __device__ __forceinline__ void dev_pair64(const Dev &D, int unit) {
 // Positions are differenced exactly in 32-bit fixed point, the pair
 // arithmetic is FP32, per-tile sums are carried in FP64.
 //
-// The sweep is bound by instruction issue (and next by the L1 wavefronts of
-// its gathers), so it is laid out to spend few instructions per list entry.
-// Per sweep of 913,408 atoms with 76 entries each: 306 us before these steps,
-// 259 us with the Hessian term, 122 to 143 us without it.
-//   - lengths stay in the replica's fixed-point unit u: separations are the
-//     converted integers (times 2^zshift on the open axis), r^2, r_0^2 and
-//     the cutoffs are in u^2, and the one factor 1/u goes to the finished
-//     sums.  Replicas whose axes share no unit use the axes' own units
-//     (scale lsb) and real lengths, with the same code;
-//   - with c = (r_0^2/r^2)^3 = 2 s^6 and w = c - 1 the force is
-//     g w r_ij, g = 12 eps c / r^2, and the Hessian term
-//     -g w u + g (14 c - 8) (r.u)/r^2 r_ij, so both share one product with eps;
-//   - four list entries are one 16-byte load, the row's position in the list
-//     is an immediate offset, and the neighbour's record is 16 bytes; r - r_O
-//     of a pair is its separation minus that of the two r_O's images, so only
-//     the Hessian term reads a second record.
+// Near the LJ minimum the force holds the cancelling factor w = 2 s^6 - 1; it
+// is evaluated as t (3 + 3 t + t^2) with t = (r_0^2 - r^2) / r^2.  Where
+// |t| < 1/4, and the FP32 r^2 would cost w its relative accuracy, r^2 is taken
+// exactly, as hi + lo, from the integer separations; elsewhere the FP32 r^2
+// gives w to a few ulps.  The row builder puts the pairs that can need the
+// exact r^2 at the head of each row, so a warp leaves that form after its
+// first groups of four.  With c = 2 s^6 = (1 + t)^3 the force is 12 eps c w /
+// r^2 r_ij and the Hessian term -f u + 12 eps c (14 c - 8) (r.u) / r^4 r_ij.
 //
-// Near the LJ minimum the force holds the cancelling factor w; it is
-// evaluated as t (3 + 3 t + t^2) with t = (r_0^2 - r^2) / r^2.  Below
-// r^2 = (4/3) r_0^2, where the FP32 r^2 would cost w its relative accuracy,
-// r^2 is taken exactly, as hi + lo, from the integer separations; beyond it
-// the FP32 r^2 gives w to a few ulps.  The row builder puts the pairs that
-// can need the exact r^2 at the head of each row, so a warp takes the exact
-// form for its first groups of four and the other one from there on.
+// With a lane to a row, what its entries give is added up one after another,
+// in the row's order, whichever entries share a packed instruction: a force is
+// then a function of the row alone, to the last bit.  It matters because the
+// LJ force jumps by 0.04 where it is cut at rc: where two trajectories part by
+// rounding (~1e-8 in positions), a pair that close to rc is cut a step sooner
+// in one of them and positions part by 1e-6 a step (a replica of 14,272 atoms
+// meets such a pair in one of ten runs of 40 steps).  Packed sums and lengths
+// in units of the fixed point, which round otherwise, did that: a step of 64 x
+// 14,272 atoms took 307 us with them and takes 315.  Four lanes to a row (small
+// batches) add up their own entries and meet in a tree; keeping the order there
+// too, through shared memory, made a step of 8 x 1,983 atoms 57.5 us for 53.8.
+//
+// The sweep is bound by instruction issue (and next by the L1 wavefronts of
+// its gathers), so it is laid out to spend few instructions per list entry:
+// four list entries are one 16-byte load, the row's position in the list is an
+// immediate offset, the neighbour's record is 16 bytes, two entries at a time
+// go through packed FP32x2 arithmetic (the same roundings as one by one); and
+// r - r_O of a pair is its separation minus that of the two r_O's images, so
+// only the Hessian term reads a second record.
 __device__ __forceinline__ float rcp_approx(float x) {
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
 // 1/x to FP32 rounding: the hardware approximation refined by one Newton
-// step, y (2 - x y), so that its error carries no bias into the forces
+// step, y + y (1 - x y), so that its error carries no bias into the forces
 // (an unrefined approximation shifts every pair force the same way, and the
 // slope sigma of Eq. 5 sums them over the whole replica).
-__device__ __forceinline__ float rcp_refined(float x) {
-    const float y = rcp_approx(x);
-    return fmaf(y, fmaf(-x, y, 1.f), y);
+__device__ __forceinline__ float2 rcp_refined(float2 x) {
+    const float2 y = make_float2(rcp_approx(x.x), rcp_approx(x.y));
+    return f2fma(y, f2fma(f2neg(x), y, f2c(1.f)), y);
 }
+
+// What two entries of a row give: force factor, Hessian factor and r - r_O of
+// the pair, energy.
+struct PairTerms {
+    float2 fr, B, ux, uy, uz, ee;
+};
 
 // S, unit: as in dev_pair64.
 template <bool Q, bool E, bool H, int S>
@@ -769,71 +790,76 @@ __device__ __forceinline__ void dev_pair32(const Dev &D, int unit) {
     const int4 pi = D.p[i];
     const int4 poi = H ? D.po[i] : make_int4(0, 0, 0, 0);
     const int ti = pi.w & 1;
-    const float sx = R.px_scale[0], sy = R.px_scale[1], sz = R.px_scale[2];
+    const float lx = R.fx_lsb[0], ly = R.fx_lsb[1], lz = R.fx_lsb[2];
     // 12 eps as FP32 hi + lo: an eps such as 0.2 is not an FP32 number, and
     // its rounding would scale every such pair force alike
     const float a0 = R.eps12f[ti][0], a1 = R.eps12f[ti][1], al0 = R.eps12l[ti][0], al1 = R.eps12l[ti][1];
-    const float q0h = R.r0u_hi[ti][0], q1h = R.r0u_hi[ti][1], q0l = R.r0u_lo[ti][0], q1l = R.r0u_lo[ti][1];
-    const float rc_lo = R.rc2u_lo, rc_hi = R.rc2u_hi, near2 = R.near2u;   // near2 is 0 without a common unit
-    float e = 0.f;
+    const float q0h = R.r0sq_hi[ti][0], q1h = R.r0sq_hi[ti][1], q0l = R.r0sq_lo[ti][0], q1l = R.r0sq_lo[ti][1];
+    const float rc_lo = D.rc2_lo_f, rc_hi = D.rc2_hi_f;
+    const bool exact = R.exact_r2 != 0;
+    // the rounding of the fixed-point unit, undone in r^2 (all axes share it
+    // when they share the unit)
+    const float corr = exact ? 2.f * R.lsb_rel[0] : 0.f;
     const int len = act ? D.nnb[i] : 0, nn = NB_LEN(len);
     const bool mix = __any_sync(0xffffffffu, (len & NB_MIXED) != 0);
-    // Two entries at once in packed FP32x2 arithmetic (one instruction for
-    // both), in stages without branches.  An entry outside the cutoff (or past
-    // the row's end) takes part at r^2 = 3e38, where every product below is
-    // zero.  near_: some lane has an entry below (4/3) r_0^2, and all take the
-    // exact r^2.  MIX: some lane's row or atom is of the tip; without one the
-    // parameters are the substrate's and nothing is selected.
+    // In stages without branches.  An entry outside the cutoff (or past the
+    // row's end) takes part at r^2 = 3e38, where every product below is zero.
+    // MIX: some lane's row or atom is of the tip; without one the parameters
+    // are the substrate's and nothing is selected.  vote: the whole warp is
+    // here, and takes the exact r^2 if one of its lanes needs it.
     constexpr float FAR = 3.0e38f;
-    float2 Fx = make_float2(0.f, 0.f), Fy = Fx, Fz = Fx, Hx = Fx, Hy = Fx, Hz = Fx;
-    auto two = [&](bool near_, bool mix, int4 pa, int4 pb, int4 poa, int4 pob, int ixa, int ixb, int iya, int iyb, int iza,
-                   int izb, float2 dx, float2 dy, float2 dz, float2 r2) {
+    auto two = [&](bool vote, bool mix, int4 pa, int4 pb, int4 poa, int4 pob, int ixa, int ixb, int iya, int iyb, int iza,
+                   int izb, float2 dx, float2 dy, float2 dz, float2 r2, PairTerms &o) {
         const bool ta = mix && (pa.w & 1), tb = mix && (pb.w & 1);
         const float2 r0h = make_float2(ta ? q1h : q0h, tb ? q1h : q0h), r0l = make_float2(ta ? q1l : q0l, tb ? q1l : q0l);
-        float2 h = r2, l = r0l;
-        if (near_) {
+        const float2 r2c = f2fma(r2, f2c(corr), r2);
+        float2 ir2 = rcp_refined(r2c);
+        float2 tt = f2mul(f2add(f2sub(r0h, r2c), r0l), ir2);
+        const bool na = exact && r2.x < FAR && fabsf(tt.x) < 0.25f, nb = exact && r2.y < FAR && fabsf(tt.y) < 0.25f;
+        if (vote ? __any_sync(0xffffffffu, na || nb) : (na || nb)) {
             float ha, la, hb, lb;
-            r2_units(ixa, iya << R.shift_y, iza << R.shift_z, ha, la);
-            r2_units(ixb, iyb << R.shift_y, izb << R.shift_z, hb, lb);
-            h = make_float2(r2.x < FAR ? ha : FAR, r2.y < FAR ? hb : FAR);
-            l = f2sub(r0l, make_float2(la, lb));
+            r2_split(R, ixa, iya, iza, ha, la);
+            r2_split(R, ixb, iyb, izb, hb, lb);
+            const float2 h = make_float2(ha, hb), ih = rcp_refined(h);
+            const float2 th = f2mul(f2add(f2sub(r0h, h), f2sub(r0l, make_float2(la, lb))), ih);
+            ir2 = make_float2(na ? ih.x : ir2.x, nb ? ih.y : ir2.y);
+            tt = make_float2(na ? th.x : tt.x, nb ? th.y : tt.y);
         }
-        // 1/r^2: the hardware approximation and one Newton step (rcp_refined)
-        float2 ir2 = make_float2(rcp_approx(h.x), rcp_approx(h.y));
-        ir2 = f2fma(ir2, f2fma(f2neg(h), ir2, f2c(1.f)), ir2);
-        // r0h holds 20 bits, so r0h - h is exact whatever the distance; the rest
-        // joins by a product: added to r0h - h it would round off alike in every
-        // pair (1.8e-7 of each force beyond 1.6 sigma, all of one sign)
-        const float2 tt = f2fma(l, ir2, f2mul(f2sub(r0h, h), ir2));
         const float2 c1 = f2add(tt, f2c(1.f));
         const float2 c = f2mul(f2mul(c1, c1), c1);                               // 2 s^6
         const float2 w = f2mul(tt, f2fma(tt, f2add(tt, f2c(3.f)), f2c(3.f)));    // 2 s^6 - 1
-        const float2 g0 = f2mul(ir2, c);
-        const float2 g = f2fma(g0, make_float2(ta ? al1 : al0, tb ? al1 : al0),
-                               f2mul(g0, make_float2(ta ? a1 : a0, tb ? a1 : a0)));
-        const float2 fr = f2mul(g, w);
-        Fx = f2fma(fr, dx, Fx);
-        Fy = f2fma(fr, dy, Fy);
-        Fz = f2fma(fr, dz, Fz);
+        const float2 eh = make_float2(ta ? a1 : a0, tb ? a1 : a0), el = make_float2(ta ? al1 : al0, tb ? al1 : al0);
+        const float2 pf = f2mul(f2mul(ir2, c), w);
+        o.fr = f2fma(pf, el, f2mul(pf, eh));
         if (E) {
             const float sa = 0.5f * c.x, sb = 0.5f * c.y;
             const float ea = fmaf(4.f * R.epsf[ti][ta] * sa, sa - 1.f, -R.shiftf[ti][ta]);
             const float eb = fmaf(4.f * R.epsf[ti][tb] * sb, sb - 1.f, -R.shiftf[ti][tb]);
-            e = fmaf(0.5f, r2.x < FAR ? ea : 0.f, e);
-            e = fmaf(0.5f, r2.y < FAR ? eb : 0.f, e);
+            o.ee = make_float2(r2.x < FAR ? ea : 0.f, r2.y < FAR ? eb : 0.f);
         }
         if (H) {
-            const float2 ux = f2mul(f2i(ixa - (int)((unsigned)poi.x - (unsigned)poa.x), ixb - (int)((unsigned)poi.x - (unsigned)pob.x)), f2c(sx));
-            const float2 uy = f2mul(f2i(iya - (int)((unsigned)poi.y - (unsigned)poa.y), iyb - (int)((unsigned)poi.y - (unsigned)pob.y)), f2c(sy));
-            const float2 uz = f2mul(f2i(iza - (int)((unsigned)poi.z - (unsigned)poa.z), izb - (int)((unsigned)poi.z - (unsigned)pob.z)), f2c(sz));
-            const float2 rdu = f2fma(dx, ux, f2fma(dy, uy, f2mul(dz, uz)));
-            const float2 B = f2mul(f2mul(g, f2fma(c, f2c(14.f), f2c(-8.f))), f2mul(ir2, rdu)), nfr = f2neg(fr);
-            Hx = f2fma(nfr, ux, f2fma(B, dx, Hx));
-            Hy = f2fma(nfr, uy, f2fma(B, dy, Hy));
-            Hz = f2fma(nfr, uz, f2fma(B, dz, Hz));
+            o.ux = f2mul(f2i(ixa - (int)((unsigned)poi.x - (unsigned)poa.x), ixb - (int)((unsigned)poi.x - (unsigned)pob.x)), f2c(lx));
+            o.uy = f2mul(f2i(iya - (int)((unsigned)poi.y - (unsigned)poa.y), iyb - (int)((unsigned)poi.y - (unsigned)pob.y)), f2c(ly));
+            o.uz = f2mul(f2i(iza - (int)((unsigned)poi.z - (unsigned)poa.z), izb - (int)((unsigned)poi.z - (unsigned)pob.z)), f2c(lz));
+            const float2 rdu = f2fma(dx, o.ux, f2fma(dy, o.uy, f2mul(dz, o.uz)));
+            const float2 pb2 = f2mul(f2mul(f2mul(f2mul(ir2, ir2), c), f2fma(c, f2c(14.f), f2c(-8.f))), rdu);
+            o.B = f2fma(pb2, el, f2mul(pb2, eh));
         }
     };
     auto sep = [](int a, int b) { return (int)((unsigned)a - (unsigned)b); };
+    float fx = 0.f, fy = 0.f, fz = 0.f, e = 0.f, hx = 0.f, hy = 0.f, hz = 0.f;
+    float2 Fx = make_float2(0.f, 0.f), Fy = Fx, Fz = Fx, Hx = Fx, Hy = Fx, Hz = Fx;     // four lanes: packed sums
+    auto add = [&](float fr, float B, float ux, float uy, float uz, float ee, float dx, float dy, float dz) {
+        fx = fmaf(fr, dx, fx);
+        fy = fmaf(fr, dy, fy);
+        fz = fmaf(fr, dz, fz);
+        if (E) e = fmaf(0.5f, ee, e);
+        if (H) {
+            hx = fmaf(-fr, ux, fmaf(B, dx, hx));
+            hy = fmaf(-fr, uy, fmaf(B, dy, hy));
+            hz = fmaf(-fr, uz, fmaf(B, dz, hz));
+        }
+    };
     bool band = false;
     const int ngroup = (nn + 3) >> 2;
     int itmax = (ngroup - sub + S - 1) / S;
@@ -856,27 +882,37 @@ __device__ __forceinline__ void dev_pair32(const Dev &D, int unit) {
         for (int u = 0; u < 4; u += 2) {
             const int ixa = sep(pi.x, p4[u].x), iya = sep(pi.y, p4[u].y), iza = sep(pi.z, p4[u].z);
             const int ixb = sep(pi.x, p4[u + 1].x), iyb = sep(pi.y, p4[u + 1].y), izb = sep(pi.z, p4[u + 1].z);
-            const float2 dx = f2mul(f2i(ixa, ixb), f2c(sx)), dy = f2mul(f2i(iya, iyb), f2c(sy)),
-                         dz = f2mul(f2i(iza, izb), f2c(sz));
+            const float2 dx = f2mul(f2i(ixa, ixb), f2c(lx)), dy = f2mul(f2i(iya, iyb), f2c(ly)),
+                         dz = f2mul(f2i(iza, izb), f2c(lz));
             float2 r2 = f2fma(dx, dx, f2fma(dy, dy, f2mul(dz, dz)));
             const bool ina = u < left && r2.x < rc_lo, inb = u + 1 < left && r2.y < rc_lo;
             band |= (u < left && r2.x < rc_hi && !ina) || (u + 1 < left && r2.y < rc_hi && !inb);
             r2.x = ina ? r2.x : FAR;
             r2.y = inb ? r2.y : FAR;
-            const float lowest = fminf(r2.x, r2.y);
-            if (!__any_sync(0xffffffffu, lowest < FAR)) continue;      // the skin shell
-            auto both = [&](bool nr, bool mx) {
-                two(nr, mx, p4[u], p4[u + 1], po4[u], po4[u + 1], ixa, ixb, iya, iyb, iza, izb, dx, dy, dz, r2);
-            };
-            const bool near_ = __any_sync(0xffffffffu, lowest < near2);
-            if (mix) {
-                if (near_) both(true, true);
-                else both(false, true);
+            if (!__any_sync(0xffffffffu, ina || inb)) continue;      // the skin shell
+            PairTerms o;
+            if (mix) two(true, true, p4[u], p4[u + 1], po4[u], po4[u + 1], ixa, ixb, iya, iyb, iza, izb, dx, dy, dz, r2, o);
+            else two(true, false, p4[u], p4[u + 1], po4[u], po4[u + 1], ixa, ixb, iya, iyb, iza, izb, dx, dy, dz, r2, o);
+            if (S == 1) {
+                add(o.fr.x, o.B.x, o.ux.x, o.uy.x, o.uz.x, o.ee.x, dx.x, dy.x, dz.x);
+                add(o.fr.y, o.B.y, o.ux.y, o.uy.y, o.uz.y, o.ee.y, dx.y, dy.y, dz.y);
             } else {
-                if (near_) both(true, false);
-                else both(false, false);
+                Fx = f2fma(o.fr, dx, Fx);
+                Fy = f2fma(o.fr, dy, Fy);
+                Fz = f2fma(o.fr, dz, Fz);
+                if (E) e = fmaf(0.5f, o.ee.y, fmaf(0.5f, o.ee.x, e));
+                if (H) {
+                    const float2 nfr = f2neg(o.fr);
+                    Hx = f2fma(nfr, o.ux, f2fma(o.B, dx, Hx));
+                    Hy = f2fma(nfr, o.uy, f2fma(o.B, dy, Hy));
+                    Hz = f2fma(nfr, o.uz, f2fma(o.B, dz, Hz));
+                }
             }
         }
+    }
+    if (S > 1) {
+        fx = Fx.x + Fx.y; fy = Fy.x + Fy.y; fz = Fz.x + Fz.y;
+        hx = Hx.x + Hx.y; hy = Hy.x + Hy.y; hz = Hz.x + Hz.y;
     }
     // Rare: pairs in a thin band around rc are cut by the oracle's FP64 test
     // (same operations), so no pair is cut at a different step than in FP64.
@@ -888,14 +924,16 @@ __device__ __forceinline__ void dev_pair32(const Dev &D, int unit) {
             const int j = D.nbr[nbr_at(row4, k)];
             const int4 pj = D.p[j];
             const int ix = sep(pi.x, pj.x), iy = sep(pi.y, pj.y), iz = sep(pi.z, pj.z);
-            const float dx = (float)ix * sx, dy = (float)iy * sy, dz = (float)iz * sz;
+            const float dx = (float)ix * lx, dy = (float)iy * ly, dz = (float)iz * lz;
             const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-            if (r2 >= rc_lo && r2 < rc_hi && exact_r2(R, xi64, D.x[j]) < D.rc2)
+            if (r2 >= rc_lo && r2 < rc_hi && exact_r2(R, xi64, D.x[j]) < D.rc2) {
+                PairTerms o;
                 two(false, true, pj, zero, H ? D.po[j] : zero, zero, ix, 0, iy, 0, iz, 0, make_float2(dx, 0.f),
-                    make_float2(dy, 0.f), make_float2(dz, 0.f), make_float2(r2, FAR));
+                    make_float2(dy, 0.f), make_float2(dz, 0.f), make_float2(r2, FAR), o);
+                add(o.fr.x, o.B.x, o.ux.x, o.uy.x, o.uz.x, o.ee.x, dx, dy, dz);
+            }
         }
     }
-    float fx = Fx.x + Fx.y, fy = Fy.x + Fy.y, fz = Fz.x + Fz.y, hx = Hx.x + Hx.y, hy = Hy.x + Hy.y, hz = Hz.x + Hz.y;
     if (S > 1) {
 #pragma unroll
         for (int o = 1; o < S; o <<= 1) {
@@ -910,24 +948,13 @@ __device__ __forceinline__ void dev_pair32(const Dev &D, int unit) {
             }
         }
     }
-    // to real units
-    fx = fmaf(fx, R.out_hi[0], fx * R.out_lo[0]);
-    fy = fmaf(fy, R.out_hi[1], fy * R.out_lo[1]);
-    fz = fmaf(fz, R.out_hi[2], fz * R.out_lo[2]);
-    if (H) {
-        hx = fmaf(hx, R.out_hi[0], hx * R.out_lo[0]);
-        hy = fmaf(hy, R.out_hi[1], hy * R.out_lo[1]);
-        hz = fmaf(hz, R.out_hi[2], hz * R.out_lo[2]);
-    }
-    const float lx = R.fx_lsb[0], ly = R.fx_lsb[1], lz = R.fx_lsb[2];
+    const bool own = act && sub == 0;
     const int4 dfi = Q ? make_int4(0, 0, 0, 0) : img_diff(pi, H ? poi : D.po[i]);
     const float4 dri = make_float4((float)dfi.x * lx, (float)dfi.y * ly, (float)dfi.z * lz, 0.f);
-    const bool own = act && sub == 0;
     // harmonic bonds of Eq. 12 at any distance, from the exact r^2 where the
     // axes share one unit (r - r_b is a small difference of two numbers near
     // r_b); A = k (r - r_b)/r, B = k r_b / r^3
     if (R.nbond > 0 && own) {
-        float bx = 0.f, by = 0.f, bz = 0.f;
         for (int b = D.bond_off[i]; b < D.bond_off[i + 1]; ++b) {
             const int j = D.bond_j[b];
             const int4 pj = D.p[j];
@@ -936,15 +963,15 @@ __device__ __forceinline__ void dev_pair32(const Dev &D, int unit) {
             const int iz = (int)((unsigned)pi.z - (unsigned)pj.z);
             const float dx = (float)ix * lx, dy = (float)iy * ly, dz = (float)iz * lz;
             float r2h = fmaf(dx, dx, fmaf(dy, dy, dz * dz)), r2l = 0.f;
-            if (R.exact_r2) r2_split(R, ix, iy, iz, r2h, r2l);
+            if (exact) r2_split(R, ix, iy, iz, r2h, r2l);
             const float rh = sqrtf(r2h);
             const float rr = rh + (fmaf(-rh, rh, r2h) + r2l) * (0.5f / rh);
             const float db = (rr - R.rbond_hi) - R.rbond_lo;
             const float ir = 1.f / rr;
             const float A = R.kbondf * db * ir;
-            bx = fmaf(-A, dx, bx);
-            by = fmaf(-A, dy, by);
-            bz = fmaf(-A, dz, bz);
+            fx = fmaf(-A, dx, fx);
+            fy = fmaf(-A, dy, fy);
+            fz = fmaf(-A, dz, fz);
             if (E) e = fmaf(0.25f * R.kbondf * db, db, e);
             if (H) {
                 const int4 poj = D.po[j];
@@ -958,11 +985,11 @@ __device__ __forceinline__ void dev_pair32(const Dev &D, int unit) {
                 hz = fmaf(A, uz, fmaf(B, dz, hz));
             }
         }
-        // undo the FP32 rounding of the per-axis fixed-point unit
-        fx += fmaf(bx, R.lsb_rel[0], bx);
-        fy += fmaf(by, R.lsb_rel[1], by);
-        fz += fmaf(bz, R.lsb_rel[2], bz);
     }
+    // undo the FP32 rounding of the per-axis fixed-point unit (uniform per axis)
+    fx = fmaf(fx, R.lsb_rel[0], fx);
+    fy = fmaf(fy, R.lsb_rel[1], fy);
+    fz = fmaf(fz, R.lsb_rel[2], fz);
     const int role = own ? ((pi.w >> 8) & 0xff) : -1;
     if (H && role == ROLE_RIGID) {
         hx += R.kr_nf * dri.x;
@@ -1032,7 +1059,7 @@ __global__ void __launch_bounds__(256, H ? 3 : 4) k_pair32(Dev D, int sweep) {
 // Sweeps with the Hessian term over the listed replicas only; true in the
 // last CTA to finish (all others' results visible to it).  The list is empty
 // in most steps, so the grid is a fixed few CTAs an SM that stride over the
-// listed tiles.
+// listed tiles.  (In the split form only batches of one lane a row get here.)
 template <int PREC, int S>
 __device__ __forceinline__ bool sweep_listed(const Dev &D, const int *list, int n, unsigned *ticket) {
     int pos = blockIdx.x, base = 0;       // place in the listed replicas' tiles, one after another
@@ -2204,18 +2231,19 @@ void launch_rebuild(const Dev &D, cudaStream_t s) {
 template <int S>
 static void pair_of(const Dev &D, int kind, cudaStream_t s) {
     const int grid = D.ntile * D.split, n = unit_threads(D);
+    const bool hot = kind == PAIR_LAZY && D.bias_on;
     if (D.prec == HD_FP64) {
         if (kind == PAIR_QUENCH) k_pair64<true, false, false, S><<<grid, n, 0, s>>>(D, SWEEP_ALL);
         else if (kind == PAIR_ENERGY) k_pair64<false, true, true, S><<<grid, n, 0, s>>>(D, SWEEP_ALL);
         else if (kind == PAIR_FULL) k_pair64<false, false, true, S><<<grid, n, 0, s>>>(D, SWEEP_ALL);
         else k_pair64<false, false, false, S><<<grid, n, 0, s>>>(D, SWEEP_PLAIN);
-        if (kind == PAIR_LAZY && D.bias_on) k_pair_hot<HD_FP64, S><<<D.hot_grid, n, 0, s>>>(D);
+        if (hot) k_pair_hot<HD_FP64, S><<<D.hot_grid, n, 0, s>>>(D);
     } else {
         if (kind == PAIR_QUENCH) k_pair32<true, false, false, S><<<grid, n, 0, s>>>(D, SWEEP_ALL);
         else if (kind == PAIR_ENERGY) k_pair32<false, true, true, S><<<grid, n, 0, s>>>(D, SWEEP_ALL);
         else if (kind == PAIR_FULL) k_pair32<false, false, true, S><<<grid, n, 0, s>>>(D, SWEEP_ALL);
         else k_pair32<false, false, false, S><<<grid, n, 0, s>>>(D, SWEEP_PLAIN);
-        if (kind == PAIR_LAZY && D.bias_on) k_pair_hot<HD_FP32_SPLIT, S><<<D.hot_grid, n, 0, s>>>(D);
+        if (hot) k_pair_hot<HD_FP32_SPLIT, 1><<<D.hot_grid, n, 0, s>>>(D);
     }
 }
 void launch_pair(const Dev &D, int kind, cudaStream_t s) {
@@ -2227,13 +2255,9 @@ void launch_scalar(const Dev &D, int mode, bool lazy, bool list, cudaStream_t s)
     k_scalar<<<D.nrep, sc_threads(D), 0, s>>>(D, mode, lazy && more, list && more);
     if (!lazy || !more) return;
     const int n = unit_threads(D), g = D.hot_grid, li = list && more;
-    if (D.prec == HD_FP64) {
-        if (D.lanes == 4) k_scalar_late<HD_FP64, 4><<<g, n, 0, s>>>(D, mode, li);
-        else k_scalar_late<HD_FP64, 1><<<g, n, 0, s>>>(D, mode, li);
-    } else {
-        if (D.lanes == 4) k_scalar_late<HD_FP32_SPLIT, 4><<<g, n, 0, s>>>(D, mode, li);
-        else k_scalar_late<HD_FP32_SPLIT, 1><<<g, n, 0, s>>>(D, mode, li);
-    }
+    if (D.prec != HD_FP64) k_scalar_late<HD_FP32_SPLIT, 1><<<g, n, 0, s>>>(D, mode, li);
+    else if (D.lanes == 4) k_scalar_late<HD_FP64, 4><<<g, n, 0, s>>>(D, mode, li);
+    else k_scalar_late<HD_FP64, 1><<<g, n, 0, s>>>(D, mode, li);
 }
 void launch_update(const Dev &D, int mode, cudaStream_t s) {
     if (D.prec == HD_FP64) k_update64<<<D.ntile, nthr(D), 0, s>>>(D, mode);
