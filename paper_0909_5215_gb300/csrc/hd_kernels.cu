@@ -1106,7 +1106,8 @@ __global__ void __launch_bounds__(256, PREC == HD_FP64 ? 1 : 3) k_pair_hot(Dev D
 //   rigid-body force = sum_rigid F - gs - DeltaV' sum_rigid grad sigma;
 //   body kicks and the clocks: t_h += dt exp(DeltaV / kT) (Eq. 3).
 // need_hess: the caller has no H.dr of this configuration; with DeltaV' != 0
-// nothing is changed then and the result is false.
+// nothing is changed then and the result is false.  ksum: the mobile atoms'
+// kinetic energy, or null to leave S.K as it is.
 //
 // One warp evaluates it (every lane calls; S and C may be in shared or global
 // memory): lane a < 3 holds axis a.  The chain of FP64 operations is all of
@@ -1116,7 +1117,7 @@ __global__ void __launch_bounds__(256, PREC == HD_FP64 ? 1 : 3) k_pair_hot(Dev D
 // one thread for all of it, 22 divisions one after another, a step of 16 x 421
 // atoms in one launch took 30.8 us; it takes 19.3 now, and the kernel of 8 x
 // 1,983 atoms 13 us where it took 21.
-__device__ bool scalar_eval(const Dev &D, int r, int mode, const double *acc, double ksum, RepState &S, Scal &C,
+__device__ bool scalar_eval(const Dev &D, int r, int mode, const double *acc, const double *ksum, RepState &S, Scal &C,
                             bool need_hess = false) {
     const unsigned full = 0xffffffffu;
     const RepDev &R = D.rep[r];
@@ -1204,7 +1205,7 @@ __device__ bool scalar_eval(const Dev &D, int r, int mode, const double *acc, do
             S.step = step + 1;
             S.n_dv[dV <= 0.0 ? 0 : (dV >= R.dvmax ? 2 : 1)] += 1;
         }
-        S.K = ksum + 0.5 * (double)R.nrig * v2;
+        if (ksum) S.K = *ksum + 0.5 * (double)R.nrig * v2;
     }
     __syncwarp();
     return true;
@@ -1215,8 +1216,8 @@ __device__ bool scalar_eval(const Dev &D, int r, int mode, const double *acc, do
 // l % 16, and every warp takes every nw-th pair, so the loads are coalesced and
 // each lane adds its own slot; the warps' sums meet in shared memory in warp
 // order.  The order is a function of the block size alone.  MAXSLOT is reduced
-// with max (-1: none).
-template <int MAXSLOT>
+// with max (-1: none).  K: the kinetic parts are wanted.
+template <int MAXSLOT, bool K = true>
 __device__ __forceinline__ void dev_scalar_acc(const Dev &D, int r, double *acc) {
     __shared__ double sm[17][NPART + 1];
     const RepDev &R = D.rep[r];
@@ -1238,7 +1239,7 @@ __device__ __forceinline__ void dev_scalar_acc(const Dev &D, int r, double *acc)
     }
     const double o = __shfl_down_sync(0xffffffffu, v, 16);
     v = mx ? fmax(v, o) : v + o;
-    if (MAXSLOT < 0) {
+    if (K && MAXSLOT < 0) {
         for (int t = (int)threadIdx.x; t < R.ntile * D.ksplit; t += blockDim.x) k += D.kpart[R.tile0 * D.ksplit + t];
         k = warp_sum(k);
     }
@@ -1287,7 +1288,7 @@ __global__ void __launch_bounds__(SC_MAX) k_scalar(Dev D, int mode, int lazy, in
     dev_scalar_acc<-1>(D, r, acc);
     if (threadIdx.x < 32) {
         Scal &C = D.sc[r];
-        const bool done = scalar_eval(D, r, mode, acc, acc[NPART], D.st[r], C, lazy && !C.need_h);
+        const bool done = scalar_eval(D, r, mode, acc, acc + NPART, D.st[r], C, lazy && !C.need_h);
         if (threadIdx.x == 0) {
             if (!done) D.h_late[atomicAdd(D.h_meta + 1, 1)] = r;
             else if (D.lazy_h) expect_slope(D, r, D.st[r], C, list);
@@ -1312,7 +1313,7 @@ __global__ void __launch_bounds__(256, PREC == HD_FP64 ? 1 : 3) k_scalar_late(De
         const int r = D.h_late[q];
         dev_scalar_acc<-1>(D, r, acc);
         if (threadIdx.x < 32) {
-            scalar_eval(D, r, mode, acc, acc[NPART], D.st[r], D.sc[r]);
+            scalar_eval(D, r, mode, acc, acc + NPART, D.st[r], D.sc[r]);
             if (threadIdx.x == 0) expect_slope(D, r, D.st[r], D.sc[r], list);
         }
         __syncthreads();
@@ -2111,9 +2112,12 @@ __global__ void __launch_bounds__(128, 4) k_persist(Dev D, int nsteps) {
     }
     __syncthreads();
     GrpBar B = {0u, 0u, false};
+    // The kinetic parts are left alone here: a CTA that is through goes on to
+    // update() and writes its own while another may still be in here.  K is
+    // formed when it is read (k_obs).
     auto scalars = [&](int mode) {
-        dev_scalar_acc<-1>(D, r, acc);
-        if (threadIdx.x < 32) scalar_eval(D, r, mode, acc, acc[NPART], St, C);
+        dev_scalar_acc<-1, false>(D, r, acc);
+        if (threadIdx.x < 32) scalar_eval(D, r, mode, acc, nullptr, St, C);
         __syncthreads();
     };
     auto update = [&](int mode) {
@@ -2175,6 +2179,8 @@ __global__ void __launch_bounds__(128, 4) k_persist(Dev D, int nsteps) {
             update(MODE_CLOSE);
             if (!grp_barrier(D, r, nc, B, nullptr)) return;
             chain(mode);
+            // MODE_SCALE writes the kinetic sums that chain() has read
+            if (!(mode & MODE_OPEN) && !grp_barrier(D, r, nc, B, nullptr)) return;
             update((mode & MODE_OPEN) ? (MODE_OPEN | MODE_NHC) : MODE_SCALE);
         }
         if (!grp_barrier(D, r, nc, B, &s_moved)) return;
