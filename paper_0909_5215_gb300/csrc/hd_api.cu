@@ -447,7 +447,7 @@ struct hd_ctx {
     hd_status status = HD_OK;
     std::string err;
     int driver = HD_DRIVER_KERNELS;
-    int persistent_ctas = 0;
+    int persistent_ctas = 0, persist_steps = 0;   // CTAs of a persistent launch, steps it takes at most
     long long launches = 0;
     std::map<int, cudaGraphExec_t> graphs;
     std::map<std::string, cudaGraphExec_t> qgraphs;
@@ -871,7 +871,44 @@ bool setup_persistent(hd_ctx *c) {
         cudaMemcpyAsync((void *)c->D.pg_count, cnt.data(), P.nrep * 4, cudaMemcpyHostToDevice, c->s) != cudaSuccess)
         return false;
     c->persistent_ctas = (int)ctarep.size();
+    c->persist_steps = persist_steps_max(*std::max_element(cnt.begin(), cnt.end()));
     return true;
+}
+
+// One cooperative launch for n steps, replayed from a graph when the runtime
+// captures it; launched directly otherwise.
+hd_status persist_steps(hd_ctx *c, int n, bool can_graph) {
+    if (can_graph && c->persist_graph_ok) {
+        auto it = c->graphs.find(n);
+        if (it == c->graphs.end()) {
+            if (c->graphs.size() >= 8) {  // keep at most 8 step counts, as on the per-phase path
+                for (auto &gx : c->graphs) cudaGraphExecDestroy(gx.second);
+                c->graphs.clear();
+            }
+            cudaGraph_t g = nullptr;
+            cudaGraphExec_t ge = nullptr;
+            bool ok = cudaStreamBeginCapture(c->s, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
+            cudaError_t le = ok ? launch_persist(c->D, c->persistent_ctas, n, c->s) : cudaErrorUnknown;
+            cudaError_t ee = ok ? cudaStreamEndCapture(c->s, &g) : cudaErrorUnknown;
+            ok = ok && le == cudaSuccess && ee == cudaSuccess && g &&
+                 cudaGraphInstantiate(&ge, g, 0) == cudaSuccess;
+            if (g) cudaGraphDestroy(g);
+            (void)cudaGetLastError();
+            if (!ok) {
+                c->persist_graph_ok = false;
+            } else {
+                it = c->graphs.emplace(n, ge).first;
+            }
+        }
+        if (c->persist_graph_ok) {
+            CK(cudaGraphLaunch(it->second, c->s));
+            c->launches += 1;
+            return HD_OK;
+        }
+    }
+    CK(launch_persist(c->D, c->persistent_ctas, n, c->s));
+    c->launches += 1;
+    return HD_OK;
 }
 
 }  // namespace
@@ -1049,38 +1086,11 @@ hd_status hd_step(hd_ctx *c, int n_steps) {
     const bool can_graph = c->s != nullptr && cs == cudaStreamCaptureStatusNone;
     if (c->timing && !c->graph_pending.empty()) harvest_all(c);
     if (c->driver == HD_DRIVER_PERSISTENT) {
-        // one cooperative launch for all n steps, replayed from a graph when the
-        // runtime captures it; launched directly otherwise
-        if (can_graph && c->persist_graph_ok) {
-            auto it = c->graphs.find(n_steps);
-            if (it == c->graphs.end()) {
-                if (c->graphs.size() >= 8) {  // keep at most 8 step counts, as on the per-phase path
-                    for (auto &gx : c->graphs) cudaGraphExecDestroy(gx.second);
-                    c->graphs.clear();
-                }
-                cudaGraph_t g = nullptr;
-                cudaGraphExec_t ge = nullptr;
-                bool ok = cudaStreamBeginCapture(c->s, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-                cudaError_t le = ok ? launch_persist(c->D, c->persistent_ctas, n_steps, c->s) : cudaErrorUnknown;
-                cudaError_t ee = ok ? cudaStreamEndCapture(c->s, &g) : cudaErrorUnknown;
-                ok = ok && le == cudaSuccess && ee == cudaSuccess && g &&
-                     cudaGraphInstantiate(&ge, g, 0) == cudaSuccess;
-                if (g) cudaGraphDestroy(g);
-                (void)cudaGetLastError();
-                if (!ok) {
-                    c->persist_graph_ok = false;
-                } else {
-                    it = c->graphs.emplace(n_steps, ge).first;
-                }
-            }
-            if (c->persist_graph_ok) {
-                CK(cudaGraphLaunch(it->second, c->s));
-                c->launches += 1;
-                return HD_OK;
-            }
+        for (int left = n_steps; left > 0;) {
+            const int n = std::min(left, c->persist_steps);
+            if (persist_steps(c, n, can_graph) != HD_OK) return c->status;
+            left -= n;
         }
-        CK(launch_persist(c->D, c->persistent_ctas, n_steps, c->s));
-        c->launches += 1;
         return HD_OK;
     }
     if (!can_graph) {

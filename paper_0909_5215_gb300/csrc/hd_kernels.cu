@@ -2034,7 +2034,8 @@ __global__ void k_adopt(Dev Q, Dev M, const int *adopt) {
 // Phases of one replica are separated by that replica's own barrier: a 64-bit
 // counter in global memory (reset before each launch) whose low half counts
 // arrivals and whose high half counts CTAs that saw an atom move half the skin
-// in the update before.  An arrival releases the CTA's writes, the poll
+// in the update before (a call of very many steps is cut into launches, so the
+// low half never carries: persist_steps_max).  An arrival releases the CTA's writes, the poll
 // acquires the others'.  Polling is bounded: after ~2^24 polls the CTA records
 // HD_ERR_TIMEOUT, raises the abort word err[3], and every CTA leaves at its
 // next barrier.  The launch is cooperative, so all CTAs are resident.  A

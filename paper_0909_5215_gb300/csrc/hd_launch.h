@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include "hd_internal.cuh"
+#include "hd_units.h"
 
 namespace hd {
 
