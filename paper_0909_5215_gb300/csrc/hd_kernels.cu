@@ -1452,8 +1452,9 @@ __device__ __forceinline__ UpdateSpan update_tile(const Dev &D, int t) {
     return {t, D.tile_start[t], D.tile_n[t], t * D.ksplit, r, D.rebuild + r};
 }
 __device__ __forceinline__ UpdateSpan update_unit(const Dev &D, int unit, int *moved) {
-    const int t = unit / D.split, w = D.block / D.split, o = (unit % D.split) * w;
-    return {t, D.tile_start[t] + o, min(w, max(0, D.tile_n[t] - o)), unit, D.tile_rep[t], moved};
+    const int t = unit / D.split;
+    const UnitSpan a = unit_span(D.tile_start[t], D.tile_n[t], D.block / D.split, unit % D.split);
+    return {t, a.first, a.n, unit, D.tile_rep[t], moved};
 }
 
 __device__ __forceinline__ void dev_update64(const Dev &D, const UpdateSpan &U, int mode, const Scal &C) {

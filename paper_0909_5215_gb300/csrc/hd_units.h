@@ -25,4 +25,16 @@ HD_HOST_DEVICE int persist_steps_max(int nc) {
     return n > 0x7fffffffull ? 0x7fffffff : (int)n;
 }
 
+// Atoms of unit k of a tile of n atoms from slot `start` on, cut into units of
+// `width`.  A ragged tile leaves its last units short or empty; an empty one
+// starts at the tile's first atom, which its threads may load.
+struct UnitSpan {
+    int first, n;
+};
+HD_HOST_DEVICE UnitSpan unit_span(int start, int n, int width, int k) {
+    const int left = n - k * width;
+    if (left <= 0) return {start, 0};
+    return {start + k * width, left < width ? left : width};
+}
+
 }  // namespace hd

@@ -36,3 +36,15 @@ def test_arrivals_of_a_launch_stay_below_two_to_the_32(tmp_path):
     # and hd_step goes by it
     api = open(os.path.join(CSRC, "hd_api.cu")).read()
     assert "std::min(left, c->persist_steps)" in api and "persist_steps_max(" in api
+
+
+def test_units_stay_inside_their_tile(tmp_path):
+    """Every unit, also an empty one, starts at an atom of its tile, and a tile's units are its atoms, once each."""
+    out = compiled(tmp_path, 'for (int w = 8; w <= 32; w *= 2) for (int n = 1; n <= 128; ++n) for (int k = 0; k < 128 / w; ++k) {'
+                             ' const UnitSpan u = unit_span(1000, n, w, k); printf("%d %d %d %d %d\\n", w, n, k, u.first, u.n); }')
+    v = [tuple(map(int, out[q:q + 5])) for q in range(0, len(out), 5)]
+    atoms = {}
+    for w, n, k, first, m in v:
+        assert 1000 <= first < 1000 + n and 0 <= m <= w and first + m <= 1000 + n
+        atoms.setdefault((w, n), []).extend(range(first, first + m))
+    assert all(got == list(range(1000, 1000 + n)) for (w, n), got in atoms.items())
