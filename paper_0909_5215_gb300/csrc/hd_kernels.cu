@@ -13,6 +13,10 @@
 //
 // Tiles: a CTA handles one tile = up to blockDim atoms of ONE replica, so any
 // per-replica quantity is a fixed-order sum of per-tile sums (deterministic).
+#include <map>
+#include <mutex>
+#include <utility>
+
 #include "hd_internal.cuh"
 #include "hd_launch.h"
 
@@ -2209,15 +2213,31 @@ static persist_fn persist_kernel(const Dev &D) {
     if (D.prec == HD_FP64) return D.lanes == 4 ? k_persist<HD_FP64, 4> : k_persist<HD_FP64, 1>;
     return D.lanes == 4 ? k_persist<HD_FP32_SPLIT, 4> : k_persist<HD_FP32_SPLIT, 1>;
 }
+// Lets kernel f use `bytes` of dynamic shared memory.  The limit belongs to the
+// kernel on a device, not to a context, and contexts of different size live
+// side by side, so it is never lowered.
+static cudaError_t allow_smem(const void *f, int bytes) {
+    static std::mutex mu;
+    static std::map<std::pair<int, const void *>, int> most;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lk(mu);
+    int &m = most[std::make_pair(dev, f)];
+    const int want = bytes > m ? bytes : m;
+    e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, want);
+    if (e == cudaSuccess) m = want;
+    return e;
+}
 cudaError_t nl_configure(const Dev &D, int *nl_blocks_per_sm) {
     const int bytes = (int)nl_smem_bytes(D, NL_THREADS / 32), pbytes = (int)persist_smem_bytes(D);
-    cudaError_t e = cudaFuncSetAttribute(k_nlist, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    cudaError_t e = allow_smem((const void *)k_nlist, bytes);
     if (e != cudaSuccess) return e;
     // the row builder is latency-bound: launch as many CTAs as fit
     *nl_blocks_per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(nl_blocks_per_sm, k_nlist, NL_THREADS, bytes);
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(persist_kernel(D), cudaFuncAttributeMaxDynamicSharedMemorySize, pbytes);
+    return allow_smem((const void *)persist_kernel(D), pbytes);
 }
 
 void launch_init(const Dev &D, const int *draw_vel, cudaStream_t s) {
