@@ -266,10 +266,11 @@ hd_status hd_timing(hd_ctx *ctx, int enable, double out[16]);
  * call at start-up, before reserving memory, or run with
  * CUDA_MODULE_LOADING=EAGER.  Every call synchronises cuda_stream (it reads
  * back an error word), so it cannot be called while that stream is being
- * captured.  Every call shares
- * the array and leaves its contents behind; counts, extent and the error
- * word are cleared at the start of each call, and calls that overlap on the
- * GPU race.  Returns HD_ERR_OVERFLOW if a row or a cell exceeded its
+ * captured.  Every call shares the array and leaves its contents behind;
+ * counts, extent and the error word are cleared at the start of each call.
+ * Calls on one GPU take turns, whichever threads and streams they come from:
+ * the stream given must not wait for work that another thread queues after
+ * its own call.  Returns HD_ERR_OVERFLOW if a row or a cell exceeded its
  * capacity, HD_ERR_NUMERIC for a non-finite position on an open axis. */
 hd_status hd_nlist_static(const double *d_pos, int n_atoms, const double box[3], const uint8_t periodic[3],
                           double rl, int maxnb, int32_t *d_nbr, int32_t *d_nnb, void *cuda_stream);

@@ -18,8 +18,10 @@
 // synchronises its stream (it reads back the error word), so no call may be
 // made while that stream is being captured into a graph.  Every call shares the array and
 // it keeps the last call's contents: the counts, the extent and the error
-// word are cleared at the start of each call, and calls that overlap on the
-// GPU race.
+// word are cleared at the start of each call.  Calls on one device therefore
+// take turns: each holds that device's lock from its first launch until its
+// stream is synchronised.  (The row build takes the grid and the atoms from the
+// array, so a call that overlapped another would write rows of its atoms.)
 #include <algorithm>
 #include <cmath>
 #include <cstddef>
@@ -323,7 +325,7 @@ __global__ void __launch_bounds__(S_THREADS) k_s_list(StaticScratch *S, const do
     }
 }
 
-std::mutex g_mu;
+std::mutex g_mu[64];
 StaticScratch *g_addr[64] = {};
 
 }  // namespace
@@ -336,16 +338,13 @@ extern "C" hd_status hd_nlist_static(const double *d_pos, int n_atoms, const dou
     if (maxnb <= 0 || maxnb > S_MAX_NB || !(rl > 0.0)) return HD_ERR_ARG;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return HD_ERR_CUDA;
-    StaticScratch *S;
-    {
-        std::lock_guard<std::mutex> lk(g_mu);
-        if (!g_addr[dev]) {
-            void *p = nullptr;
-            if (cudaGetSymbolAddress(&p, g_static_scratch) != cudaSuccess || !p) return HD_ERR_CUDA;
-            g_addr[dev] = static_cast<StaticScratch *>(p);
-        }
-        S = g_addr[dev];
+    std::lock_guard<std::mutex> lk(g_mu[dev]);
+    if (!g_addr[dev]) {
+        void *p = nullptr;
+        if (cudaGetSymbolAddress(&p, g_static_scratch) != cudaSuccess || !p) return HD_ERR_CUDA;
+        g_addr[dev] = static_cast<StaticScratch *>(p);
     }
+    StaticScratch *S = g_addr[dev];
     cudaStream_t s = (cudaStream_t)cuda_stream;
     Grid G;
     memset(&G, 0, sizeof G);
