@@ -707,6 +707,9 @@ hd_status upload_reps(hd_ctx *c) {
     return HD_OK;
 }
 
+// Kernels of a list rebuild (launch_rebuild).
+int rebuild_kernels(const hd_ctx *c) { return c->P.nrep > PLAN_MAX ? 4 : 3; }
+
 // Kernels of one BAOAB step after the opening half (list, pair, scalars, update).
 // next_last: the step after this one is the last of its call.
 void queue_step(hd_ctx *c, int mode, bool next_last, std::vector<hd_ctx::Span> *sink) {
@@ -720,7 +723,7 @@ void queue_step(hd_ctx *c, int mode, bool next_last, std::vector<hd_ctx::Span> *
     c->launches += (c->D.any_eig ? 2 : 0) + (lazy && c->D.bias_on ? 2 : 0);
     if (!c->D.any_nhc) {
         { Timed t(c, sink, T_UPDATE); launch_update(c->D, mode, c->s); }
-        c->launches += 6;
+        c->launches += 3 + rebuild_kernels(c);
         return;
     }
     // a Nose-Hoover chain needs the kinetic sums of the closing kick before
@@ -728,7 +731,7 @@ void queue_step(hd_ctx *c, int mode, bool next_last, std::vector<hd_ctx::Span> *
     { Timed t(c, sink, T_UPDATE); launch_update(c->D, MODE_CLOSE, c->s); }
     launch_nhc(c->D, mode, c->s);
     { Timed t(c, sink, T_UPDATE); launch_update(c->D, (mode & MODE_OPEN) ? (MODE_OPEN | MODE_NHC) : MODE_SCALE, c->s); }
-    c->launches += 8;
+    c->launches += 5 + rebuild_kernels(c);
 }
 
 void queue_steps(hd_ctx *c, int n, std::vector<hd_ctx::Span> *sink) {
@@ -749,7 +752,7 @@ hd_status refresh_md(hd_ctx *c, bool relist) {
         CK(cudaMemcpyAsync(c->D.rebuild, two.data(), two.size() * 4, cudaMemcpyHostToDevice, c->s));
         c->h2d += (long long)two.size() * 4;
         launch_rebuild(c->D, c->s);
-        c->launches += 3;
+        c->launches += rebuild_kernels(c);
         CK(cudaStreamSynchronize(c->s));
     }
     launch_pair(c->D, PAIR_ENERGY, c->s);
@@ -1024,7 +1027,7 @@ hd_status hd_create(const hd_replica_desc *reps, int n_rep, const hd_params *p, 
     launch_update(c->D, MODE_KIN, c->s);  // kinetic energy of the initial velocities
     launch_nhc(c->D, MODE_KIN, c->s);     // the chains start from it
     launch_obs(c->D, c->s);
-    c->launches += 9 + (c->D.any_eig ? 2 : 0);
+    c->launches += 6 + rebuild_kernels(c) + (c->D.any_eig ? 2 : 0);
     CK(cudaGetLastError());
     c->qdisp.assign(P.nrep, 0.0);
     c->qflag.assign(P.nrep, 0);
@@ -1127,8 +1130,8 @@ hd_status hd_step(hd_ctx *c, int n_steps) {
     }
     CK(cudaGraphLaunch(it->second, c->s));
     if (c->timing) c->graph_pending.push_back(key);
-    c->launches += (c->D.any_nhc ? 3 + 8LL * n_steps : 2 + 6LL * n_steps) + (c->D.any_eig ? 2LL * n_steps : 0) +
-                   (c->D.lazy_h && c->D.bias_on ? 2LL * (n_steps - 1) : 0);
+    c->launches += (c->D.any_nhc ? 3 + 5LL * n_steps : 2 + 3LL * n_steps) + (long long)rebuild_kernels(c) * n_steps +
+                   (c->D.any_eig ? 2LL * n_steps : 0) + (c->D.lazy_h && c->D.bias_on ? 2LL * (n_steps - 1) : 0);
     return HD_OK;
 }
 
@@ -1181,7 +1184,7 @@ hd_status hd_quench(hd_ctx *c, int method, double ftol, int max_iter, double ste
         if (qg) CK(cudaGraphLaunch(qg, c->s));
         else
             for (int k = 0; k < chunk; ++k) launch_qiter(Q, max_iter, c->s);
-        c->launches += 6LL * chunk;
+        c->launches += (3LL + rebuild_kernels(c)) * chunk;
         done_iters += chunk;
         CK(cudaGetLastError());
         CK(cudaMemcpyAsync(st.data(), c->D.st, R * sizeof(RepState), cudaMemcpyDeviceToHost, c->s));

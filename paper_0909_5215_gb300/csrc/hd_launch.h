@@ -12,7 +12,7 @@ void launch_init(const Dev &D, const int *draw_vel, cudaStream_t s);
 // replicas whose rebuild plan each CTA of the binning makes in its shared memory; with
 // more of them a kernel of its own makes it first
 constexpr int PLAN_MAX = 4000;
-void launch_rebuild(const Dev &D, cudaStream_t s);            // 3 kernels, flag-gated per replica
+void launch_rebuild(const Dev &D, cudaStream_t s);            // 3 kernels (4 above PLAN_MAX), flag-gated per replica
 void launch_rebuild_prep(const Dev &D, cudaStream_t s);       // the first 2: plan and bin, cell sort
 void launch_nlist(const Dev &D, cudaStream_t s);              // the 3rd: rows from the cells
 // FULL: force and H.(r - r_O); ENERGY: per-atom LJ energies too (observables, not

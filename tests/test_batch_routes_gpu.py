@@ -35,9 +35,12 @@ def test_plan_of_more_than_4000_replicas(hd, oracle_mod):
     p = M.Params(prec=0, bias_on=0)
     a = hd.Batch(reps, p, driver=hd.HD_DRIVER_KERNELS)
     b = hd.Batch([reps[k] for k in some], p, driver=hd.HD_DRIVER_KERNELS)
+    at = a.info()["launches"], b.info()["launches"]
     for n in (1, 40):
         a.step(n)
         b.step(n)
+    # the plan is a kernel of its own
+    assert b.info()["launches"] - at[1] == 2 * 2 + 6 * 41 and a.info()["launches"] - at[0] == 2 * 2 + 7 * 41
     oa, ob = a.obs(), b.obs()
     assert ob[:, NREB].max() > 0 and (oa[:, NREB] > 0).sum() > 100
     for q, k in enumerate(some):
