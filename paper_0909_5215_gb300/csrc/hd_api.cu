@@ -241,8 +241,6 @@ bool make_plan(const hd_replica_desc *reps, int n_rep, const hd_params *p, Plan 
         R.boost_max = std::exp(d.dvmax / d.kT);
         R.c_ou = std::exp(-d.gamma * p->dt);
         R.s_ou = std::sqrt((1.0 - R.c_ou * R.c_ou) * d.kT);
-        R.c_ouf = (float)R.c_ou;
-        R.s_ouf = (float)R.s_ou;
         R.kspring = d.k_spring;
         R.fnormal = d.f_normal;
         R.slider[0] = d.slider[0];
@@ -260,7 +258,6 @@ bool make_plan(const hd_replica_desc *reps, int n_rep, const hd_params *p, Plan 
                 R.sig2[a][b] = sig * sig;
                 R.shift[a][b] = 4.0 * eps * (sc6 * sc6 - sc6);
                 R.epsf[a][b] = (float)eps;
-                R.sig2f[a][b] = (float)(sig * sig);
                 R.shiftf[a][b] = (float)R.shift[a][b];
                 const double r0sq = std::cbrt(2.0) * sig * sig;   // LJ minimum 2^(1/6) sigma, squared
                 R.r0sq_hi[a][b] = (float)r0sq;
@@ -639,8 +636,6 @@ void fill_dev(hd_ctx *c) {
     D.ey = at<double>(b, P.o_ey);
     D.ecoef = at<double>(b, P.o_ecoef);
     D.epart = at<double>(b, P.o_epart);
-    D.nl_pow2 = 32;
-    while (D.nl_pow2 < P.maxnb) D.nl_pow2 <<= 1;
     {
         int dev = 0, nsm = 148;
         cudaGetDevice(&dev);

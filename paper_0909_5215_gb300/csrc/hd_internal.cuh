@@ -76,7 +76,7 @@ struct RepDev {
     long long slide_step0;       // step count of the configuration at which slider[0] was set
     double dvmax, sig_lo, sig_hi;
     double eps[2][2], sig2[2][2], shift[2][2];
-    float epsf[2][2], sig2f[2][2], shiftf[2][2];
+    float epsf[2][2], shiftf[2][2];
     // fine fixed point of the pair sweep: q = rint(x * scale - origin * scale)
     // mod 2^32, taken as the low word of fma(x, scale, fx_add) with
     // fx_add = 1.5 2^52 - origin * scale (a common offset of at most half a
@@ -88,7 +88,7 @@ struct RepDev {
     double cell_lo, cell_inv_w;  // open axis: origin and inverse width of the cell grid
     double open_lim;             // escape bound |x - origin| on the open axis
     double kr_n;                 // k / n_rig (spring Hessian per rigid atom)
-    float kr_nf, c_ouf, s_ouf, pad1;
+    float kr_nf, pad1;
     // exact squared distances: all axes share one fixed-point unit u (the open
     // axis counts 2^zshift units per step); u^2 = lsb2_hi + lsb2_lo
     int exact_r2, zshift, shift_y, shift_z;
@@ -180,7 +180,7 @@ struct Dev {
     const int *pg_first, *pg_count;  // persistent launch: first CTA and CTA count of each replica
     const int *bond_off, *bond_j;    // per slot: bond partners (slots) in bond_j[bond_off[i] .. bond_off[i+1])
     int fault_rep;               // test hook (-1 off): a CTA of this replica skips one barrier arrival
-    int nl_pow2, nl_grid;        // neighbour-row buffer (power of two >= maxnb), k_nlist CTAs
+    int nl_grid;                 // k_nlist CTAs
     int any_nhc;                 // some replica runs a Nose-Hoover chain: the update splits around it
     int any_eig;                 // some replica has the eigenvalue bias
     dbl4 *eq, *ev, *ew, *eg;     // eigenvalue bias: Krylov bases, eigenvector, work vector, grad epsilon
