@@ -353,7 +353,7 @@ bool make_plan(const hd_replica_desc *reps, int n_rep, const hd_params *p, Plan 
     P.cell_cap = p->cell_cap > 0 ? p->cell_cap : ((2 * max_occ + 8 + 7) / 8) * 8;
     // Lanes that share a row of the pair sweep: with a thread a row, batches of
     // fewer than ~8 warps an SM leave it waiting for its gathers (8 x 1,983
-    // atoms: 34.5 us a sweep with 1, 20.9 with 4; 8 x 113 atoms, FP64, one
+    // atoms: 26.8 us a sweep with 1, 20.0 with 4; 8 x 113 atoms, FP64, one
     // launch: 66.6 and 47.7 us a step); beyond that the split only adds work
     // (57,088 atoms FP64: 513 us with 1, 570 with 4).
     P.lanes = P.split = P.natom / 32 < 152 * 8 ? 4 : 1;
@@ -952,10 +952,11 @@ hd_status hd_create(const hd_replica_desc *reps, int n_rep, const hd_params *p, 
     // Leave the Hessian term out of the sweeps where it is not used: always
     // without a bias; with one, where the sweep is long enough to pay for the
     // two launches more (~5 us) that a step then takes.  Measured per sweep with
-    // and without it: 259 and 122 to 143 us at 913,408 atoms (split form), 54 and 49
-    // at 121,000, where the launches cost what it saves; 514 and 327 us at
-    // 57,088 in the FP64 form, whose pipe the term fills.  The eigenvalue bias
-    // keeps the plain order.
+    // and without it: 322 and 172 us at 913,408 atoms (split form), 105 and 61 at
+    // 228,352, 55 and 40 at 114,176; 517 and 315 us at 57,088 in the FP64 form,
+    // whose pipe the term fills.  (The split form's line dates from a sweep that
+    // took 54 and 49 us at 121,000 atoms; where it would lie now has not been
+    // measured.)  The eigenvalue bias keeps the plain order.
     c->D.lazy_h = !c->P.any_eig && (!c->D.bias_on || c->P.natom >= (c->P.prec == HD_FP64 ? 8192 : 200000));
     Plan &P = c->P;
     const size_t N = P.natom;

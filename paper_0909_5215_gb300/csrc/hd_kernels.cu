@@ -1119,8 +1119,8 @@ __global__ void __launch_bounds__(256, PREC == HD_FP64 ? 1 : 3) k_pair_hot(Dev D
 // other quotients by reciprocals that the host set, the exponential only
 // inside the band (its value at DeltaV_max is the host's, at 0 it is 1).  With
 // one thread for all of it, 22 divisions one after another, a step of 16 x 421
-// atoms in one launch took 30.8 us; it takes 19.3 now, and the kernel of 8 x
-// 1,983 atoms 13 us where it took 21.
+// atoms in one launch took 30.8 us; with the warp it took 19.3, and the kernel of
+// 8 x 1,983 atoms 13 us where it took 21.
 __device__ bool scalar_eval(const Dev &D, int r, int mode, const double *acc, const double *ksum, RepState &S, Scal &C,
                             bool need_hess = false) {
     const unsigned full = 0xffffffffu;
@@ -1263,7 +1263,7 @@ __device__ __forceinline__ void dev_scalar_acc(const Dev &D, int r, double *acc)
 // the band of Eq. 14; sigma itself needs the forces alone.  So the sweeps of
 // a large batch leave the Hessian term out for the replicas that are not
 // expected in their band (lazy = 1): it costs the sweep a second gather and
-// about 40% of its instructions.  After each evaluation the next slope is
+// nearly doubles its time (322 and 172 us at 913,408 atoms).  After each evaluation the next slope is
 // expected within two of the largest recent changes of the slope; a replica
 // whose band reaches there goes on the list that k_pair_hot sweeps with H.  If
 // another one lands in its band all the same, its evaluation is put off
