@@ -351,12 +351,9 @@ bool make_plan(const hd_replica_desc *reps, int n_rep, const hd_params *p, Plan 
         for (int i = 0; i < P.natom; ++i) P.bond_j.insert(P.bond_j.end(), part[i].begin(), part[i].end());
     }
     P.cell_cap = p->cell_cap > 0 ? p->cell_cap : ((2 * max_occ + 8 + 7) / 8) * 8;
-    // Lanes that share a row of the pair sweep: with a thread a row, batches of
-    // fewer than ~8 warps an SM leave it waiting for its gathers (8 x 1,983
-    // atoms: 26.8 us a sweep with 1, 20.0 with 4; 8 x 113 atoms, FP64, one
-    // launch: 66.6 and 47.7 us a step); beyond that the split only adds work
-    // (57,088 atoms FP64: 513 us with 1, 570 with 4).
-    P.lanes = P.split = P.natom / 32 < 152 * 8 ? 4 : 1;
+    long long natom3 = 0;
+    for (int r = 0; r < n_rep; ++r) natom3 += reps[r].dim == 3 ? reps[r].n_atoms : 0;
+    P.lanes = P.split = row_lanes(P.natom, natom3, P.prec == HD_FP64, p->driver == HD_DRIVER_PERSISTENT);
     // The persistent launch cuts tiles into smaller units while SMs are idle:
     // 8 atoms (one warp) up to 4,864 atoms, 16 up to 9,728 (4 CTAs an SM).
     if (p->driver == HD_DRIVER_PERSISTENT && P.lanes == 4)
