@@ -36,6 +36,7 @@ constexpr int S_MAX_ATOMS = 65536;
 constexpr int S_MAX_CELLS = 16384;
 constexpr int S_CELL_CAP = 64;
 constexpr int S_MAX_NB = 160;
+constexpr int S_SPARSE = 6;      // mean atoms a cell below which the row build takes a warp a row
 constexpr int S_THREADS = 256;   // row build: 8 warps share one cell's staged stencil
 
 struct Grid {
@@ -187,27 +188,114 @@ __global__ void k_s_bin(StaticScratch *S, Grid G0, double bx, double by, double 
         const long long v = __double2ll_rn((pos[3 * i + a] - G.origin[a]) * G.scale[a]);
         q[a] = (int)(unsigned int)(unsigned long long)v;
     }
-    S->pfix[i] = make_int4(q[0], q[1], q[2], 0);
     const int cx = s_cell(G, 0, q[0], pos[3 * i]), cy = s_cell(G, 1, q[1], pos[3 * i + 1]),
               cz = s_cell(G, 2, q[2], pos[3 * i + 2]);
     const int c = (cz * G.nc[1] + cy) * G.nc[0] + cx;
+    S->pfix[i] = make_int4(q[0], q[1], q[2], c);
     const int slot = atomicAdd(&S->cell_cnt[c], 1);
     if (slot < S_CELL_CAP) S->cell_atoms[c * S_CELL_CAP + slot] = i;
     else atomicCAS(&S->err[0], 0, HD_ERR_OVERFLOW);
 }
 
-// Row i: every j != i with FP64 minimum-image r^2 < rl^2 (the FP32 test on
-// exact fixed-point differences decides outside a thin band), ascending j.
+// Stencil cell of `lane` around cell c: (lane % 3, lane / 3 % 3, lane / 9) of
+// -1, 0, 1 along each axis, as far as it exists; its atoms (0 where there is none).
+__device__ __forceinline__ int s_stencil(const StaticScratch *S, const Grid &G, int c, int lane, int &cell) {
+    const int ci[3] = {c % G.nc[0], (c / G.nc[0]) % G.nc[1], c / (G.nc[0] * G.nc[1])};
+    const int d[3] = {lane % 3 - 1, (lane / 3) % 3 - 1, lane / 9 - 1};
+    bool ok = lane < 27;
+    int q[3];
+    for (int a = 0; a < 3; ++a) {
+        q[a] = ci[a] + d[a];
+        if (G.nc[a] == 1) {
+            ok = ok && d[a] == 0;
+            q[a] = 0;
+        } else if (G.periodic[a]) {
+            q[a] = (q[a] + G.nc[a]) % G.nc[a];
+        } else {
+            ok = ok && q[a] >= 0 && q[a] < G.nc[a];
+        }
+    }
+    cell = ok ? (q[2] * G.nc[1] + q[1]) * G.nc[0] + q[0] : 0;
+    return ok ? min(S->cell_cnt[cell], S_CELL_CAP) : 0;
+}
+
+// Sum over the lanes up to this one.
+__device__ __forceinline__ int s_scan(int v, int lane) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += t;
+    }
+    return v;
+}
+
+// Is j (image pj) in row i: the FP32 test on exact fixed-point differences
+// decides outside a thin band.
+__device__ __forceinline__ bool s_in(const Grid &G, const double *pos, int i, int4 pi, int j, int4 pj) {
+    if (j == i) return false;
+    const float dx = (float)(int)((unsigned)pi.x - (unsigned)pj.x) * G.lsb[0];
+    const float dy = (float)(int)((unsigned)pi.y - (unsigned)pj.y) * G.lsb[1];
+    const float dz = (float)(int)((unsigned)pi.z - (unsigned)pj.z) * G.lsb[2];
+    const float r2 = dx * dx + dy * dy + dz * dz;
+    if (r2 < G.rl2_lo) return true;
+    if (r2 >= G.rl2_hi) return false;
+    return s_r2(G, pos + 3 * (size_t)i, pos + 3 * (size_t)j) < G.rl2;
+}
+
+// A warp adds its accepted candidates to the row in buf (cnt so far).
+__device__ __forceinline__ int s_add(bool in, int j, int lane, int maxnb, int cnt, int *buf) {
+    const unsigned hit = __ballot_sync(0xffffffffu, in);
+    const int at = cnt + __popc(hit & ((1u << lane) - 1u));
+    if (in && at < maxnb) buf[at] = j;
+    return cnt + __popc(hit);
+}
+
+// The warp sorts the cnt entries in buf by rank (the count of smaller ones)
+// and writes row i.
+__device__ __forceinline__ void s_write_row(StaticScratch *S, int i, int cnt, int maxnb, int lane, int *buf, int *srt,
+                                            int *nbr, int *nnb) {
+    if (cnt > maxnb) {
+        if (lane == 0) atomicCAS(&S->err[0], 0, HD_ERR_OVERFLOW);
+        cnt = maxnb;
+    }
+    // fill the last group of four so that it ranks after every entry
+    if (lane < 4 && (cnt & ~3) + lane >= cnt && (cnt & ~3) + lane < S_MAX_NB) buf[(cnt & ~3) + lane] = 0x7fffffff;
+    __syncwarp();
+    const int4 *b4 = reinterpret_cast<const int4 *>(buf);
+    for (int k = lane; k < cnt; k += 32) {
+        const int v = buf[k];
+        int rank = 0;
+        for (int q = 0; q < (cnt + 3) >> 2; ++q) {
+            const int4 u = b4[q];
+            rank += (u.x < v) + (u.y < v) + (u.z < v) + (u.w < v);
+        }
+        srt[rank] = v;
+    }
+    __syncwarp();
+    int *row = nbr + (size_t)i * maxnb;
+    for (int k = lane; k < maxnb; k += 32) row[k] = k < cnt ? srt[k] : -1;
+    if (lane == 0) nnb[i] = cnt;
+    __syncwarp();
+}
+
+// Row i: every j != i with FP64 minimum-image r^2 < rl^2, ascending j.
 //
 // One CTA builds the rows of one cell's atoms: it stages the cell's stencil
 // (27 cells, ~675 candidates in a dense crystal) in shared memory once, then
 // a warp per atom tests 32 candidates at a time, packs the accepted ones by
-// ballot and sorts them by rank (the count of smaller entries, read four at a
-// time from shared memory).  Both loops are issue-bound: ~21 x 20 + 480
+// ballot and sorts them by rank (read four at a time from shared memory).
+// Both loops are issue-bound: ~21 x 20 + 480
 // instructions an atom.  A thread per atom that kept its row sorted in global
 // memory by insertion made a call at 14,272 atoms (rows of 76) take 978 us;
 // with this build, and one wait for the GPU instead of two, it takes 92 us.
-__global__ void __launch_bounds__(S_THREADS) k_s_list(StaticScratch *S, const double *pos, int maxnb, int *nbr,
+//
+// Where cells hold few atoms (below S_SPARSE on the average: a gas, a thin
+// film under much vacuum) a CTA a cell leaves most warps without a row and
+// waits at the staging barriers instead.  There a warp takes a row by itself
+// and reads the candidates where they lie: 20,000 atoms in 15,625 cells 59 us
+// a call, with a CTA a cell 143, with a thread an atom 120.  1,728 cells of 6
+// atoms on the average 50 us and 58, of 8 atoms 69 and 62, of 12 94 and 82.
+__global__ void __launch_bounds__(S_THREADS) k_s_list(StaticScratch *S, const double *pos, int n, int maxnb, int *nbr,
                                                      int *nnb) {
     __shared__ Grid G;
     __shared__ int s_off[28], s_cell_id[27], s_nst;
@@ -217,39 +305,38 @@ __global__ void __launch_bounds__(S_THREADS) k_s_list(StaticScratch *S, const do
     if (threadIdx.x == 0) G = S->grid;
     __syncthreads();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const unsigned full = 0xffffffffu, below = (1u << lane) - 1u;
+    const unsigned full = 0xffffffffu;
+    if (n < S_SPARSE * G.ncell) {
+        for (int i = blockIdx.x * (S_THREADS / 32) + w; i < n; i += gridDim.x * (S_THREADS / 32)) {
+            const int4 pi = S->pfix[i];
+            int cell;
+            const int mine = s_stencil(S, G, pi.w, lane, cell), incl = s_scan(mine, lane);
+            const int tot = __shfl_sync(full, incl, 31), first = cell * S_CELL_CAP - (incl - mine);
+            int cnt = 0;
+            for (int base = 0; base < tot; base += 32) {
+                const int t = base + lane;
+                int k = 0;        // stencil cell of candidate t: the first one whose sum is above t
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1)
+                    if (__shfl_sync(full, incl, k + o - 1) <= t) k += o;
+                const int at = __shfl_sync(full, first, k) + t;
+                const int j = t < tot ? S->cell_atoms[at] : i;
+                cnt = s_add(s_in(G, pos, i, pi, j, S->pfix[j]), j, lane, maxnb, cnt, buf[w]);
+            }
+            s_write_row(S, i, cnt, maxnb, lane, buf[w], srt[w], nbr, nnb);
+        }
+        return;
+    }
     for (int c = blockIdx.x; c < G.ncell; c += gridDim.x) {
         const int m = min(S->cell_cnt[c], S_CELL_CAP);
         if (m == 0) continue;   // the same for every thread
         if (w == 0) {
-            // lane k: stencil cell (k % 3, k / 3 % 3, k / 9) of -1, 0, 1 along each axis
-            const int ci[3] = {c % G.nc[0], (c / G.nc[0]) % G.nc[1], c / (G.nc[0] * G.nc[1])};
-            const int d[3] = {lane % 3 - 1, (lane / 3) % 3 - 1, lane / 9 - 1};
-            bool ok = lane < 27;
-            int q[3];
-            for (int a = 0; a < 3; ++a) {
-                q[a] = ci[a] + d[a];
-                if (G.nc[a] == 1) {
-                    ok = ok && d[a] == 0;
-                    q[a] = 0;
-                } else if (G.periodic[a]) {
-                    q[a] = (q[a] + G.nc[a]) % G.nc[a];
-                } else {
-                    ok = ok && q[a] >= 0 && q[a] < G.nc[a];
-                }
-            }
-            const int cc = ok ? (q[2] * G.nc[1] + q[1]) * G.nc[0] + q[0] : 0;
-            const int cnt = ok ? min(S->cell_cnt[cc], S_CELL_CAP) : 0;
-            int incl = cnt;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int t = __shfl_up_sync(full, incl, o);
-                if (lane >= o) incl += t;
-            }
+            int cell;
+            const int cnt = s_stencil(S, G, c, lane, cell), incl = s_scan(cnt, lane);
             const unsigned has = __ballot_sync(full, cnt > 0);
             if (cnt > 0) {
-                const int k = __popc(has & below);
-                s_cell_id[k] = cc;
+                const int k = __popc(has & ((1u << lane) - 1u));
+                s_cell_id[k] = cell;
                 s_off[k] = incl - cnt;
             }
             if (lane == 31) {
@@ -270,56 +357,15 @@ __global__ void __launch_bounds__(S_THREADS) k_s_list(StaticScratch *S, const do
             }
         }
         __syncthreads();
-        const float lx = G.lsb[0], ly = G.lsb[1], lz = G.lsb[2];
         for (int a = w; a < m; a += S_THREADS / 32) {
             const int i = S->cell_atoms[c * S_CELL_CAP + a];
             const int4 pi = S->pfix[i];
             int cnt = 0;
             for (int base = 0; base < tot; base += 32) {
-                bool in = false;
-                int j = 0;
-                if (base + lane < tot) {
-                    const int4 pj = sp[base + lane];
-                    j = pj.w;
-                    if (j != i) {
-                        const float dx = (float)(int)((unsigned)pi.x - (unsigned)pj.x) * lx;
-                        const float dy = (float)(int)((unsigned)pi.y - (unsigned)pj.y) * ly;
-                        const float dz = (float)(int)((unsigned)pi.z - (unsigned)pj.z) * lz;
-                        const float r2 = dx * dx + dy * dy + dz * dz;
-                        if (r2 < G.rl2_lo) in = true;
-                        else if (r2 >= G.rl2_hi) in = false;
-                        else in = s_r2(G, pos + 3 * (size_t)i, pos + 3 * (size_t)j) < G.rl2;
-                    }
-                }
-                const unsigned hit = __ballot_sync(full, in);
-                if (in) {
-                    const int at = cnt + __popc(hit & below);
-                    if (at < maxnb) buf[w][at] = j;
-                }
-                cnt += __popc(hit);
+                const int4 pj = base + lane < tot ? sp[base + lane] : make_int4(0, 0, 0, i);
+                cnt = s_add(s_in(G, pos, i, pi, pj.w, pj), pj.w, lane, maxnb, cnt, buf[w]);
             }
-            if (cnt > maxnb) {
-                if (lane == 0) atomicCAS(&S->err[0], 0, HD_ERR_OVERFLOW);
-                cnt = maxnb;
-            }
-            // fill the last group of four so that it ranks after every entry
-            if (lane < 4 && (cnt & ~3) + lane >= cnt && (cnt & ~3) + lane < S_MAX_NB) buf[w][(cnt & ~3) + lane] = 0x7fffffff;
-            __syncwarp();
-            const int4 *b4 = reinterpret_cast<const int4 *>(buf[w]);
-            for (int k = lane; k < cnt; k += 32) {
-                const int v = buf[w][k];
-                int rank = 0;
-                for (int q = 0; q < (cnt + 3) >> 2; ++q) {
-                    const int4 u = b4[q];
-                    rank += (u.x < v) + (u.y < v) + (u.z < v) + (u.w < v);
-                }
-                srt[w][rank] = v;
-            }
-            __syncwarp();
-            int *row = nbr + (size_t)i * maxnb;
-            for (int k = lane; k < maxnb; k += 32) row[k] = k < cnt ? srt[w][k] : -1;
-            if (lane == 0) nnb[i] = cnt;
-            __syncwarp();
+            s_write_row(S, i, cnt, maxnb, lane, buf[w], srt[w], nbr, nnb);
         }
         __syncthreads();   // the staging buffer is reused by the next cell
     }
@@ -364,7 +410,7 @@ extern "C" hd_status hd_nlist_static(const double *d_pos, int n_atoms, const dou
     k_s_bin<<<nb, 128, 0, s>>>(S, G, box[0], box[1], box[2], need_ext, d_pos, n_atoms);
     // the number of cells stays on the device: a fixed grid (five CTAs an SM
     // fit beside their shared memory) strides over them
-    k_s_list<<<std::min(760, n_atoms), S_THREADS, 0, s>>>(S, d_pos, maxnb, d_nbr, d_nnb);
+    k_s_list<<<std::min(760, n_atoms), S_THREADS, 0, s>>>(S, d_pos, n_atoms, maxnb, d_nbr, d_nnb);
     if (cudaGetLastError() != cudaSuccess) return HD_ERR_CUDA;
     int err[4];
     if (cudaMemcpyAsync(err, S->err, sizeof err, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
