@@ -1064,17 +1064,36 @@ __global__ void __launch_bounds__(256, H ? 3 : 4) k_pair32(Dev D, int sweep) {
 // last CTA to finish (all others' results visible to it).  The list is empty
 // in most steps, so the grid is a fixed few CTAs an SM that stride over the
 // listed tiles.  (In the split form only batches of one lane a row get here.)
+// A CTA looks for its tiles 32 replicas at a time, every warp alike: with one
+// replica after another, a step of 3,900 x 113 atoms that were all listed took
+// 1,347 us.
 template <int PREC, int S>
 __device__ __forceinline__ bool sweep_listed(const Dev &D, const int *list, int n, unsigned *ticket) {
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
     int pos = blockIdx.x, base = 0;       // place in the listed replicas' tiles, one after another
-    for (int q = 0; q < n; ++q) {
-        const RepDev &R = D.rep[list[q]];
-        const int t0 = R.tile0 * D.split, nt = R.ntile * D.split;
-        for (; pos < base + nt; pos += gridDim.x) {
-            if (PREC == HD_FP64) dev_pair64<false, false, true, S>(D, t0 + pos - base);
-            else dev_pair32<false, false, true, S>(D, t0 + pos - base);
+    for (int q0 = 0; q0 < n; q0 += 32) {
+        int mine = 0, t0 = 0;
+        if (q0 + lane < n) {
+            const RepDev &R = D.rep[list[q0 + lane]];
+            mine = R.ntile * D.split;
+            t0 = R.tile0 * D.split;
         }
-        base += nt;
+        int upto = mine;                  // tiles of the replicas up to this lane's
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(full, upto, o);
+            if (lane >= o) upto += u;
+        }
+        const int all = __shfl_sync(full, upto, 31);
+        t0 -= upto - mine;
+        for (; pos < base + all; pos += gridDim.x) {
+            const int k = __ffs(__ballot_sync(full, upto > pos - base)) - 1;
+            const int unit = __shfl_sync(full, t0, k) + pos - base;
+            if (PREC == HD_FP64) dev_pair64<false, false, true, S>(D, unit);
+            else dev_pair32<false, false, true, S>(D, unit);
+        }
+        base += all;
     }
     __shared__ unsigned s_tick;
     __syncthreads();
