@@ -701,6 +701,8 @@ hd_status upload_reps(hd_ctx *c) {
 
 // Kernels of a list rebuild (launch_rebuild).
 int rebuild_kernels(const hd_ctx *c) { return c->P.nrep > PLAN_MAX ? 4 : 3; }
+// Kernels more in a step whose sweep forms the Hessian term on demand: k_scalar_late, k_pair_hot.
+int lazy_kernels(const hd_ctx *c) { return !c->D.lazy_h || !c->D.bias_on ? 0 : c->P.prec == HD_FP64 ? 1 : 2; }
 
 // Kernels of one BAOAB step after the opening half (list, pair, scalars, update).
 // next_last: the step after this one is the last of its call.
@@ -712,7 +714,7 @@ void queue_step(hd_ctx *c, int mode, bool next_last, std::vector<hd_ctx::Span> *
     { Timed t(c, sink, T_PAIR); launch_pair(c->D, last ? PAIR_ENERGY : lazy ? PAIR_LAZY : PAIR_FULL, c->s); }
     if (c->D.any_eig) { Timed t(c, sink, T_EIG); launch_eig(c->D, c->s); }
     { Timed t(c, sink, T_SCALAR); launch_scalar(c->D, mode, lazy, !last && !next_last, c->s); }
-    c->launches += (c->D.any_eig ? 2 : 0) + (lazy && c->D.bias_on ? 2 : 0);
+    c->launches += (c->D.any_eig ? 2 : 0) + (lazy ? lazy_kernels(c) : 0);
     if (!c->D.any_nhc) {
         { Timed t(c, sink, T_UPDATE); launch_update(c->D, mode, c->s); }
         c->launches += 3 + rebuild_kernels(c);
@@ -948,7 +950,8 @@ hd_status hd_create(const hd_replica_desc *reps, int n_rep, const hd_params *p, 
     c->Q.any_nhc = c->D.any_nhc;
     // Leave the Hessian term out of the sweeps where it is not used: always
     // without a bias; with one, where the sweep is long enough to pay for the
-    // two launches more (~5 us) that a step then takes.  Measured per sweep with
+    // launches more (two in the split form, ~5 us, one in the FP64 form) that a
+    // step then takes.  Measured per sweep with
     // and without it: 322 and 172 us at 913,408 atoms (split form), 105 and 61 at
     // 228,352, 55 and 40 at 114,176; 517 and 315 us at 57,088 in the FP64 form,
     // whose pipe the term fills.  (The split form's line dates from a sweep that
@@ -1124,7 +1127,7 @@ hd_status hd_step(hd_ctx *c, int n_steps) {
     CK(cudaGraphLaunch(it->second, c->s));
     if (c->timing) c->graph_pending.push_back(key);
     c->launches += (c->D.any_nhc ? 3 + 5LL * n_steps : 2 + 3LL * n_steps) + (long long)rebuild_kernels(c) * n_steps +
-                   (c->D.any_eig ? 2LL * n_steps : 0) + (c->D.lazy_h && c->D.bias_on ? 2LL * (n_steps - 1) : 0);
+                   (c->D.any_eig ? 2LL * n_steps : 0) + (long long)lazy_kernels(c) * (n_steps - 1);
     return HD_OK;
 }
 

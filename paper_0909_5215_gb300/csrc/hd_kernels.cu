@@ -1045,15 +1045,24 @@ __device__ __forceinline__ void dev_pair32(const Dev &D, int unit) {
     }
 }
 
-// Which replicas an MD sweep covers: all of them; those that go without the
-// Hessian term; those that were predicted to need it (see k_scalar).
-enum { SWEEP_ALL = 0, SWEEP_PLAIN = 1 };
-
 template <bool Q, bool E, bool H, int S>
-__global__ void __launch_bounds__(256) k_pair64(Dev D, int sweep) {
-    if (sweep == SWEEP_PLAIN && D.sc[D.tile_rep[blockIdx.x / D.split]].need_h) return;
-    dev_pair64<Q, E, H, S>(D, blockIdx.x);
+__global__ void __launch_bounds__(256) k_pair64(Dev D) { dev_pair64<Q, E, H, S>(D, blockIdx.x); }
+// The Hessian term only for the replicas expected to need it (see
+// expect_slope).  Both kinds share the launch: an FP64 sweep is as long as one
+// row takes until the batch fills the chip twice, so two sweeps one after the
+// other took twice that (100 x 113 atoms, some in their band: 105 us a step, 74
+// now; all in their band 79 and 73; 4 x 14,272 atoms, one in its band: 9.5 and
+// 8.3 ms for 20 steps).
+template <int S>
+__global__ void __launch_bounds__(256) k_pair64_lazy(Dev D) {
+    if (D.sc[D.tile_rep[blockIdx.x / D.split]].need_h) dev_pair64<false, false, true, S>(D, blockIdx.x);
+    else dev_pair64<false, false, false, S>(D, blockIdx.x);
 }
+
+// Which replicas a split-form MD sweep covers: all of them; those that go
+// without the Hessian term (k_pair_hot sweeps the others: the sweep without it
+// runs in 64 registers, with it in 80).
+enum { SWEEP_ALL = 0, SWEEP_PLAIN = 1 };
 template <bool Q, bool E, bool H, int S>
 __global__ void __launch_bounds__(256, H ? 3 : 4) k_pair32(Dev D, int sweep) {
     if (sweep == SWEEP_PLAIN && D.sc[D.tile_rep[blockIdx.x / D.split]].need_h) return;
@@ -1107,12 +1116,11 @@ __device__ __forceinline__ bool sweep_listed(const Dev &D, const int *list, int 
     return true;
 }
 
-// The replicas predicted to need the Hessian term (h_meta[0] of them).
-template <int PREC, int S>
-__global__ void __launch_bounds__(256, PREC == HD_FP64 ? 1 : 3) k_pair_hot(Dev D) {
+// The replicas of the split form predicted to need the Hessian term (h_meta[0] of them).
+__global__ void __launch_bounds__(256, 3) k_pair_hot(Dev D) {
     const int n = D.h_meta[0];
     if (n == 0) return;
-    if (sweep_listed<PREC, S>(D, D.h_list, n, (unsigned *)D.h_meta + 2) && threadIdx.x == 0) {
+    if (sweep_listed<HD_FP32_SPLIT, 1>(D, D.h_list, n, (unsigned *)D.h_meta + 2) && threadIdx.x == 0) {
         D.h_meta[0] = 0;
         D.h_meta[2] = 0;
     }
@@ -1282,13 +1290,13 @@ __device__ __forceinline__ void dev_scalar_acc(const Dev &D, int r, double *acc)
 // the band of Eq. 14; sigma itself needs the forces alone.  So the sweeps of
 // a large batch leave the Hessian term out for the replicas that are not
 // expected in their band (lazy = 1): it costs the sweep a second gather and
-// nearly doubles its time (322 and 172 us at 913,408 atoms).  After each evaluation the next slope is
-// expected within two of the largest recent changes of the slope; a replica
-// whose band reaches there goes on the list that k_pair_hot sweeps with H.  If
-// another one lands in its band all the same, its evaluation is put off
+// nearly doubles its time (322 and 172 us at 913,408 atoms).  After each
+// evaluation the next slope is expected within two of the largest recent changes of the slope; a replica
+// whose band reaches there is swept with H (split form: by k_pair_hot, from a
+// list).  If another one lands in its band all the same, its evaluation is put off
 // (h_meta[1], k_scalar_late) until k_scalar_late has swept it with H, so the
 // result never depends on the guess.  list = 0: the next sweep takes H for
-// everyone (the last step of a call, whose H can be read).
+// everyone (the last step of a call, whose H can be read), or the form is FP64.
 __device__ void expect_slope(const Dev &D, int r, RepState &S, Scal &C, int list) {
     const RepDev &R = D.rep[r];
     const double step = fabs(C.sigma - S.h_sig);
@@ -2278,19 +2286,18 @@ void launch_rebuild(const Dev &D, cudaStream_t s) {
 template <int S>
 static void pair_of(const Dev &D, int kind, cudaStream_t s) {
     const int grid = D.ntile * D.split, n = unit_threads(D);
-    const bool hot = kind == PAIR_LAZY && D.bias_on;
     if (D.prec == HD_FP64) {
-        if (kind == PAIR_QUENCH) k_pair64<true, false, false, S><<<grid, n, 0, s>>>(D, SWEEP_ALL);
-        else if (kind == PAIR_ENERGY) k_pair64<false, true, true, S><<<grid, n, 0, s>>>(D, SWEEP_ALL);
-        else if (kind == PAIR_FULL) k_pair64<false, false, true, S><<<grid, n, 0, s>>>(D, SWEEP_ALL);
-        else k_pair64<false, false, false, S><<<grid, n, 0, s>>>(D, SWEEP_PLAIN);
-        if (hot) k_pair_hot<HD_FP64, S><<<D.hot_grid, n, 0, s>>>(D);
+        if (kind == PAIR_QUENCH) k_pair64<true, false, false, S><<<grid, n, 0, s>>>(D);
+        else if (kind == PAIR_ENERGY) k_pair64<false, true, true, S><<<grid, n, 0, s>>>(D);
+        else if (kind == PAIR_FULL) k_pair64<false, false, true, S><<<grid, n, 0, s>>>(D);
+        else if (D.bias_on) k_pair64_lazy<S><<<grid, n, 0, s>>>(D);
+        else k_pair64<false, false, false, S><<<grid, n, 0, s>>>(D);
     } else {
         if (kind == PAIR_QUENCH) k_pair32<true, false, false, S><<<grid, n, 0, s>>>(D, SWEEP_ALL);
         else if (kind == PAIR_ENERGY) k_pair32<false, true, true, S><<<grid, n, 0, s>>>(D, SWEEP_ALL);
         else if (kind == PAIR_FULL) k_pair32<false, false, true, S><<<grid, n, 0, s>>>(D, SWEEP_ALL);
         else k_pair32<false, false, false, S><<<grid, n, 0, s>>>(D, SWEEP_PLAIN);
-        if (hot) k_pair_hot<HD_FP32_SPLIT, 1><<<D.hot_grid, n, 0, s>>>(D);
+        if (kind == PAIR_LAZY && D.bias_on) k_pair_hot<<<D.hot_grid, n, 0, s>>>(D);
     }
 }
 void launch_pair(const Dev &D, int kind, cudaStream_t s) {
@@ -2299,9 +2306,9 @@ void launch_pair(const Dev &D, int kind, cudaStream_t s) {
 }
 void launch_scalar(const Dev &D, int mode, bool lazy, bool list, cudaStream_t s) {
     const bool more = D.lazy_h && D.bias_on;
-    k_scalar<<<D.nrep, sc_threads(D), 0, s>>>(D, mode, lazy && more, list && more);
+    const int n = unit_threads(D), g = D.hot_grid, li = list && more && D.prec != HD_FP64;
+    k_scalar<<<D.nrep, sc_threads(D), 0, s>>>(D, mode, lazy && more, li);
     if (!lazy || !more) return;
-    const int n = unit_threads(D), g = D.hot_grid, li = list && more;
     if (D.prec != HD_FP64) k_scalar_late<HD_FP32_SPLIT, 1><<<g, n, 0, s>>>(D, mode, li);
     else if (D.lanes == 4) k_scalar_late<HD_FP64, 4><<<g, n, 0, s>>>(D, mode, li);
     else k_scalar_late<HD_FP64, 1><<<g, n, 0, s>>>(D, mode, li);
